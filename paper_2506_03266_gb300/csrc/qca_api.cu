@@ -102,9 +102,9 @@ int decode_path(int L, int v, int m_max) {
   return fast_path_for(L, v, m_max);
 }
 
-int launch_decode(const DecodeArgs& a, cudaStream_t stream) {
-  if (a.shots == 0) return QCA_OK;
-  if (int rc = check_aligned(a.out_steps, 4, "out_steps")) return rc;
+// The sweeps that keep the message fields: the on-chip, large-lattice or
+// generic one.
+static int launch_planes(const DecodeArgs& a, cudaStream_t stream) {
   int path = decode_path(a.L, a.v, a.m_max);
   // The on-chip and large-lattice kernels read the input and write the
   // correction as 32-bit words.  A caller array or shot block off a 4-byte
@@ -114,6 +114,20 @@ int launch_decode(const DecodeArgs& a, cudaStream_t stream) {
   if (path == 3) return launch_tiled(a, stream);
   if (path > 0) return launch_fast(a, stream);
   return launch_generic(a, stream);
+}
+
+int launch_decode(const DecodeArgs& a, cudaStream_t stream) {
+  if (a.shots == 0) return QCA_OK;
+  if (int rc = check_aligned(a.out_steps, 4, "out_steps")) return rc;
+  // v = 3 decodes from the syndrome history at any size from 8 on, unless the
+  // caller chose a kernel for the size
+  if (!history_takes(a.L, a.v) || path_forced(a.L)) return launch_planes(a, stream);
+  int rc = launch_history(a, stream);
+  if (rc || !history_may_leave_pending(a.L)) return rc;
+  DecodeArgs rest = a;
+  rest.only_pending = 1;
+  rest.queue = nullptr;
+  return launch_planes(rest, stream);
 }
 
 static int dispatch(DecodeArgs& a, cudaStream_t stream) { return launch_decode(a, stream); }
@@ -379,8 +393,8 @@ int qca_decode_batch_host(const uint8_t* syndrome, int L, int64_t shots, int max
 
 int qca_free_workspace(void) {
   int rc = generic_workspace_release();
-  const int rc2 = tiled_workspace_release();
-  if (rc == QCA_OK) rc = rc2;
+  const int rc2 = tiled_workspace_release(), rc3 = history_workspace_release();
+  if (rc == QCA_OK) rc = rc2 ? rc2 : rc3;
   std::lock_guard<std::mutex> lk(g_stage_mu);
   int dev = 0;
   cudaGetDevice(&dev);

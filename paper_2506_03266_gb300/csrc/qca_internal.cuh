@@ -52,7 +52,13 @@ struct DecodeArgs {
   // Some shot block starts off a 4-byte boundary (packed uneven batches with
   // odd L): only the byte-access generic sweep may read it.
   int bytewise;
+  // Decode only the shots whose out_steps is kStepsPending (the others are done).
+  int only_pending;
 };
+
+// out_steps of a shot that the history sweep leaves to the sweeps with message
+// planes (it needs a syndrome older than the ones it keeps).
+constexpr int kStepsPending = -1;
 
 // Byte offset of shot `shot`'s input block: [2][L][L] noise, or [L][L] sigma.
 __host__ __device__ __forceinline__ int64_t shot_offset_of(const DecodeArgs& a, int64_t shot) {
@@ -146,6 +152,14 @@ int launch_generic(const DecodeArgs& a, cudaStream_t stream);
 int generic_workspace_release();
 int fast_path_for(int L, int v, int m_max);  // 0 generic, 1 single-CTA, 2 two-CTA cluster
 int launch_fast(const DecodeArgs& a, cudaStream_t stream);
+// Sizes above 128 for which the four-CTA form of the on-chip sweep is chosen.
+bool four_cta_chosen(int L);
+// History sweep (v = 3, 8 <= L <= 1024): whether it takes the call, whether it
+// may leave shots pending (up to L = 256), and the launch.
+bool history_takes(int L, int v);
+bool history_may_leave_pending(int L);
+int launch_history(const DecodeArgs& a, cudaStream_t stream);
+int history_workspace_release();
 // Large-lattice kernel (cluster of 8 CTAs per shot, state in global memory).
 int tiled_path_for(int L, int v, int m_max);  // 1 if it takes (L, v, m_max)
 int launch_tiled(const DecodeArgs& a, cudaStream_t stream);
@@ -154,6 +168,7 @@ int generic_forced(int L);  // qca_set_kernel_path(L, 0) is in effect
 // Kernel path for (L, v, m_max) with the overrides applied: 0 generic,
 // 1 / 2 on-chip (one CTA / two-CTA cluster), 3 tiled; and the launch.
 int decode_path(int L, int v, int m_max);
+bool path_forced(int L);  // a kernel path or form was chosen for L by the caller
 int launch_decode(const DecodeArgs& a, cudaStream_t stream);
 // Mixed lattice sizes in one persistent launch (on-chip sweep): the group
 // size of a lattice size in it (0 two-CTA pair, else 512, 256, 128 or 64

@@ -926,9 +926,24 @@ __global__ void __launch_bounds__(CL == 1 ? 1024 : (CL == 2 ? 512 : 256), CL == 
     if (CL > 1) Cluster<CL>::sync();
     return k;
   };
-  for (int64_t k = next_work(-1); k < a.shots; k = next_work(k)) {
-    const int64_t shot = a.shot_list ? (int64_t)a.shot_list[k] : k;
-    decode_shot<CL, KW>(a, g, smem, shot, G);
+  auto shot_of = [&](int64_t k) { return a.shot_list ? (int64_t)a.shot_list[k] : k; };
+  if (a.only_pending) {
+    // the shots the history sweep left: the threads look at as many shots at a
+    // time (every CTA of a cluster reads a shot's state before it is decoded)
+    for (int64_t k0 = (int64_t)cid * blockDim.x; k0 < a.shots;
+         k0 += (int64_t)nclusters * blockDim.x) {
+      const bool mine = k0 + tid < a.shots && a.out_steps[shot_of(k0 + tid)] == kStepsPending;
+      if (!__syncthreads_or(mine)) continue;
+      for (int i = 0; i < (int)blockDim.x && k0 + i < a.shots; ++i) {
+        const int64_t shot = shot_of(k0 + i);
+        if (a.out_steps[shot] != kStepsPending) continue;
+        Cluster<CL>::sync();  // all have read it
+        decode_shot<CL, KW>(a, g, smem, shot, G);
+      }
+    }
+  } else {
+    for (int64_t k = next_work(-1); k < a.shots; k = next_work(k))
+      decode_shot<CL, KW>(a, g, smem, shot_of(k), G);
   }
   // no CTA of a cluster leaves while a partner could still reach its shared memory
   if (CL > 1) Cluster<CL>::sync();
@@ -1231,6 +1246,8 @@ int fast_path_for(int L, int v, int m_max) {
   if (!make_geom(L, m_max, CL, KW, g, threads, smem)) return 0;
   return CL > 2 ? 2 : CL;
 }
+
+bool four_cta_chosen(int L) { return L >= 0 && L <= QCA_MAX_L && g_cluster4[L]; }
 
 int launch_fast(const DecodeArgs& a, cudaStream_t stream) {
   int CL, KW, threads;

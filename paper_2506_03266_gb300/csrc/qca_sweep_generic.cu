@@ -50,6 +50,12 @@ __global__ void __launch_bounds__(kThreads) sweep_generic_kernel(DecodeArgs a, u
   };
   for (int64_t k = next_work(-1); k < a.shots; k = next_work(k)) {
     const int64_t shot = a.shot_list ? (int64_t)a.shot_list[k] : k;
+    if (a.only_pending) {
+      // the shots the history sweep left; all threads read the state first
+      const bool done = a.out_steps[shot] != kStepsPending;
+      __syncthreads();
+      if (done) continue;
+    }
     const int64_t base = shot_offset_of(a, shot);
     const uint8_t* in = a.in + base;
     int any = 0;

@@ -703,6 +703,11 @@ int generic_forced(int L) {
   return (L >= 3 && L <= QCA_MAX_L && g_path_override[L] == 0) ? 1 : 0;
 }
 
+bool path_forced(int L) {
+  std::call_once(g_override_once, init_overrides);
+  return (L >= 3 && L <= QCA_MAX_L && g_path_override[L] >= 0) || four_cta_chosen(L);
+}
+
 int launch_tiled(const DecodeArgs& a, cudaStream_t stream) {
   if (a.shots == 0) return QCA_OK;
   TiledGeom g;
