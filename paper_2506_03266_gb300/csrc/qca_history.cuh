@@ -20,8 +20,8 @@
 // One CTA of NT threads decodes one shot.  A step runs in one of three modes:
 //   dense   many anyons: distance 1 of all anyons 32 sites per bitmap word, the
 //           undecided ones (a few per cent) listed and searched one by one;
-//   listed  at most sparse_max anyons, one thread per anyon for slice 0, a
-//           whole warp per anyon beyond it;
+//   listed  at most sparse_max anyons, one thread per anyon for slices 0 to 4
+//           (a (6k + 7)^2 neighbourhood), a whole warp per anyon beyond them;
 //   few     at most 8 anyons: one warp runs all remaining steps by itself, one
 //           lane per (anyon, slice), from a ring of the last anyon sets.
 // Flipped links are marked in a map, so that a link crossed from both ends
@@ -37,6 +37,8 @@ namespace hist {
 
 constexpr int kFew = 8;        // most anyons of the few-anyon mode
 constexpr int kFewRing = 128;  // steps of anyon sets it keeps (more than 85)
+constexpr int kArchiveSets = 86;  // steps of archived sets (more than 85)
+constexpr uint16_t kNoSet = 0xFFFF;
 constexpr int kLargeRing = 88; // syndromes kept per shot above L = 256 (more than 85)
 constexpr uint32_t kFull = 0xffffffffu;
 
@@ -44,13 +46,31 @@ struct Geom {
   int L;
   int lws;         // log2 of the 32-bit words per bitmap row
   int nws;         // words of one site bitmap (L << lws)
+  int nslot;       // words of a bitmap's place in shared memory (a multiple of 4)
   int kmask;       // syndromes kept in shared memory, less one (a power of two less one)
-  int spill;       // most older syndromes kept in the correction block (0: none needed)
+  int spill;       // whether syndromes older than those are needed at all
+  int kthread;     // oldest slice a single thread can search: min(4, (L - 7) / 6)
+  int c_global;    // correction and link maps are kept in the correction block
   int kmax;        // oldest slice a message can come from: (m_max - 1) / 3
   int sparse_max;  // most anyons of the listed mode
   int list_cap;    // entries of the anyon list
   // word offsets in the CTA's shared memory (L <= 256) or its global slot
-  int o_C, o_F, o_list, o_few, o_misc;
+  int o_C, o_F, o_list, o_table, o_few, o_snap, o_misc;  // (o_F: LARGE only)
+  int tmask;       // entries of the crossing table, less one
+};
+
+// Syndromes that have left shared memory, in the shot's correction block (2 L^2
+// bytes, not written before the shot ends): a set of at most `cap` anyons as a
+// list of 16-bit sites, one place for each of the last 86 steps, taken when the
+// set is listed; a larger one as a bitmap, in a ring of nb places.  Anyons
+// never multiply, so the bitmaps are the first syndromes of the shot.  Blocks
+// too small for lists (L < 55) are all bitmaps.
+struct Archive {
+  uint16_t* sets;     // [kArchiveSets][cap]
+  uint32_t* bitmaps;  // [nb][nws]
+  int cap, nb;
+  int gone;           // one more than the last bitmap's step
+  int next;           // syndromes moved so far
 };
 
 __device__ __forceinline__ int wrap_lo(int i, int L) { return i < 0 ? i + L : i; }
@@ -72,9 +92,11 @@ __device__ __forceinline__ uint32_t row_any(const uint32_t* row, int wpr, int L,
                                             int reach) {
   uint32_t any = 0;
   if (2 * reach + 1 >= L) {
+#pragma unroll 1
     for (int w = 0; w < wpr; ++w) any |= row[w];
   } else {
     int c = wrap_lo(x - reach, L);
+#pragma unroll 1
     for (int left = 2 * reach + 1; left > 0; left -= 32) {
       any |= row_bits_wrapped(row, wpr, L, c, left < 32 ? left : 32);
       c = wrap_hi(c + 32, L);
@@ -91,43 +113,56 @@ __device__ __forceinline__ uint32_t slice_limit(int m_max, int k) {
   return n >= 3 ? 0xFFFu : (n == 2 ? 0xFFu : (n == 1 ? 0xFu : 0u));
 }
 
-// Slice 0 of the anyon at (x, y), by one thread: a 7 x 7 neighbourhood.
-__device__ __forceinline__ uint32_t slice0(const uint32_t* sig, int lws, int L, int x, int y) {
+// Slice k of the anyon at (x, y) by one thread, from the bitmap of sigma_{t-k}:
+// the (6k + 7) x (6k + 7) neighbourhood, a row window per row; needs 6k + 7 <=
+// 31 and <= L.
+__device__ __forceinline__ uint32_t slice_thread(const uint32_t* sig, int lws, int L, int x, int y,
+                                                 int k) {
   const int wpr = 1 << lws;
-  const int s = wrap_lo(x - 3, L);
+  const int r = 3 * k + 3, n = 2 * r + 1;
+  const int s = wrap_lo(x - r, L);
   const int w0 = s >> 5, sh = s & 31;
   const int w1 = min(w0 + 1, wpr - 1);
   const int sl = w0 < wpr - 1 ? 32 - sh : 32;  // 1 .. 32
-  const int n0 = s + 7 > L ? L - s : 0;        // columns before the wrap, if any
-  uint32_t r[7];  // bit i: column x - 3 + i of row y - 3 + j
-#pragma unroll
-  for (int j = 0; j < 7; ++j) {
-    const int yy = wrap_hi(wrap_lo(y + j - 3, L), L);
+  const int n0 = s + n > L ? L - s : 0;        // columns before the wrap, if any
+  const uint32_t mask = (1u << n) - 1u;
+  int yy = wrap_lo(y - r, L);
+  auto next = [&]() {  // bit i: column x - r + i of the next row
     const uint32_t* row = sig + (yy << lws);
     uint32_t v = (row[w0] >> sh) | __funnelshift_lc(0u, row[w1], sl);
     if (n0) v |= row[0] << n0;  // the bits past column L - 1 are 0
-    r[j] = v & 0x7Fu;
-  }
-  const uint32_t v1 = r[2] | r[3] | r[4];
-  const uint32_t v2 = v1 | r[1] | r[5];
-  const uint32_t v3 = v2 | r[0] | r[6];
+    ++yy;
+    if (yy == L) yy = 0;
+    return v & mask;
+  };
+  // rows y - r .. y + r; the distances' cone sections across the rows are
+  // |j| <= 3k + 1, 3k + 2, 3k + 3
+  const uint32_t u3 = next(), u2 = next(), u1 = next();
+  uint32_t v1 = u1;
+#pragma unroll 1
+  for (int i = 0; i < n - 6; ++i) v1 |= next();
+  const uint32_t d1 = next(), d2 = next(), d3 = next();
+  v1 |= d1;
+  const uint32_t v2 = v1 | u2 | d2, v3 = v2 | u3 | d3;
   // +x comes from column x - d, -x from x + d, +y from row y - d, -y from y + d
-  uint32_t m = ((v1 >> 2) & 1u) | ((v1 >> 3) & 2u);
-  m |= ((v2 << 3) & 0x10u) | (v2 & 0x20u);
-  m |= ((v3 << 8) & 0x100u) | ((v3 << 3) & 0x200u);
-  m |= (r[2] & 0x1Cu) ? 0x4u : 0u;
-  m |= (r[4] & 0x1Cu) ? 0x8u : 0u;
-  m |= (r[1] & 0x3Eu) ? 0x40u : 0u;
-  m |= (r[5] & 0x3Eu) ? 0x80u : 0u;
-  m |= r[0] ? 0x400u : 0u;
-  m |= r[6] ? 0x800u : 0u;
+  uint32_t m = ((v1 >> 2) & 1u) | (((v1 >> (n - 3)) & 1u) << 1);
+  m |= ((v2 << 3) & 0x10u) | (((v2 >> (n - 2)) & 1u) << 5);
+  m |= ((v3 << 8) & 0x100u) | ((v3 >> (n - 1)) << 9);
+  const uint32_t m1 = (mask >> 4) << 2, m2 = (mask >> 2) << 1;
+  if (u1 & m1) m |= 0x4u;
+  if (d1 & m1) m |= 0x8u;
+  if (u2 & m2) m |= 0x40u;
+  if (d2 & m2) m |= 0x80u;
+  if (u3) m |= 0x400u;
+  if (d3) m |= 0x800u;
   return m;
 }
 
-// Slice k >= 1 of the anyon at (x, y) by a whole warp, from the bitmap of
-// sigma_{t-k}: a lane per row for the x fields (three columns on either side),
-// six lanes for the y fields' rows.
-__device__ __forceinline__ uint32_t slice_warp(const uint32_t* sig, int lws, int L, int x, int y,
+// Any slice of the anyon at (x, y) by a whole warp: a lane per row for the x
+// fields (three columns on either side), six lanes for the y fields' rows.  For
+// the far slices, which few anyons reach: a function of its own, since the
+// kernel is bound by instruction fetch when every use is a copy.
+static __device__ __noinline__ uint32_t slice_warp(const uint32_t* sig, int lws, int L, int x, int y,
                                                int k, int lane) {
   const int wpr = 1 << lws;
   const int r = 3 * k + 3;
@@ -136,6 +171,7 @@ __device__ __forceinline__ uint32_t slice_warp(const uint32_t* sig, int lws, int
   const int cl = wrap_lo(x - r % L, L);              // columns x - 3k - 3 ..
   const int cr = wrap_hi(x + (3 * k + 1) % L, L);    // columns x + 3k + 1 ..
   uint32_t m = 0;
+#pragma unroll 1
   for (int i = lane; i < nrows; i += 32) {
     const int j = i - half;
     const uint32_t* row = sig + (wrap_hi(wrap_lo(y + j, L), L) << lws);
@@ -156,8 +192,21 @@ __device__ __forceinline__ uint32_t slice_warp(const uint32_t* sig, int lws, int
   return __reduce_or_sync(kFull, m);
 }
 
-// Slice k of the anyon at (xa, ya) against one anyon (xb, yb) of sigma_{t-k};
-// c = (3k + 1) mod L.
+// Slice k of the anyon at (xa, ya) against one anyon (xb, yb) of sigma_{t-k}, for
+// slices within half the torus (3k + 3 <= (L - 1) / 2): the larger of the two
+// coordinate distances decides.
+__device__ __forceinline__ uint32_t slice_near(int xa, int ya, int xb, int yb, int L, int k) {
+  const int half = L >> 1;
+  int sx = xa - xb, sy = ya - yb;
+  if (sx > half) sx -= L;
+  if (sx < -half) sx += L;
+  if (sy > half) sy -= L;
+  if (sy < -half) sy += L;
+  const int ax = abs(sx), ay = abs(sy), d = max(ax, ay), e = d - 3 * k - 1;
+  if ((unsigned)e >= 3u) return 0;
+  return ((ax == d ? (sx > 0 ? 1u : 2u) : 0u) | (ay == d ? (sy > 0 ? 4u : 8u) : 0u)) << (4 * e);
+}
+// The same for any slice; c = (3k + 1) mod L.
 __device__ __forceinline__ uint32_t slice_pair(int xa, int ya, int xb, int yb, int L, int k,
                                                int c) {
   const int dx = wrap_lo(xa - xb, L), dy = wrap_lo(ya - yb, L);
@@ -173,6 +222,19 @@ __device__ __forceinline__ uint32_t slice_pair(int xa, int ya, int xb, int yb, i
   if (epy < 3 && ax <= 3 * k + 1 + epy) m |= 4u << (4 * epy);
   if (emy < 3 && ax <= 3 * k + 1 + emy) m |= 8u << (4 * emy);
   return m;
+}
+
+// The same against all n anyons of an archived set, by a whole warp.
+static __device__ __noinline__ uint32_t slice_list(const uint16_t* set, int n, int L, int x, int y,
+                                                   int k, int lane) {
+  const int c = (3 * k + 1) % L;
+  uint32_t m = 0;
+#pragma unroll 1
+  for (int i = lane; i < n; i += 32) {
+    const uint32_t e = set[i];
+    m |= slice_pair(x, y, (int)(e & 0xFFu), (int)(e >> 8), L, k, c);
+  }
+  return __reduce_or_sync(kFull, m);
 }
 
 // Direction from the fields heard at the smallest distance (h0, never 0) and,
@@ -193,151 +255,206 @@ __device__ __forceinline__ int direction(uint32_t h0, uint32_t h1, int tie_order
   return 4;
 }
 
-// Whether the next distance's hits are needed beside h0 (literal ties).
-__device__ __forceinline__ bool needs_next(uint32_t h0, int tie_order) {
-  return tie_order == QCA_TIE_LITERAL && !(h0 & 10u);
+// The counter draws, out of line: options that most calls leave off.
+struct Keys {
+  uint64_t move, bal;
+};
+static __device__ __noinline__ uint64_t key_of(uint64_t key, int64_t shot, int t) {
+  return move_step_key(key, shot, t);
+}
+// Random move of the anyon at site r, or 0.
+static __device__ __noinline__ int draw_move(uint64_t key, uint64_t thr, uint32_t r) {
+  const uint64_t u = splitmix64(key ^ (uint64_t)r);
+  return u < thr ? 1 + (int)(splitmix64(u) >> 62) : 0;
+}
+static __device__ __noinline__ int draw_balance(int code, uint64_t key, uint32_t r) {
+  return balance_resolve(code, key, r);
 }
 
-// 16 bytes of 0 / 1 -> 16 bits; ANY: of zero / nonzero.
-template <bool ANY>
-__device__ __forceinline__ uint32_t pack4(uint32_t w) {
-  if (ANY) w = ((((w & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | w) & 0x80808080u) >> 7;
-  return (w * 0x01020408u) >> 24;
+// 16 bytes -> 16 bits: bit 0 of each byte, or (any) whether it is not 0.
+__device__ __forceinline__ uint32_t pack4(uint32_t w) { return (w * 0x01020408u) >> 24; }
+__device__ __forceinline__ uint32_t nonzero4(uint32_t w) {
+  return ((((w & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | w) & 0x80808080u) >> 7;
 }
-template <bool ANY>
-__device__ __forceinline__ uint32_t pack16(uint4 v) {
-  return pack4<ANY>(v.x) | (pack4<ANY>(v.y) << 4) | (pack4<ANY>(v.z) << 8) |
-         (pack4<ANY>(v.w) << 12);
+__device__ __forceinline__ uint32_t pack16(uint4 v, bool any) {
+  if (any) v = make_uint4(nonzero4(v.x), nonzero4(v.y), nonzero4(v.z), nonzero4(v.w));
+  return pack4(v.x) | (pack4(v.y) << 4) | (pack4(v.z) << 8) | (pack4(v.w) << 12);
 }
 // 4 bits -> 4 bytes of 0 / 1.
 __device__ __forceinline__ uint32_t unpack4(uint32_t nib) {
   return (nib * 0x00204081u) & 0x01010101u;
 }
-
-// rows x L bytes at src -> bitmap rows (2^lws words each, padding bits 0).
-template <int NT, bool ANY>
-__device__ __forceinline__ void load_bits(const uint8_t* src, int rows, int L, int lws,
-                                          uint32_t* dst, int tid) {
-  if ((L & 15) == 0 && (reinterpret_cast<uintptr_t>(src) & 15) == 0) {
-    // 16 bytes per lane and access: a warp reads 512 contiguous bytes
-    const int vpr = L >> 4, n = rows * vpr;
-    const uint4* s16 = reinterpret_cast<const uint4*>(src);
-    uint16_t* d16 = reinterpret_cast<uint16_t*>(dst);
-    const int dr = NT / vpr, dc = NT - dr * vpr;
-    int r = tid / vpr, c = tid - r * vpr;
-#pragma unroll 8
-    for (int i = tid; i < n; i += NT) {
-      const uint4 v = __ldcs(s16 + i);
-      d16[(r << (lws + 1)) + c] = (uint16_t)pack16<ANY>(v);
-      r += dr;
-      c += dc;
-      if (c >= vpr) {
-        c -= vpr;
-        ++r;
-      }
-    }
-    return;
-  }
-  // any size and alignment: a bitmap word per thread from aligned 32-bit
-  // loads, single bytes at the two ends of the block
-  const uint8_t* end = src + (size_t)rows * L;
-  const int wpr = 1 << lws;
-  for (int i = tid; i < rows << lws; i += NT) {
-    const int r = i >> lws, x0 = (i & (wpr - 1)) << 5;
-    if (x0 >= L) continue;
-    const int n = min(32, L - x0);
-    const uint8_t* p = src + (size_t)r * L + x0;
-    const int mis = (int)(reinterpret_cast<uintptr_t>(p) & 3);
-    const uint8_t* q = p - mis;
-    uint64_t acc = 0;
-    const int nw = (mis + n + 3) >> 2;
-    for (int w = 0; w < nw; ++w, q += 4) {
-      uint32_t v = 0;
-      if (q >= src && q + 4 <= end) {
-        v = *reinterpret_cast<const uint32_t*>(q);
-      } else {
-        for (int b = 0; b < 4; ++b)
-          if (q + b >= src && q + b < end) v |= (uint32_t)q[b] << (8 * b);
-      }
-      acc |= (uint64_t)(pack4<ANY>(v) & 0xFu) << (4 * w);
-    }
-    const uint32_t bits = (uint32_t)(acc >> mis);
-    dst[i] = n == 32 ? bits : bits & ((1u << n) - 1u);
-  }
+__device__ __forceinline__ uint4 unpack16(uint32_t b) {
+  return make_uint4(unpack4(b & 15u), unpack4((b >> 4) & 15u), unpack4((b >> 8) & 15u),
+                    unpack4((b >> 12) & 15u));
 }
 
-// Bitmap rows -> rows x L bytes of 0 / 1 at out.
-template <int NT>
-__device__ __forceinline__ void store_bits(uint8_t* out, int rows, int L, int lws,
-                                           const uint32_t* src, int tid) {
-  if ((L & 15) == 0 && (reinterpret_cast<uintptr_t>(out) & 15) == 0) {
-    const int vpr = L >> 4, n = rows * vpr;
-    uint4* o16 = reinterpret_cast<uint4*>(out);
-    const uint16_t* s16 = reinterpret_cast<const uint16_t*>(src);
-    const int dr = NT / vpr, dc = NT - dr * vpr;
-    int r = tid / vpr, c = tid - r * vpr;
-#pragma unroll 4
-    for (int i = tid; i < n; i += NT) {
-      const uint32_t b = s16[(r << (lws + 1)) + c];
-      __stcs(o16 + i, make_uint4(unpack4(b & 15u), unpack4((b >> 4) & 15u),
-                                 unpack4((b >> 8) & 15u), unpack4(b >> 12)));
-      r += dr;
-      c += dc;
-      if (c >= vpr) {
-        c -= vpr;
-        ++r;
-      }
-    }
-    return;
-  }
-  // any size and alignment: aligned groups of four bytes, single bytes at the ends
+// rows x L bytes at src -> bitmap rows (2^lws words each), any size and
+// alignment: 16-byte groups of the flat block (single bytes at its two ends),
+// whose bits go to the two or three rows they belong to.  dst is zeroed before.
+static __device__ __noinline__ void load_flat(const uint8_t* src, int rows, int L, int lws,
+                                              uint32_t* dst, bool any, int tid, int nt) {
   const int total = rows * L;
-  const int head = (int)((4 - (reinterpret_cast<uintptr_t>(out) & 3)) & 3);
-  for (int i = tid; 4 * i - 4 + head < total; i += NT) {
-    const int f0 = 4 * i - 4 + head;  // group 0 holds the bytes before the first boundary
-    const int fs = max(f0, 0);
-    int r = fs / L, x = fs - r * L;
-    uint32_t v = 0;
-    for (int b = fs - f0; b < 4; ++b) {
-      if (f0 + b >= total) break;
-      v |= ((src[(r << lws) + (x >> 5)] >> (x & 31)) & 1u) << (8 * b);
-      if (++x == L) {
-        x = 0;
-        ++r;
+  const int skew = (int)(reinterpret_cast<uintptr_t>(src) & 15);
+#pragma unroll 2
+  for (int i = tid; 16 * i < total + skew; i += nt) {
+    int f = 16 * i - skew;
+    uint32_t b = 0;
+    if (f >= 0 && f + 16 <= total) {
+      b = pack16(*reinterpret_cast<const uint4*>(src + f), any);
+    } else {
+#pragma unroll 1
+      for (int q = 0; q < 16; ++q)
+        if (f + q >= 0 && f + q < total && (any ? src[f + q] != 0 : src[f + q] & 1)) b |= 1u << q;
+      if (f < 0) {
+        b >>= -f;
+        f = 0;
       }
     }
-    if (f0 >= 0 && f0 + 4 <= total) {
-      *reinterpret_cast<uint32_t*>(out + f0) = v;
-    } else {
-      for (int b = 0; b < 4; ++b)
-        if (f0 + b >= 0 && f0 + b < total) out[f0 + b] = (uint8_t)(v >> (8 * b));
+    int r = f / L, x = f - r * L;
+    while (b) {
+      const uint32_t v = L - x < 16 ? b & ((1u << (L - x)) - 1u) : b;
+      uint32_t* row = dst + (r << lws);
+      const int sh = x & 31;
+      if (v << sh) atomicOr(&row[x >> 5], v << sh);
+      if (sh > 16 && v >> (32 - sh)) atomicOr(&row[(x >> 5) + 1], v >> (32 - sh));
+      b = L - x < 16 ? b >> (L - x) : 0;
+      x = 0;
+      ++r;
     }
   }
 }
 
-// Words of the few-anyon mode: the ring of anyon sets and one snapshot of it
-// (orbit detection); entries are 16 bits up to L = 256, 32 bits above.
-template <bool LARGE>
-constexpr int kFewWords = 2 * kFewRing * kFew / (LARGE ? 1 : 2);
+// Bitmap rows -> rows x L bytes of 0 / 1 at out, any size and alignment.
+static __device__ __noinline__ void store_flat(uint8_t* out, int rows, int L, int lws,
+                                               const uint32_t* src, int tid, int nt) {
+  const int total = rows * L, wpr = 1 << lws;
+  const int skew = (int)(reinterpret_cast<uintptr_t>(out) & 15);
+#pragma unroll 1
+  for (int i = tid; 16 * i < total + skew; i += nt) {
+    const int f0 = 16 * i - skew, f = max(f0, 0);
+    int r = f / L, x = f - r * L;
+    uint32_t b = 0;
+    for (int have = f - f0; have < 16 && r < rows; ++r) {
+      const uint32_t* row = src + (r << lws);
+      const int w = x >> 5;
+      uint32_t v = __funnelshift_r(row[w], w + 1 < wpr ? row[w + 1] : 0u, x & 31);
+      if (L - x < 16) v &= (1u << (L - x)) - 1u;
+      b |= (v & 0xFFFFu) << have;
+      have += L - x;
+      x = 0;
+    }
+    if (f0 >= 0 && f0 + 16 <= total) {
+      __stcs(reinterpret_cast<uint4*>(out + f0), unpack16(b));
+    } else {
+#pragma unroll 1
+      for (int q = 0; q < 16; ++q)
+        if (f0 + q >= 0 && f0 + q < total) out[f0 + q] = (uint8_t)((b >> q) & 1u);
+    }
+  }
+}
 
-template <int NT, bool LARGE>
+// The same for rows of whole 16-byte groups on a 16-byte boundary: a warp
+// moves 512 contiguous bytes at a time.
+template <int NT>
+__device__ __forceinline__ void load_rows(const uint8_t* src, int rows, int L, int lws,
+                                          uint32_t* dst, bool any, int tid) {
+  const int vpr = L >> 4, n = rows * vpr;
+  const uint4* s16 = reinterpret_cast<const uint4*>(src);
+  uint16_t* d16 = reinterpret_cast<uint16_t*>(dst);
+  const int dr = NT / vpr, dc = NT - dr * vpr;
+  int r = tid / vpr, c = tid - r * vpr;
+#pragma unroll 4
+  for (int i = tid; i < n; i += NT) {
+    d16[(r << (lws + 1)) + c] = (uint16_t)pack16(__ldcs(s16 + i), any);
+    r += dr;
+    c += dc;
+    if (c >= vpr) {
+      c -= vpr;
+      ++r;
+    }
+  }
+}
+template <int NT>
+__device__ __forceinline__ void store_rows(uint8_t* out, int rows, int L, int lws,
+                                           const uint32_t* src, int tid) {
+  const int vpr = L >> 4, n = rows * vpr;
+  uint4* o16 = reinterpret_cast<uint4*>(out);
+  const uint16_t* s16 = reinterpret_cast<const uint16_t*>(src);
+  const int dr = NT / vpr, dc = NT - dr * vpr;
+  int r = tid / vpr, c = tid - r * vpr;
+#pragma unroll 2
+  for (int i = tid; i < n; i += NT) {
+    __stcs(o16 + i, unpack16(s16[(r << (lws + 1)) + c]));
+    r += dr;
+    c += dc;
+    if (c >= vpr) {
+      c -= vpr;
+      ++r;
+    }
+  }
+}
+
+// Words of the few-anyon mode's ring of anyon sets, and of each of the two
+// snapshots of it (orbit detection); entries are 16 bits up to L = 256, 32 bits
+// above.
+template <bool LARGE>
+constexpr int kFewWords = kFewRing * kFew / (LARGE ? 1 : 2);
+
+// Whether the kmax + 1 anyon sets up to step t equal those up to step t_snap
+// of the snapshot; `words` 32-bit words per set.  By one warp.
+static __device__ __noinline__ bool sets_repeat(const uint32_t* now, const uint32_t* snap, int t,
+                                                int t_snap, int kmax, int words, int lane) {
+  bool same = true;
+#pragma unroll 1
+  for (int i = lane; i <= kmax && same; i += 32) {
+    const uint32_t* p = now + ((t - i) & (kFewRing - 1)) * words;
+    const uint32_t* q = snap + ((t_snap - i) & (kFewRing - 1)) * words;
+#pragma unroll 1
+    for (int b = 0; b < words; ++b) same = same && p[b] == q[b];
+  }
+  return __all_sync(kFull, same);
+}
+
+// First step from t on whose outcome is that of step max_steps of an orbit of
+// period P (the correction repeats with period 2P).
+static __device__ __noinline__ int orbit_stop(int t, int P, int max_steps) {
+  const int R = max_steps - t, per = R / P;
+  return t + (R - per * P) + ((per & 1) ? P : 0);
+}
+
+// PLAIN: lexicographic ties, a balanced axis stays, no random moves (the
+// default rules); the other forms read the rules from the arguments.
+template <int NT, bool LARGE, bool PLAIN>
 struct Decoder {
   using Ent = typename std::conditional<LARGE, uint32_t, uint16_t>::type;
+  // crossing table: bits of a link (word of the link maps and bit), steps it
+  // tells apart
+  static constexpr int kIdBits = LARGE ? 21 : 17;
+  static constexpr int kEpochs = LARGE ? 1023 : 16383;
 
   const DecodeArgs& a;
   const Geom& g;
   uint32_t* ring;    // [kmask + 1][nws] (LARGE: [kLargeRing][nws])
   uint32_t* C;       // [2][nws] correction
-  uint32_t* F;       // [2][nws] links flipped this step
+  uint32_t* F;       // LARGE or c_global: [2][nws] links flipped in a dense step
   uint32_t* list;    // [list_cap] anyons (y << 16 | x)
-  Ent* few;          // [kFewRing][kFew], then the snapshot
+  uint32_t* table;   // [tmask + 1] links crossed toward an anyon in a listed step
+  Ent* few;          // [kFewRing][kFew]
+  uint32_t* snap;    // [2][kFewWords] snapshots of it
   int* misc;         // 0-2 rotating counters, 3 miss, 4 steps, 5 flag, 6-7 cuts
-  uint32_t* spill;   // [nspill][nws] in the correction block
-  int nspill;
+  uint16_t* nset;    // [128] anyons in the archived set of a step, or kNoSet
+  Archive ar;
   int64_t shot;
   int tid, lane, warp;
   int ph;            // rotating counter in use
   int tb;            // step of the newest bitmap
+
+  __device__ __forceinline__ bool literal() const {
+    return !PLAIN && a.tie_order == QCA_TIE_LITERAL;
+  }
+  __device__ __forceinline__ bool moves_random() const { return !PLAIN && a.move_thr != 0; }
+  __device__ __forceinline__ bool balance_random() const { return !PLAIN && a.balance_rule != 0; }
 
   __device__ __forceinline__ void sync() const {
     if (NT == 32) {
@@ -350,27 +467,20 @@ struct Decoder {
   // bitmap of sigma_s for a step s <= tb + 1 (tb + 1: the next one, being made)
   __device__ __forceinline__ uint32_t* slot(int s) const {
     if (LARGE) return ring + (size_t)(s % kLargeRing) * g.nws;
-    return ring + (s & g.kmask) * g.nws;
+    return ring + (s & g.kmask) * g.nslot;
   }
-  // bitmap of the older sigma_s, or null when it is no longer kept
-  __device__ __forceinline__ const uint32_t* past(int s) const {
-    if (LARGE) return slot(s);
-    const int oldest = tb - g.kmask + 1;  // the slot of tb + 1 is already reused
-    if (s >= oldest) return slot(s);
-    if (s < oldest - nspill) return nullptr;
-    return spill + (s % nspill) * g.nws;
+  // oldest syndrome whose bitmap is in its slot
+  __device__ __forceinline__ int oldest() const { return LARGE ? 0 : ar.next; }
+  // x- / y-link map of dense step t: their own place, or the two slots with the
+  // oldest syndromes
+  __device__ __forceinline__ bool maps_in_slots() const { return !LARGE && !g.c_global; }
+  __device__ __forceinline__ uint32_t* map_x(int t) const {
+    return maps_in_slots() ? slot(t + 2) : F;
+  }
+  __device__ __forceinline__ uint32_t* map_y(int t) const {
+    return maps_in_slots() ? slot(t + 3) : F + g.nws;
   }
 
-  // Sum of n over the CTA through rotating counter ph; ends with a barrier.
-  __device__ __forceinline__ int total(int n) {
-    n = __reduce_add_sync(kFull, n);
-    if (NT == 32) {
-      __syncwarp();
-      return n;
-    }
-    if (lane == 0 && n) atomicAdd(&misc[ph], n);
-    return next_counter();
-  }
   // Barrier, value of counter ph, and on to the next one (the one after it is cleared).
   __device__ __forceinline__ int next_counter() {
     sync();
@@ -380,89 +490,161 @@ struct Decoder {
     ph = ph == 2 ? 0 : ph + 1;
     return v;
   }
+  // Barrier with the OR of p over the CTA.
+  __device__ __forceinline__ bool sync_or(bool p) const {
+    if (NT == 32) {
+      const bool any = __any_sync(kFull, p);
+      __syncwarp();
+      return any;
+    }
+    return __syncthreads_or(p);
+  }
+  // Sum of n over the CTA; ends with a barrier.
+  __device__ __forceinline__ int total(int n) {
+    n = __reduce_add_sync(kFull, n);
+    if (NT == 32) {
+      __syncwarp();
+      return n;
+    }
+    if (lane == 0 && n) atomicAdd(&misc[ph], n);
+    return next_counter();
+  }
+  // Place of this thread's n entries in a list of all threads' entries.
+  __device__ __forceinline__ int places(int n) {
+    int incl = n;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(kFull, incl, o);
+      if (lane >= o) incl += v;
+    }
+    int base = 0;
+    if (lane == 31 && incl) base = atomicAdd(&misc[ph], incl);
+    return __shfl_sync(kFull, base, 31) + incl - n;
+  }
 
-  // Makes sigma_s (in its slot) the newest bitmap: moves the oldest one out of
-  // the slot of s + 1, copies sigma_s there (the listed mode flips bits in it)
-  // and, if asked, lists the anyons.  Returns their number; ends with a barrier.
-  __device__ __forceinline__ int advance(int s, bool do_list) {
-    const uint32_t* cur = slot(s);
-    uint32_t* nxt = slot(s + 1);
-    const int old = s + 1 - (g.kmask + 1);
-    uint32_t* sp = (!LARGE && nspill && old >= 0) ? spill + (old % nspill) * g.nws : nullptr;
-    const int wsm = (1 << g.lws) - 1;
-    int n = 0;
-    for (int w = tid; w < g.nws; w += NT) {
-      const uint32_t v = cur[w];
-      if (sp) sp[w] = nxt[w];
-      nxt[w] = v;
-      n += __popc(v);
+  // Makes sigma_s (in its slot) the newest bitmap, and moves the syndrome in the
+  // slot of s + 1 to the archive, in a dense step perhaps also those in the slots
+  // of s + 2 and s + 3, which become the link maps.  listed: copies sigma_s to the
+  // slot of s + 1, where the moves will flip bits, and lists the anyons; returns
+  // their number.  Ends with a barrier.
+  __device__ __forceinline__ int advance(int s, bool listed) {
+    const uint4* cur = reinterpret_cast<const uint4*>(slot(s));
+    uint4* nxt = reinterpret_cast<uint4*>(slot(s + 1));
+    const int n4 = g.nslot >> 2;
+    if (!LARGE) {
+      const int end = (listed || !maps_in_slots() ? s + 1 : s + 3) - g.kmask;
+      bool any = false;
+#pragma unroll 1
+      for (; ar.next < end; ++ar.next) {
+        const int old = ar.next;
+        if (!g.spill || nset[old & 127] != kNoSet) continue;
+        // (the archive is on a 4-byte boundary)
+        uint32_t* to = ar.bitmaps + (old % ar.nb) * g.nws;
+        const uint32_t* from = slot(old);
+#pragma unroll 2
+        for (int w = tid; w < g.nws; w += NT) to[w] = from[w];
+        ar.gone = old + 1;
+        any = true;
+      }
+      if (any) sync();
     }
     tb = s;
-    if (do_list) {
-      int incl = n;
+    if (!listed) {
+      if (!LARGE && tid == 0) nset[s & 127] = kNoSet;
+      sync();
+      return 0;
+    }
+    int n = 0;
+#pragma unroll 2
+    for (int i = tid; i < n4; i += NT) {
+      const uint4 v = cur[i];
+      nxt[i] = v;
+      n += __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w);
+    }
+    int pos = places(n);
+    if (n) {
+      uint16_t* set = ar.sets + (LARGE ? 0 : (s % kArchiveSets) * ar.cap);
+      const int wsm = (1 << g.lws) - 1;
+#pragma unroll 1
+      for (int i = tid; i < n4; i += NT) {
+        const uint4 v = cur[i];
+        if (!(v.x | v.y | v.z | v.w)) continue;
+        const uint32_t q4[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int v = __shfl_up_sync(kFull, incl, o);
-        if (lane >= o) incl += v;
-      }
-      int base = 0;
-      if (lane == 31 && incl) base = atomicAdd(&misc[ph], incl);
-      base = __shfl_sync(kFull, base, 31);
-      int pos = base + incl - n;
-      if (n) {
-        for (int w = tid; w < g.nws; w += NT) {
-          uint32_t b = cur[w];
+        for (int q = 0; q < 4; ++q) {
+          uint32_t b = q4[q];
+          const int w = 4 * i + q;
           const uint32_t yx = ((uint32_t)(w >> g.lws) << 16) | ((w & wsm) << 5);
           while (b) {
-            const int q = __ffs(b) - 1;
+            const uint32_t e = yx + __ffs(b) - 1;
             b &= b - 1;
-            if (pos < g.list_cap) list[pos] = yx + q;
+            list[pos] = e;
+            if (!LARGE && pos < ar.cap) set[pos] = (uint16_t)((e >> 8) | (e & 0xFFu));
             ++pos;
           }
         }
       }
-      return next_counter();
     }
-    sync();
-    return 0;
+    const int all = next_counter();
+    if (!LARGE && tid == 0) nset[s & 127] = all <= ar.cap ? (uint16_t)all : kNoSet;
+    return all;
   }
 
   __device__ __forceinline__ uint32_t site(int x, int y) const { return (uint32_t)(y * g.L + x); }
 
-  // Slices 1 .. of the anyon at (x, y) by the whole warp; returns the first
-  // slice's hits (0: nothing heard) and its index in k.
+  // One slice of the anyon at (x, y) by the whole warp, wherever the syndrome is.
+  __device__ __forceinline__ uint32_t far_slice(int x, int y, int t, int k) const {
+    const int s = t - k;
+    const uint32_t* sig = nullptr;
+    uint32_t m = 0;
+    if (LARGE || s >= oldest()) {
+      sig = slot(s);
+    } else if (nset[s & 127] != kNoSet) {
+      m = slice_list(ar.sets + (s % kArchiveSets) * ar.cap, nset[s & 127], g.L, x, y, k, lane);
+    } else if (s >= ar.gone - ar.nb) {
+      sig = ar.bitmaps + (s % ar.nb) * g.nws;
+    } else {
+      misc[3] = 1;  // the shot needs a syndrome that is no longer kept
+    }
+    if (sig) m = slice_warp(sig, g.lws, g.L, x, y, k, lane);
+    return m & slice_limit(a.m_max, k);
+  }
+  // Slices from k on by the whole warp; returns the first slice's hits (0:
+  // nothing heard) and its index in k.
   __device__ __forceinline__ uint32_t search_far(int x, int y, int t, int& k) const {
     const int last = min(t, g.kmax);
+    uint32_t m = 0;
+#pragma unroll 1
     for (; k <= last; ++k) {
-      const uint32_t* sig = past(t - k);
-      if (!sig) {
-        misc[3] = 1;  // the shot needs a syndrome that is no longer kept
-        return 0;
-      }
-      const uint32_t m = slice_warp(sig, g.lws, g.L, x, y, k, lane) & slice_limit(a.m_max, k);
-      if (m) return m;
+      m = far_slice(x, y, t, k);
+      if (m || (!LARGE && misc[3])) break;
     }
-    return 0;
+    return m;
   }
 
-  struct Keys {
-    uint64_t move, bal;
-  };
   __device__ __forceinline__ Keys keys_of(int t) const {
     Keys q{0, 0};
-    if (a.move_thr) q.move = move_step_key(a.move_key, a.shot_offset + shot, t);
-    if (a.balance_rule) q.bal = move_step_key(a.balance_key, a.shot_offset + shot, t);
+    if (moves_random()) q.move = key_of(a.move_key, a.shot_offset + shot, t);
+    if (balance_random()) q.bal = key_of(a.balance_key, a.shot_offset + shot, t);
     return q;
   }
-  // Random move of the anyon at site r, or 0.
-  __device__ __forceinline__ int drawn_move(const Keys& q, uint32_t r) const {
-    if (!a.move_thr) return 0;
-    const uint64_t u = splitmix64(q.move ^ (uint64_t)r);
-    return u < a.move_thr ? 1 + (int)(splitmix64(u) >> 62) : 0;
-  }
-  __device__ __forceinline__ int resolve(int dir, const Keys& q, uint32_t r) const {
-    if (dir >= 5) dir = a.balance_rule ? balance_resolve(dir, q.bal, r) : 0;
+  // The move of the anyon at (x, y) that hears h0 (and h1 at the next distance).
+  __device__ __forceinline__ int move_of(const Keys& key, int x, int y, uint32_t h0,
+                                         uint32_t h1) const {
+    int dir = h0 ? direction(h0, h1, PLAIN ? QCA_TIE_LEX : a.tie_order) : 0;
+    if (dir >= 5) dir = balance_random() ? draw_balance(dir, key.bal, site(x, y)) : 0;
+    if (moves_random()) {
+      const int d = draw_move(key.move, a.move_thr, site(x, y));
+      if (d) dir = d;
+    }
     return dir;
+  }
+  // Hits at the smallest distance of a slice's hits, and at the next one (0
+  // past the slice's third distance).
+  __device__ __forceinline__ void nearest(uint32_t m, uint32_t& h0, uint32_t& h1) const {
+    const int d4 = (__ffs(m) - 1) & ~3;
+    h0 = (m >> d4) & 15u;
+    h1 = (m >> (d4 + 4)) & 15u;
   }
 
   // Lower end of the link an anyon at (x, y) crosses when it moves: word of the
@@ -473,41 +655,66 @@ struct Decoder {
     bit = 1u << (lx & 31);
     return (dir >= 3 ? g.nws : 0) + (ly << g.lws) + (lx >> 5);
   }
+  __device__ __forceinline__ uint32_t site_after(int x, int y, int dir) const {
+    if (dir == 1) x = wrap_hi(x + 1, g.L);
+    if (dir == 2) x = wrap_lo(x - 1, g.L);
+    if (dir == 3) y = wrap_hi(y + 1, g.L);
+    if (dir == 4) y = wrap_lo(y - 1, g.L);
+    return ((uint32_t)y << 16) | x;
+  }
 
-  // Decides and marks the moves of the n listed anyons at step t.  LISTED: the
-  // correction and the copy of sigma in the next slot are flipped at once and
-  // the marked words are returned in mark[] (4 per thread at most); else only
-  // the link map is marked.
-  template <bool LISTED>
-  __device__ __forceinline__ void move_listed(int n, int t, int (&mark)[4]) {
-    constexpr int NW = NT / 32;
+  // Whether this is the first crossing of a link (id) in step t: the anyons that
+  // cross it toward one another both ask.  Entries carry the step, so the table
+  // is cleared only once in kEpochs + 1 steps.
+  __device__ __forceinline__ bool first_crossing(uint32_t id, int t) const {
+    const uint32_t key = ((uint32_t)(t & kEpochs) + 1u) << kIdBits | id;
+    uint32_t h = (id * 0x9E3779B1u) >> 16;
+#pragma unroll 1
+    for (;; ++h) {
+      uint32_t* e = &table[h & g.tmask];
+      uint32_t old = *(volatile uint32_t*)e;
+      while ((old >> kIdBits) != (key >> kIdBits)) {  // free in this step
+        const uint32_t was = atomicCAS(e, old, key);
+        if (was == old) return true;
+        old = was;
+      }
+      if (old == key) return false;
+    }
+  }
+
+  // Decides and marks the moves of the n listed anyons at step t, a thread per
+  // anyon.  listed: the correction and the copy of sigma in the next slot are
+  // flipped at once; else (dense step) only the link map is marked.  Returns
+  // whether this thread's anyons moved.
+  __device__ __forceinline__ bool move_listed(int n, int t, bool listed) {
+    bool moved = false;
     const uint32_t* sig = slot(t);
     uint32_t* sn = slot(t + 1);
     const Keys key = keys_of(t);
-    const uint32_t lim0 = slice_limit(a.m_max, 0);
-    const bool far = t > 0 && g.kmax > 0;
-    auto one = [&](int it, int& mk) {
-      // consecutive list entries go to different warps
-      const int i = it * NT + lane * NW + warp;
+    const int last = min(t, g.kmax);
+    const int lastt = min(min(last, g.kthread), t - oldest());
+#pragma unroll 1
+    for (int i0 = tid - lane; i0 < n; i0 += NT) {
+      const int i = i0 + lane;
       const bool act = i < n;
-      int x = 0, y = 0, dir = 0, k = 0;
+      int x = 0, y = 0, k = 0;
       uint32_t m = 0;
-      bool need = false, edge = false;
       if (act) {
         const uint32_t e = list[i];
         x = e & 0xFFFFu;
         y = e >> 16;
-        dir = drawn_move(key, site(x, y));
-        if (!dir) {
-          m = slice0(sig, g.lws, g.L, x, y) & lim0;
-          need = far && m == 0;
+#pragma unroll 1
+        for (;; ++k) {
+          m = slice_thread(slot(t - k), g.lws, g.L, x, y, k) & slice_limit(a.m_max, k);
+          if (m || k >= lastt) break;
         }
       }
-      uint32_t todo = __ballot_sync(kFull, need);
+      uint32_t todo = __ballot_sync(kFull, act && m == 0 && lastt < last);
+#pragma unroll 1
       while (todo) {
         const int src = __ffs(todo) - 1;
         todo &= todo - 1;
-        int kk = 1;
+        int kk = lastt + 1;
         const uint32_t mm = search_far(__shfl_sync(kFull, x, src), __shfl_sync(kFull, y, src), t,
                                        kk);
         if (lane == src) {
@@ -516,257 +723,349 @@ struct Decoder {
         }
       }
       uint32_t h0 = 0, h1 = 0;
-      if (m) {
-        const int d4 = (__ffs(m) - 1) & ~3;
-        h0 = (m >> d4) & 15u;
-        h1 = (m >> (d4 + 4)) & 15u;  // 0 past the slice's third distance
-        edge = d4 == 8 && needs_next(h0, a.tie_order) && k < min(t, g.kmax);
-      }
-      todo = __ballot_sync(kFull, edge);
-      while (todo) {
-        // the next distance is the first one of the next slice
-        const int src = __ffs(todo) - 1;
-        todo &= todo - 1;
-        const int ks = __shfl_sync(kFull, k, src) + 1;
-        const uint32_t* ps = past(t - ks);
-        uint32_t mm = 0;
-        if (ps) {
-          mm = slice_warp(ps, g.lws, g.L, __shfl_sync(kFull, x, src), __shfl_sync(kFull, y, src),
-                          ks, lane) & slice_limit(a.m_max, ks);
-        } else {
-          misc[3] = 1;
+      if (m) nearest(m, h0, h1);
+      if (literal()) {
+        // the next distance may be the first one of the next slice
+        todo = __ballot_sync(kFull, h0 && !(m & 0xFFu) && !(h0 & 10u) && k < last);
+#pragma unroll 1
+        while (todo) {
+          const int src = __ffs(todo) - 1;
+          todo &= todo - 1;
+          const uint32_t mm = far_slice(__shfl_sync(kFull, x, src), __shfl_sync(kFull, y, src), t,
+                                        __shfl_sync(kFull, k, src) + 1);
+          if (lane == src) h1 = mm & 15u;
         }
-        if (lane == src) h1 = mm & 15u;
       }
-      if (h0) dir = resolve(direction(h0, h1, a.tie_order), key, site(x, y));
+      const int dir = act ? move_of(key, x, y, h0, h1) : 0;
       if (dir) {
+        moved = true;
         uint32_t bit;
         const int w = link_of(x, y, dir, bit);
-        if (LISTED) {
-          mk = w;
-          if (!(atomicOr(&F[w], bit) & bit)) {
-            const int nx = dir == 1 ? wrap_hi(x + 1, g.L) : (dir == 2 ? wrap_lo(x - 1, g.L) : x);
-            const int ny = dir == 3 ? wrap_hi(y + 1, g.L) : (dir == 4 ? wrap_lo(y - 1, g.L) : y);
+        if (!listed) {
+          atomicOr(w < g.nws ? map_x(t) + w : map_y(t) + (w - g.nws), bit);
+        } else {
+          const uint32_t to = site_after(x, y, dir);
+          const int nx = to & 0xFFFFu, ny = to >> 16;
+          const int wn = (ny << g.lws) + (nx >> 5);
+          // two anyons that swap sites cross one link, which flips once
+          if (!((sig[wn] >> (nx & 31)) & 1u) ||
+              first_crossing((uint32_t)w << 5 | (__ffs(bit) - 1), t)) {
             atomicXor(&C[w], bit);
             atomicXor(&sn[(y << g.lws) + (x >> 5)], 1u << (x & 31));
-            atomicXor(&sn[(ny << g.lws) + (nx >> 5)], 1u << (nx & 31));
+            atomicXor(&sn[wn], 1u << (nx & 31));
           }
-        } else {
-          atomicOr(&F[w], bit);
         }
       }
-    };
-    if (LISTED) {
-#pragma unroll
-      for (int it = 0; it < 4; ++it) {
-        mark[it] = -1;
-        if (it * NT < n) one(it, mark[it]);
-      }
-    } else {
-      int unused;
-      for (int it = 0; it * NT < n; ++it) one(it, unused);
     }
+    return moved;
   }
 
-  // One anyon decided by one thread alone, all slices (the list is full).
-  // A static function on a copy, so that the kernel's own state stays in registers.
-  static __device__ __noinline__ int decide_alone(const Decoder self, int x, int y, int t,
-                                                  const Keys key) {
-    return self.decide(x, y, t, key);
+  // Dense steps go through the bitmaps in strips of rows: lane group of 2^lws
+  // lanes = the words of a row, each group a strip of consecutive rows, so that
+  // a row is read once and its neighbours in the row come by shuffles.
+  struct Strip {
+    int j;              // word of the row
+    int jl, jr;         // lanes of the words to the left and to the right
+    int sl, top;        // bit of the left word that is column x - 1 of this word's first
+                        // column, bit of this word that is its last column
+    uint32_t valid;     // this word's columns
+    int y0, y1;         // rows
+  };
+  __device__ __forceinline__ Strip strip() const {
+    const int lws = g.lws, wpr = 1 << lws, lastw = (g.L - 1) >> 5, lastb = (g.L - 1) & 31;
+    const int H = (g.L + (NT >> lws) - 1) / (NT >> lws);
+    Strip p;
+    p.j = lane & (wpr - 1);
+    const int base = lane - p.j;
+    p.jl = base + (p.j == 0 ? lastw : p.j - 1);
+    p.jr = base + (p.j >= lastw ? 0 : p.j + 1);
+    p.sl = p.j == 0 ? lastb : 31;
+    p.top = p.j == lastw ? lastb : 31;
+    p.valid = p.j < lastw ? kFull : (p.j == lastw ? kFull >> (31 - lastb) : 0u);
+    p.y0 = min((tid >> lws) * H, g.L);
+    p.y1 = min(p.y0 + H, g.L);
+    return p;
   }
-  __device__ __forceinline__ int decide(int x, int y, int t, const Keys& key) const {
-    int dir = drawn_move(key, site(x, y));
-    if (dir) return dir;
-    const int last = min(t, g.kmax);
-    uint32_t h0 = 0;
-    for (int k = 0; k <= last; ++k) {
-      const uint32_t* sig = past(t - k);
-      if (!sig) {
-        misc[3] = 1;
-        return 0;
-      }
-      uint32_t m = 0;
-      if (k == 0) {
-        m = slice0(sig, g.lws, g.L, x, y);
-      } else {
-        for (int d = 1; d <= 3; ++d) {
-          const int reach = 3 * k + d, dr = reach % g.L, wpr = 1 << g.lws;
-          const int xl = wrap_lo(x - dr, g.L), xr = wrap_hi(x + dr, g.L);
-          const int half = min(reach, g.L >> 1);
-          uint32_t h = 0;
-          for (int j = -half; j <= half; ++j) {
-            const uint32_t* row = sig + (wrap_hi(wrap_lo(y + j, g.L), g.L) << g.lws);
-            h |= ((row[xl >> 5] >> (xl & 31)) & 1u) | (((row[xr >> 5] >> (xr & 31)) & 1u) << 1);
-          }
-          h |= row_any(sig + (wrap_lo(y - dr, g.L) << g.lws), wpr, g.L, x, reach) << 2;
-          h |= row_any(sig + (wrap_hi(y + dr, g.L) << g.lws), wpr, g.L, x, reach) << 3;
-          m |= h << (4 * (d - 1));
-        }
-      }
-      m &= slice_limit(a.m_max, k);
-      if (h0) return resolve(direction(h0, m & 15u, a.tie_order), key, site(x, y));
-      if (m) {
-        const int d4 = (__ffs(m) - 1) & ~3;
-        h0 = (m >> d4) & 15u;
-        if (d4 < 8 || !needs_next(h0, a.tie_order))
-          return resolve(direction(h0, (m >> (d4 + 4)) & 15u, a.tie_order), key, site(x, y));
-      }
-    }
-    return h0 ? resolve(direction(h0, 0, a.tie_order), key, site(x, y)) : 0;
+  __device__ __forceinline__ int strip_rows() const {
+    return (g.L + (NT >> g.lws) - 1) / (NT >> g.lws);
+  }
+  // v shifted by one column: bit x = column x - 1 / x + 1 of the row
+  __device__ __forceinline__ uint32_t from_left(uint32_t v, const Strip& p) const {
+    return (v << 1) | ((__shfl_sync(kFull, v, p.jl) >> p.sl) & 1u);
+  }
+  __device__ __forceinline__ uint32_t from_right(uint32_t v, const Strip& p) const {
+    return (v >> 1) | ((__shfl_sync(kFull, v, p.jr) & 1u) << p.top);
   }
 
-  // Dense step t: distance 1 of every anyon 32 sites at a time, the others
-  // listed.  Marks the crossed links; returns the number listed (ends with a
-  // barrier).
-  __device__ __forceinline__ int mark_dense(int t) {
-    const uint32_t* sig = slot(t);
-    const int L = g.L, lws = g.lws, wsm = (1 << lws) - 1;
-    const int lastw = (L - 1) >> 5, lastb = (L - 1) & 31;
+  // Dense step t: distance 1 of every anyon, 32 sites per word.  Writes the link
+  // map, and the undecided anyons as a bitmap to the next slot; returns this
+  // thread's number of them.
+  __device__ __forceinline__ int mark_dense(int t, const Strip& p) {
+    const uint32_t* sig = slot(t) + p.j;
+    uint32_t* open = slot(t + 1) + p.j;
+    uint32_t *fxp = map_x(t) + p.j, *fyp = map_y(t) + p.j;
+    const int L = g.L, lws = g.lws, H = strip_rows();
     const Keys key = keys_of(t);
-    const bool lit = a.tie_order == QCA_TIE_LITERAL;
-    for (int w = tid; w < g.nws; w += NT) {
-      const uint32_t c = sig[w];
-      if (!c) continue;
-      const int y = w >> lws, j = w & wsm;
-      const int yu = y == 0 ? L - 1 : y - 1, yd = y == L - 1 ? 0 : y + 1;
-      const int jl = j == 0 ? lastw : j - 1, jr = j == lastw ? 0 : j + 1;
-      const int sl = j == 0 ? lastb : 31, top = j == lastw ? lastb : 31;
-      uint32_t todo;
-      if (a.move_thr) {
-        todo = c;  // any anyon may be drawn to move: one by one
-      } else {
-        const uint32_t *ru = sig + (yu << lws), *r0 = sig + (y << lws), *rd = sig + (yd << lws);
-        const uint32_t u = ru[j], d = rd[j];
-        const uint32_t ul = (ru[jl] >> sl) & 1u, cl = (r0[jl] >> sl) & 1u, dl = (rd[jl] >> sl) & 1u;
-        const uint32_t ur = (ru[jr] & 1u) << top, cr = (r0[jr] & 1u) << top,
-                       dr = (rd[jr] & 1u) << top;
-        const uint32_t v = u | c | d;
-        const uint32_t px = (v << 1) | ul | cl | dl;  // anyon in column x - 1
-        const uint32_t mx = (v >> 1) | ur | cr | dr;  // in column x + 1
-        const uint32_t py = u | (u << 1) | ul | (u >> 1) | ur;
-        const uint32_t my = d | (d << 1) | dl | (d >> 1) | dr;
-        uint32_t mpx, mmx, mpy, mmy, bx, by;  // moves +x, -x, +y, -y; balanced axes
-        todo = c & ~(px | mx | py | my);
-        mpy = c & my & ~py;
-        by = c & my & py;
-        uint32_t xs = c & ~my & (px | mx);
-        mmy = c & py & ~(my | px | mx);
-        if (lit) {
-          // +x or +y alone at distance 1 may lose to -y or -x at distance 2
-          todo |= c & ~(my | mx) & (px | py);
-          xs &= mx;
-          mmy = 0;
-        }
-        mpx = xs & mx & ~px;
-        mmx = xs & px & ~mx;
-        bx = xs & px & mx;
-        if (a.balance_rule) {
-          for (uint32_t b = bx; b; b &= b - 1) {
-            const int q = __ffs(b) - 1;
-            if (balance_resolve(5, key.bal, site((j << 5) + q, y)) == 1) mpx |= 1u << q;
-            else mmx |= 1u << q;
-          }
-          for (uint32_t b = by; b; b &= b - 1) {
-            const int q = __ffs(b) - 1;
-            if (balance_resolve(6, key.bal, site((j << 5) + q, y)) == 3) mpy |= 1u << q;
-            else mmy |= 1u << q;
-          }
-        }
-        const uint32_t fx = mpx | (mmx >> 1);
-        if (fx) atomicOr(&F[w], fx);
-        if (mmx & 1u) atomicOr(&F[(y << lws) + jl], 1u << sl);
-        if (mpy) atomicOr(&F[g.nws + w], mpy);
-        if (mmy) atomicOr(&F[g.nws + (yu << lws) + j], mmy);
+    const bool on = p.valid != 0 && p.y0 < L;
+    int n = 0, y = p.y0;
+    auto row = [&](int r) { return on ? sig[wrap_hi(wrap_lo(r, L), L) << lws] : 0u; };
+    // rows y - 1 (u), y (c), y + 1 (d), each with its shifted copies
+    uint32_t u = row(y - 1), c = row(y);
+    uint32_t ul = from_left(u, p), ur = from_right(u, p);
+    uint32_t cl = from_left(c, p), cr = from_right(c, p);
+    uint32_t up = 0;  // +y moves of the row before
+    // one row more than the strip has: its -y moves cross the last row's links
+#pragma unroll 1
+    for (int i = 0; i <= H; ++i, ++y) {
+      const uint32_t d = row(y + 1);
+      const uint32_t dl = from_left(d, p), dr = from_right(d, p);
+      const uint32_t px = ul | cl | dl;  // anyon in column x - 1
+      const uint32_t mx = ur | cr | dr;  // in column x + 1
+      const uint32_t py = u | ul | ur, my = d | dl | dr;
+      uint32_t todo = c & ~(px | mx | py | my);
+      uint32_t mpy = c & my & ~py;  // moves +y
+      uint32_t xs = c & ~my & (px | mx);
+      uint32_t mmy = c & py & ~(my | px | mx);
+      if (literal()) {
+        // +x or +y alone at distance 1 may lose to -y or -x at distance 2
+        todo |= c & ~(my | mx) & (px | py);
+        xs &= mx;
+        mmy = 0;
       }
-      if (todo) {
-        int pos = atomicAdd(&misc[ph], __popc(todo));
-        while (todo) {
-          const int q = __ffs(todo) - 1;
-          todo &= todo - 1;
-          if (pos < g.list_cap) {
-            list[pos] = ((uint32_t)y << 16) | ((j << 5) + q);
-          } else {
-            const int x = (j << 5) + q;
-            const int dir = decide_alone(*this, x, y, t, key);
-            if (dir) {
-              uint32_t bit;
-              const int lw = link_of(x, y, dir, bit);
-              atomicOr(&F[lw], bit);
-            }
-          }
-          ++pos;
+      uint32_t mpx = xs & mx & ~px, mmx = xs & px & ~mx;
+      if (balance_random()) {
+#pragma unroll 1
+        for (uint32_t b = xs & px & mx; b; b &= b - 1) {
+          const int q = __ffs(b) - 1;
+          if (draw_balance(5, key.bal, site((p.j << 5) + q, wrap_hi(y, L))) == 1) mpx |= 1u << q;
+          else mmx |= 1u << q;
         }
+#pragma unroll 1
+        for (uint32_t b = c & my & py; b; b &= b - 1) {
+          const int q = __ffs(b) - 1;
+          if (draw_balance(6, key.bal, site((p.j << 5) + q, wrap_hi(y, L))) == 3) mpy |= 1u << q;
+          else mmy |= 1u << q;
+        }
+      }
+      if (moves_random()) {  // any anyon may be drawn to move: one by one
+        todo = c;
+        mpx = mmx = mpy = mmy = 0;
+      }
+      const uint32_t fx = mpx | from_right(mmx, p);
+      if (on) {
+        if (i > 0 && y <= p.y1) fyp[(y - 1) << lws] = up | mmy;
+        if (y < p.y1) {
+          fxp[y << lws] = fx;
+          open[y << lws] = todo;
+          n += __popc(todo);
+        }
+      }
+      up = mpy;
+      u = c, ul = cl, ur = cr;
+      c = d, cl = dl, cr = dr;
+    }
+    return n;
+  }
+
+  // Anyons r0 .. r0 + list_cap - 1 of the undecided ones to the list (this
+  // thread's n start at place pos).
+  __device__ __forceinline__ void list_open(int t, const Strip& p, int n, int pos, int r0) {
+    if (n == 0 || pos >= r0 + g.list_cap || pos + n <= r0) return;
+    const uint32_t* open = slot(t + 1) + p.j;
+#pragma unroll 1
+    for (int y = p.y0; y < p.y1; ++y) {
+      uint32_t b = open[y << g.lws];
+      while (b) {
+        const uint32_t e = ((uint32_t)y << 16) | ((p.j << 5) + __ffs(b) - 1);
+        b &= b - 1;
+        if (pos >= r0 && pos < r0 + g.list_cap) list[pos - r0] = e;
+        ++pos;
       }
     }
-    return min(next_counter(), g.list_cap);
   }
 
   // sigma_{t+1} and the correction from the marked links; the anyons left (ends
-  // with a barrier).
-  __device__ __forceinline__ int apply_dense(int t) {
-    const uint32_t* sig = slot(t);
-    uint32_t* sn = slot(t + 1);
-    const int L = g.L, lws = g.lws, wsm = (1 << lws) - 1;
-    const int lastw = (L - 1) >> 5, lastb = (L - 1) & 31;
+  // with a barrier).  moved: whether a link of this thread's flipped.
+  __device__ __forceinline__ int apply_dense(int t, const Strip& p, bool& moved) {
+    const uint32_t* sig = slot(t) + p.j;
+    uint32_t* sn = slot(t + 1) + p.j;
+    const uint32_t *fxp = map_x(t) + p.j, *fyp = map_y(t) + p.j;
+    uint32_t *cx = C + p.j, *cy = C + g.nws + p.j;
+    const int lws = g.lws, H = strip_rows();
+    const bool on = p.valid != 0 && p.y0 < g.L;
     int n = 0;
-    for (int w = tid; w < g.nws; w += NT) {
-      const int y = w >> lws, j = w & wsm;
-      if (j > lastw) continue;  // padding word (stays 0)
-      const int yu = y == 0 ? L - 1 : y - 1;
-      const uint32_t fx = F[w], fy = F[g.nws + w], fu = F[g.nws + (yu << lws) + j];
-      const uint32_t carry =
-          j ? F[w - 1] >> 31 : (F[(y << lws) + lastw] >> lastb) & 1u;
-      const uint32_t valid = j == lastw ? kFull >> (31 - lastb) : kFull;
-      const uint32_t s = sig[w] ^ ((fx ^ ((fx << 1) | carry) ^ fy ^ fu) & valid);
-      sn[w] = s;
-      n += __popc(s);
-      if (fx) C[w] ^= fx;
-      if (fy) C[g.nws + w] ^= fy;
+    if (!on && p.y0 < g.L) {  // padding words stay 0
+#pragma unroll 1
+      for (int y = p.y0; y < p.y1; ++y) sn[y << lws] = 0;
+    }
+    uint32_t fu = on ? fyp[wrap_lo(p.y0 - 1, g.L) << lws] : 0u;
+#pragma unroll 2
+    for (int y = p.y0; y < p.y0 + H; ++y) {
+      const bool in = on && y < p.y1;
+      const int o = y << lws;
+      const uint32_t fx = in ? fxp[o] : 0u;
+      const uint32_t fxl = from_left(fx, p);
+      if (in) {
+        const uint32_t fy = fyp[o];
+        const uint32_t s = sig[o] ^ ((fx ^ fxl ^ fy ^ fu) & p.valid);
+        sn[o] = s;
+        n += __popc(s);
+        fu = fy;
+        moved |= (fx | fy) != 0;
+        if (t == 0) {
+          cx[o] = fx;
+          cy[o] = fy;
+        } else if (maps_in_slots()) {
+          cx[o] ^= fx;
+          cy[o] ^= fy;
+        } else {
+          // (no value comes back, so a correction in global memory costs no wait)
+          if (fx) atomicXor(&cx[o], fx);
+          if (fy) atomicXor(&cy[o], fy);
+        }
+      }
     }
     return total(n);
   }
 
   // --------------------------------------------------------- few anyons
   __device__ __forceinline__ Ent enc(uint32_t p) const {
-    return LARGE ? (Ent)p : (Ent)(((p >> 16) << 8) | (p & 0xFFu));
+    return LARGE ? (Ent)p : (Ent)((p >> 8) | (p & 0xFFu));
   }
   __device__ __forceinline__ uint32_t dec(Ent e) const {
-    return LARGE ? (uint32_t)e : (((uint32_t)e >> 8) << 16) | ((uint32_t)e & 0xFFu);
+    return LARGE ? (uint32_t)e : (((uint32_t)e & 0xFF00u) << 8) | ((uint32_t)e & 0xFFu);
+  }
+  __device__ __forceinline__ Ent* set_of(int s) const {
+    return few + (s & (kFewRing - 1)) * kFew;
   }
   // Hits of slice k against the anyon set of step s (a set shorter than 8
-  // entries is filled with its first one).
-  __device__ __forceinline__ uint32_t slice_set(int s, int x, int y, int k) const {
-    const uint4* p = reinterpret_cast<const uint4*>(few + (s & (kFewRing - 1)) * kFew);
-    uint32_t e[kFew];
-    const uint4 v = p[0];
-    if constexpr (LARGE) {
-      const uint4 u = p[1];
-      e[0] = v.x, e[1] = v.y, e[2] = v.z, e[3] = v.w;
-      e[4] = u.x, e[5] = u.y, e[6] = u.z, e[7] = u.w;
-    } else {
-      e[0] = v.x & 0xFFFFu, e[1] = v.x >> 16, e[2] = v.y & 0xFFFFu, e[3] = v.y >> 16;
-      e[4] = v.z & 0xFFFFu, e[5] = v.z >> 16, e[6] = v.w & 0xFFFFu, e[7] = v.w >> 16;
-    }
-    int c = 3 * k + 1;
-    if (c >= g.L) c %= g.L;
+  // entries is filled with its first one); near: slice_near serves.
+  __device__ __forceinline__ uint32_t slice_set(int s, int x, int y, int k, bool near) const {
+    const Ent* e = set_of(s);
+    const Ent first = e[0];
+    Ent b = first;
     uint32_t m = 0;
-#pragma unroll
-    for (int q = 0; q < kFew; ++q) {
-      if (q > 0 && e[q] == e[0]) break;
-      const uint32_t b = dec((Ent)e[q]);
-      m |= slice_pair(x, y, (int)(b & 0xFFFFu), (int)(b >> 16), g.L, k, c);
+    int q = 0;
+    if (near) {
+#pragma unroll 1
+      do {
+        const uint32_t yx = dec(b);
+        m |= slice_near(x, y, (int)(yx & 0xFFFFu), (int)(yx >> 16), g.L, k);
+        if (++q == kFew) break;
+        b = e[q];
+      } while (b != first);
+    } else {
+      int c = 3 * k + 1;
+      if (c >= g.L) c %= g.L;
+#pragma unroll 1
+      do {
+        const uint32_t yx = dec(b);
+        m |= slice_pair(x, y, (int)(yx & 0xFFFFu), (int)(yx >> 16), g.L, k, c);
+        if (++q == kFew) break;
+        b = e[q];
+      } while (b != first);
     }
     return m & slice_limit(a.m_max, k);
   }
-  // Slice k of one anyon at step t by the whole warp, from the set or the bitmap.
-  __device__ __forceinline__ uint32_t slice_any(int x, int y, int t, int k, int tf) const {
-    if (t - k >= tf) return slice_set(t - k, x, y, k);
-    const uint32_t* sig = past(t - k);
-    if (!sig) {
-      misc[3] = 1;
-      return 0;
+  // Writes the anyons with alive set (np on lanes 0 .. n - 1) as the set of step
+  // t, sorted; returns the anyon of lane i < number in pos.
+  __device__ __forceinline__ uint32_t write_set(int t, uint32_t alive, uint32_t np, int n) {
+    int rank = 0;
+#pragma unroll 1
+    for (int q = 0; q < n; ++q) {
+      const uint32_t v = __shfl_sync(kFull, np, q);
+      rank += ((alive >> q) & 1u) && v < np;
     }
-    return slice_warp(sig, g.lws, g.L, x, y, k, lane) & slice_limit(a.m_max, k);
+    Ent* row = set_of(t);
+    const int left = __popc(alive);
+    if ((alive >> lane) & 1u) row[rank] = enc(np);
+    __syncwarp();
+    if (lane >= left && lane < kFew) row[lane] = row[0];
+    __syncwarp();
+    return lane < left ? dec(row[lane]) : 0u;
+  }
+
+  // Steps of two anyons from t on, for as long as they hear one another's (or
+  // their own) sites of the steps since t_pair: a loop
+  // short enough for the nearest instruction cache, since a pair that never
+  // meets runs it alone for hundreds of steps.  Stops before step t_event, before
+  // a step at which a snapshot's last set comes back (watched), and before a step
+  // it cannot decide; returns that step.  n becomes 0 when the pair meets.
+  __device__ __forceinline__ int pair_steps(int t, int t_pair, uint32_t& pos, int& n, int near,
+                                            bool watched, int t_kept, int t_moving,
+                                            int t_event) const {
+    constexpr int kWords = kFew * (int)sizeof(Ent) / 4;
+    const uint32_t* now = reinterpret_cast<const uint32_t*>(few);
+    uint32_t p0 = __shfl_sync(kFull, pos, 0), p1 = __shfl_sync(kFull, pos, 1);
+    const uint32_t none = LARGE ? kFull : 0u;  // no set begins with this word
+    uint32_t e1 = none, e2 = none;
+    if (watched && t_kept >= 0) e1 = snap[(t_kept & (kFewRing - 1)) * kWords];
+    if (watched && t_moving >= 0)
+      e2 = snap[kFewRing * kWords + (t_moving & (kFewRing - 1)) * kWords];
+    const int kk = lane & 15;
+    const int klim = min(near, a.m_max / 3) - 1;  // slices that m_max does not cut
+    const bool second = lane >= 16;
+#pragma unroll 1
+    for (const int t0 = t; t < t_event;) {
+      const uint32_t e = now[(t & (kFewRing - 1)) * kWords];
+      if ((e == e1 || e == e2) && t > t0) break;
+      const uint32_t pa = second ? p1 : p0;
+      const int xa = pa & 0xFFFFu, ya = pa >> 16;
+      const int lim = min(klim, t - t_pair);
+      uint32_t hm = 0;
+#pragma unroll 1
+      for (int k = kk; k - kk <= lim; k += 16) {
+        uint32_t m = 0;
+        if (k <= lim) {
+          const Ent* set = set_of(t - k);
+          const uint32_t b0 = dec(set[0]), b1 = dec(set[1]);
+          m = slice_near(xa, ya, (int)(b0 & 0xFFFFu), (int)(b0 >> 16), g.L, k) |
+              slice_near(xa, ya, (int)(b1 & 0xFFFFu), (int)(b1 >> 16), g.L, k);
+        }
+        const uint32_t seg = (__ballot_sync(kFull, m != 0) >> (lane & 16)) & 0xFFFFu;
+        const uint32_t mm = __shfl_sync(kFull, m, (lane & 16) | ((__ffs(seg) - 1) & 15));
+        if (!hm && seg) hm = mm;
+        if (__all_sync(kFull, hm != 0)) break;
+      }
+      if (lim == klim && !__all_sync(kFull, hm != 0)) {
+        // beyond half the torus
+        const int lim2 = min((a.m_max / 3) - 1, t - t_pair);
+#pragma unroll 1
+        for (int k = lim + 1 + kk; k - kk <= lim2; k += 16) {
+          uint32_t m = 0;
+          if (k <= lim2) m = slice_set(t - k, xa, ya, k, false);
+          const uint32_t seg = (__ballot_sync(kFull, m != 0) >> (lane & 16)) & 0xFFFFu;
+          const uint32_t mm = __shfl_sync(kFull, m, (lane & 16) | ((__ffs(seg) - 1) & 15));
+          if (!hm && seg) hm = mm;
+          if (__all_sync(kFull, hm != 0)) break;
+        }
+      }
+      uint32_t h0 = 0, h1 = 0;
+      if (hm) nearest(hm, h0, h1);
+      // (literal ties may ask for a distance of the next slice)
+      if (!__all_sync(kFull, hm != 0 && !(literal() && !(hm & 0xFFu) && !(h0 & 10u)))) break;
+      int dir = direction(h0, h1, PLAIN ? QCA_TIE_LEX : a.tie_order);
+      if (dir >= 5) dir = 0;
+      const uint32_t np = dir ? site_after(xa, ya, dir) : pa;
+      const uint32_t q0 = __shfl_sync(kFull, np, 0), q1 = __shfl_sync(kFull, np, 16);
+      const bool swap = q0 == p1 && q1 == p0;
+      if (kk == 0 && dir && !(swap && second)) {
+        uint32_t bit;
+        const int w = link_of(xa, ya, dir, bit);
+        atomicXor(&C[w], bit);
+      }
+      ++t;
+      if (swap || q0 == q1) {
+        n = 0;
+        return t;
+      }
+      p0 = min(q0, q1);
+      p1 = max(q0, q1);
+      if (lane < kFew) set_of(t)[lane] = enc(lane == 1 ? p1 : p0);
+      __syncwarp();
+    }
+    pos = lane == 0 ? p0 : (lane == 1 ? p1 : 0u);
+    return t;
   }
 
   // All steps from t on, with n <= 8 anyons in the list, by one warp.  Leaves
@@ -780,23 +1079,18 @@ struct Decoder {
   // snapshot that is renewed at doubling intervals (Brent's cycle search), and
   // the shot stops at the first step whose outcome is the budget's.
   __device__ __forceinline__ void few_steps(int t, int n) {
-    const int L = g.L, tf = t;
-    const bool lit = a.tie_order == QCA_TIE_LITERAL;
-    const bool watch = a.move_thr == 0 && a.balance_rule == QCA_BALANCE_STAY;
-    Ent* snap = few + kFewRing * kFew;
-    int t_snap = -1, t_renew = tf + g.kmax + 1, interval = 64, t_stop = -1;
-    int flag = 0;
-    uint32_t pos = lane < n ? list[lane] : 0;
-    {  // sorted set of the first step
-      int rank = 0;
-      for (int q = 0; q < n; ++q) rank += __shfl_sync(kFull, pos, q) < pos;
-      if (lane < n) few[(t & (kFewRing - 1)) * kFew + rank] = enc(pos);
-      __syncwarp();
-      Ent* row = few + (t & (kFewRing - 1)) * kFew;
-      if (lane >= n && lane < kFew) row[lane] = row[0];
-      __syncwarp();
-      pos = lane < n ? dec(row[lane]) : 0;
-    }
+    constexpr int kWords = kFew * (int)sizeof(Ent) / 4;
+    const int tf = t;
+    uint32_t* const now = reinterpret_cast<uint32_t*>(few);
+    const bool watch = !moves_random() && !balance_random();
+    // the two snapshots' steps (-1: none), when the next ones are due
+    int t_kept = -1, t_moving = -1, due_kept = 0, due_moving = 0, interval = 0;
+    int n_before = 0, t_stop = -1, flag = 0;
+    const int near = (g.L - 1) / 6;  // slices within half the torus
+    int t_pair = 1 << 30;            // first step with two anyons
+    uint32_t pos = lane < n ? list[lane] : 0u;
+    pos = write_set(t, (1u << n) - 1u, pos, n);
+#pragma unroll 1
     while (n) {
       if (t >= a.max_steps || t == t_stop) {
         flag = 2;
@@ -804,83 +1098,125 @@ struct Decoder {
         break;
       }
       if (watch && t_stop < 0) {
-        if (t_snap >= 0 && t > t_snap) {
-          const Ent* now = few + (t & (kFewRing - 1)) * kFew;
-          const Ent* then = snap + (t_snap & (kFewRing - 1)) * kFew;
-          bool same = lane >= kFew || now[lane] == then[lane];
-          if (__all_sync(kFull, same)) {
-            for (int i = lane; i <= g.kmax && same; i += 32) {
-              const Ent* p = few + ((t - i) & (kFewRing - 1)) * kFew;
-              const Ent* q = snap + ((t_snap - i) & (kFewRing - 1)) * kFew;
-#pragma unroll
-              for (int b = 0; b < kFew; ++b) same = same && p[b] == q[b];
-            }
-            if (__all_sync(kFull, same)) {
-              const int P = t - t_snap, R = a.max_steps - t, per = R / P;
-              t_stop = t + (R - per * P) + ((per & 1) ? P : 0);
-              if (t_stop == t) continue;
-            }
-          }
+        if (n != n_before) {
+          // the number of anyons changed: a new orbit, if it is one
+          n_before = n;
+          if (n == 2) t_pair = t;
+          t_kept = t_moving = -1;
+          due_moving = max(t, tf) + g.kmax + 1;
+          due_kept = due_moving + g.kmax + 1;
+          interval = 64;
         }
-        if (t_stop < 0 && t >= t_renew) {
+        const uint32_t e = now[(t & (kFewRing - 1)) * kWords];
+        if (t_kept >= 0 && e == snap[(t_kept & (kFewRing - 1)) * kWords] &&
+            sets_repeat(now, snap, t, t_kept, g.kmax, kWords, lane))
+          t_stop = orbit_stop(t, t - t_kept, a.max_steps);
+        uint32_t* const snap2 = snap + kFewRing * kWords;
+        if (t_stop < 0 && t_moving >= 0 && e == snap2[(t_moving & (kFewRing - 1)) * kWords] &&
+            sets_repeat(now, snap2, t, t_moving, g.kmax, kWords, lane))
+          t_stop = orbit_stop(t, t - t_moving, a.max_steps);
+        if (t_stop >= 0) continue;
+        const bool keep = t_kept < 0 && t >= due_kept;
+        if (keep || t >= due_moving) {
           // (kFewRing entries cover the kmax + 1 <= 85 sets ending at t)
-          for (int i = lane; i < kFewRing * kFew; i += 32) snap[i] = few[i];
-          t_snap = t;
-          t_renew = t + interval;
-          interval <<= 1;
+#pragma unroll 1
+          for (int i = lane; i < kFewRing * kWords; i += 32) {
+            if (keep) snap[i] = now[i];
+            else snap2[i] = now[i];
+          }
+          if (keep) {
+            t_kept = t;
+          } else {
+            t_moving = t;
+            due_moving = t + interval;
+            interval <<= 1;
+          }
           __syncwarp();
         }
       }
-      const Keys key = keys_of(t);
+      if (watch && n == 2 && t > t_pair) {
+        const int t1 = pair_steps(
+            t, t_pair, pos, n, near, t_stop < 0, t_kept, t_moving,
+            min(a.max_steps,
+                t_stop >= 0 ? t_stop : (t_kept < 0 ? min(due_kept, due_moving) : due_moving)));
+        if (t1 != t) {
+          t = t1;
+          continue;
+        }
+      }
       const int last = min(t, g.kmax), lastl = min(last, t - tf);
       // lanes = (anyon, slice)
       const int lgS = n <= 2 ? 4 : (n <= 4 ? 3 : 2), S = 1 << lgS;
       const int ai = lane >> lgS, kk = lane & (S - 1);
       const uint32_t pa = __shfl_sync(kFull, pos, ai);
       const int xa = pa & 0xFFFFu, ya = pa >> 16;
-      uint32_t h0 = 0, h1 = 0;
-      int kf = 0;
-      bool done = ai >= n, edge = false;
-      for (int kb = 0; kb <= lastl; kb += S) {
+      uint32_t hm = 0;  // hits of the first slice with any
+      int kf = 0;       // that slice
+#pragma unroll 1
+      for (int kb = 0; kb <= lastl;) {
+        const bool nr = kb < near;
+        const int lim = nr ? min(lastl, near - 1) : lastl;
         uint32_t m = 0;
-        if (!done && kb + kk <= lastl) m = slice_set(t - kb - kk, xa, ya, kb + kk);
+        if (ai < n && !hm && kb + kk <= lim) m = slice_set(t - kb - kk, xa, ya, kb + kk, nr);
         const uint32_t seg = (__ballot_sync(kFull, m != 0) >> (ai << lgS)) & ((1u << S) - 1u);
-        const int src = (ai << lgS) + (seg ? __ffs(seg) - 1 : 0);
-        const uint32_t hm = __shfl_sync(kFull, m, src);
-        if (!done && seg) {
-          const int d4 = (__ffs(hm) - 1) & ~3;
-          h0 = (hm >> d4) & 15u;
-          h1 = (hm >> (d4 + 4)) & 15u;
-          kf = kb + src - (ai << lgS);
-          edge = d4 == 8 && needs_next(h0, a.tie_order) && kf < last;
-          done = true;
+        const int f = seg ? __ffs(seg) - 1 : 0;
+        const uint32_t mm = __shfl_sync(kFull, m, (ai << lgS) + f);
+        if (!hm && seg) {
+          hm = mm;
+          kf = kb + f;
         }
-        if (__all_sync(kFull, done)) break;
+        if (__all_sync(kFull, ai >= n || hm)) break;
+        kb = min(kb + S, lim + 1);
       }
-      // anyons that hear nothing from the sets: the bitmaps before them
-      uint32_t todo = __ballot_sync(kFull, kk == 0 && ai < n && h0 == 0 && lastl < last);
-      while (todo) {
-        const int src = __ffs(todo) - 1;
-        todo &= todo - 1;
-        int k = lastl + 1;
-        const uint32_t mm = search_far(__shfl_sync(kFull, xa, src), __shfl_sync(kFull, ya, src), t,
-                                       k);
-        if (lane == src && mm) {
-          const int d4 = (__ffs(mm) - 1) & ~3;
-          h0 = (mm >> d4) & 15u;
-          h1 = (mm >> (d4 + 4)) & 15u;
-          kf = k;
-          edge = d4 == 8 && needs_next(h0, a.tie_order) && k < last;
+      // anyons that hear nothing from the sets: the bitmaps before them, two
+      // slices at a time on two lanes of each anyon, the far ones by the warp
+      if (lastl < last) {
+        const int lastt = min(last, min(g.kthread, t - oldest()));
+        int kb = lastl + 1;
+        uint32_t open = __ballot_sync(kFull, ai < n && !hm);
+#pragma unroll 1
+        for (; kb <= lastt && open; kb += 2) {
+          uint32_t m = 0;
+          const int k = kb + kk;
+          if (kk < 2 && k <= lastt && ai < n && !hm)
+            m = slice_thread(slot(t - k), g.lws, g.L, xa, ya, k) & slice_limit(a.m_max, k);
+          const uint32_t m0 = __shfl_sync(kFull, m, ai << lgS);
+          const uint32_t m1 = __shfl_sync(kFull, m, (ai << lgS) + 1);
+          if (!hm && (m0 | m1)) {
+            hm = m0 ? m0 : m1;
+            kf = m0 ? kb : kb + 1;
+          }
+          open = __ballot_sync(kFull, ai < n && !hm);
+        }
+        if (lastt < last) {
+          open = __ballot_sync(kFull, kk == 0 && ai < n && !hm);
+#pragma unroll 1
+          while (open) {
+            const int src = __ffs(open) - 1;
+            open &= open - 1;
+            int k = max(lastl, lastt) + 1;
+            const uint32_t mm =
+                search_far(__shfl_sync(kFull, xa, src), __shfl_sync(kFull, ya, src), t, k);
+            if (lane == src) {
+              hm = mm;
+              kf = k;
+            }
+          }
         }
       }
-      if (lit) {
-        todo = __ballot_sync(kFull, kk == 0 && edge);
+      uint32_t h0 = 0, h1 = 0;
+      if (hm) nearest(hm, h0, h1);
+      if (literal()) {
+        uint32_t todo = __ballot_sync(
+            kFull, kk == 0 && h0 && !(hm & 0xFFu) && !(h0 & 10u) && kf < last);
+#pragma unroll 1
         while (todo) {
           const int src = __ffs(todo) - 1;
           todo &= todo - 1;
+          const int xs = __shfl_sync(kFull, xa, src), ys = __shfl_sync(kFull, ya, src);
+          const int ks = __shfl_sync(kFull, kf, src) + 1;
           const uint32_t mm =
-              slice_any(__shfl_sync(kFull, xa, src), __shfl_sync(kFull, ya, src), t,
-                        __shfl_sync(kFull, kf, src) + 1, tf);
+              t - ks >= tf ? slice_set(t - ks, xs, ys, ks, false) : far_slice(xs, ys, t, ks);
           if (lane == src) h1 = mm & 15u;
         }
       }
@@ -890,53 +1226,39 @@ struct Decoder {
       h0 = __shfl_sync(kFull, h0, (lane << lgS) & 31);
       h1 = __shfl_sync(kFull, h1, (lane << lgS) & 31);
       const int x = pos & 0xFFFFu, y = pos >> 16;
-      int dir = 0;
-      if (lane < n) {
-        dir = drawn_move(key, site(x, y));
-        if (!dir && h0) dir = resolve(direction(h0, h1, a.tie_order), key, site(x, y));
-      }
+      const Keys key = keys_of(t);
+      const int dir = lane < n ? move_of(key, x, y, h0, h1) : 0;
       uint32_t np = pos, bit = 0;
       int lw = 0;
       if (dir) {
         lw = link_of(x, y, dir, bit);
-        const int nx = dir == 1 ? wrap_hi(x + 1, L) : (dir == 2 ? wrap_lo(x - 1, L) : x);
-        const int ny = dir == 3 ? wrap_hi(y + 1, L) : (dir == 4 ? wrap_lo(y - 1, L) : y);
-        np = ((uint32_t)ny << 16) | nx;
+        np = site_after(x, y, dir);
       }
-      // a link crossed from both ends flips once and takes both anyons;
-      // otherwise the anyons are where an odd number of them end
-      int crossed = 0, first_cross = 1;
+      // a link crossed from both ends (the two anyons swap sites) flips once and
+      // takes both; otherwise the anyons are where an odd number of them end
+      bool swap = false, first = true;
+#pragma unroll 1
       for (int q = 0; q < n; ++q) {
-        const uint32_t bq = __shfl_sync(kFull, bit, q);
-        const int wq = __shfl_sync(kFull, lw, q);
-        const bool eq = dir && bq == bit && wq == lw;
-        crossed += eq;
-        if (eq && q < lane) first_cross = 0;
+        const uint32_t to = __shfl_sync(kFull, np, q), from = __shfl_sync(kFull, pos, q);
+        if (dir && to == pos && from == np) {
+          swap = true;
+          first = q > lane;
+        }
       }
-      if (dir && first_cross) atomicXor(&C[lw], bit);
-      const bool stays = lane < n && crossed < 2;
+      if (dir && first) atomicXor(&C[lw], bit);
+      const bool stays = lane < n && !swap;
       if (!stays) np = 0x80000000u | lane;
       int same = 0, lower = 0;
+#pragma unroll 1
       for (int q = 0; q < n; ++q) {
         const uint32_t v = __shfl_sync(kFull, np, q);
         same += v == np;
         lower += v == np && q < lane;
       }
-      const bool alive = stays && (same & 1) && lower == 0;
-      const uint32_t am = __ballot_sync(kFull, alive);
-      int rank = 0;
-      for (int q = 0; q < n; ++q) {
-        const uint32_t v = __shfl_sync(kFull, np, q);
-        rank += ((am >> q) & 1u) && v < np;
-      }
+      const uint32_t am = __ballot_sync(kFull, stays && (same & 1) && lower == 0);
       ++t;
+      pos = write_set(t, am, np, n);
       n = __popc(am);
-      Ent* row = few + (t & (kFewRing - 1)) * kFew;
-      if (alive) row[rank] = enc(np);
-      __syncwarp();
-      if (lane >= n && lane < kFew) row[lane] = row[0];
-      __syncwarp();
-      pos = lane < n ? dec(row[lane]) : 0;
     }
     if (lane == 0) {
       misc[4] = t;
@@ -945,14 +1267,46 @@ struct Decoder {
   }
 
   // ------------------------------------------------------------ one shot
+  __device__ __forceinline__ void zero(uint32_t* p, int words) const {
+#pragma unroll 2
+    for (int w = tid; w < words; w += NT) p[w] = 0;
+  }
+  __device__ __forceinline__ void load(const uint8_t* src, int rows, uint32_t* dst, bool any) {
+    const int L = g.L;
+    if ((L & 15) == 0 && (reinterpret_cast<uintptr_t>(src) & 15) == 0) {
+      if (L & 31) {
+        zero(dst, rows << g.lws);
+        sync();
+      }
+      load_rows<NT>(src, rows, L, g.lws, dst, any, tid);
+    } else {
+      zero(dst, rows << g.lws);
+      sync();
+      load_flat(src, rows, L, g.lws, dst, any, tid, NT);
+    }
+  }
+
   __device__ __forceinline__ void run() {
     const int L = g.L, LL = L * L, lws = g.lws;
     const int lastw = (L - 1) >> 5, lastb = (L - 1) & 31;
     const uint8_t* N = a.in + shot_offset_of(a, shot);
     uint8_t* outC = a.out_C + correction_offset_of(a, shot);
-    spill = reinterpret_cast<uint32_t*>(
-        (reinterpret_cast<uintptr_t>(outC) + 3) & ~(uintptr_t)3);
-    nspill = min(g.spill, (2 * LL - (int)(reinterpret_cast<uint8_t*>(spill) - outC)) / (4 * g.nws));
+    if (!LARGE) {
+      uint8_t* room = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(outC) + 3) &
+                                                 ~(uintptr_t)3);
+      if (g.c_global) {
+        C = reinterpret_cast<uint32_t*>(room);
+        F = C + 2 * g.nws;
+        room += 16 * g.nws;
+      }
+      const int bytes = 2 * LL - (int)(room - outC), bm = 4 * g.nws;
+      ar.cap = bytes / (4 * kArchiveSets);
+      if (ar.cap < 2 * kFew) ar.cap = 0;
+      ar.nb = (bytes - 2 * kArchiveSets * ar.cap) / bm;
+      ar.bitmaps = reinterpret_cast<uint32_t*>(room);
+      ar.sets = reinterpret_cast<uint16_t*>(room + ar.nb * bm);
+      ar.gone = ar.next = 0;
+    }
     if (tid < 8) misc[tid] = 0;
     ph = 0;
     tb = 0;
@@ -960,30 +1314,28 @@ struct Decoder {
     int wx = 0, wy = 0, n = 0;
     uint32_t* s0 = slot(0);
     if (a.from_sigma) {
-      for (int w = tid; w < g.nws; w += NT) s0[w] = 0;
-      sync();
-      load_bits<NT, true>(N, L, L, lws, s0, tid);
-      for (int w = tid; w < 2 * g.nws; w += NT) C[w] = 0;
-      for (int w = tid; w < 2 * g.nws; w += NT) F[w] = 0;
-      sync();
-      for (int w = tid; w < g.nws; w += NT) n += __popc(s0[w]);
-    } else {
-      // the link bits, in the correction's place
-      if (L & 31) {
-        for (int w = tid; w < 2 * g.nws; w += NT) C[w] = 0;
+      if (lastw < (1 << lws) - 1) {
+        zero(s0, g.nws);  // the padding words, which no row of bytes covers
         sync();
       }
-      load_bits<NT, false>(N, 2 * L, L, lws, C, tid);
-      for (int w = tid; w < 2 * g.nws; w += NT) F[w] = 0;
+      load(N, L, s0, true);
+      sync();
+#pragma unroll 1
+      for (int w = tid; w < g.nws; w += NT) n += __popc(s0[w]);
+    } else {
+      // the link bits, in slots not yet in use
+      uint32_t* B = LARGE ? C : ring + 2 * g.nslot;
+      load(N, 2 * L, B, false);
       sync();
       const int wsm = (1 << lws) - 1;
+#pragma unroll 2
       for (int w = tid; w < g.nws; w += NT) {
         const int y = w >> lws, j = w & wsm;
         uint32_t s = 0;
         if (j <= lastw) {
           const int yu = y == 0 ? L - 1 : y - 1;
-          const uint32_t bx = C[w], by = C[g.nws + w], bu = C[g.nws + (yu << lws) + j];
-          const uint32_t carry = j ? C[w - 1] >> 31 : (C[(y << lws) + lastw] >> lastb) & 1u;
+          const uint32_t bx = B[w], by = B[g.nws + w], bu = B[g.nws + (yu << lws) + j];
+          const uint32_t carry = j ? B[w - 1] >> 31 : (B[(y << lws) + lastw] >> lastb) & 1u;
           s = (bx ^ ((bx << 1) | carry) ^ by ^ bu) &
               (j == lastw ? kFull >> (31 - lastb) : kFull);
           if (j == 0) wx ^= (int)(bx & 1u);
@@ -992,16 +1344,29 @@ struct Decoder {
         s0[w] = s;
         n += __popc(s);
       }
-      sync();
-      for (int w = tid; w < 2 * g.nws; w += NT) C[w] = 0;
     }
     n = total(n);
+    if (!LARGE && tid < 4 * (g.kmask + 1) && g.nws + (tid & 3) < g.nslot)
+      ring[(tid >> 2) * g.nslot + g.nws + (tid & 3)] = 0;  // the slots' last words
     int t = 0, flag = 0;
-    if (n) advance(0, n <= g.sparse_max);
-    // ---- steps
+    bool listed = n <= g.sparse_max;
+    if (listed || a.max_steps == 0) {  // else the first dense step writes it
+      zero(C, 2 * g.nws);
+      if (listed) zero(table, g.tmask + 1);
+      sync();
+    }
+    // ---- steps.  With the deterministic rules a shot whose anyons have not
+    // moved for kmax + 1 steps never moves again.
+    const bool watch = !moves_random() && !balance_random();
+    int still = 0;
+#pragma unroll 1
     while (n) {
-      if (t >= a.max_steps) {
+      const int nl = advance(t, listed);
+      if (listed) n = nl;
+      if (n == 0) break;
+      if (t >= a.max_steps || still > g.kmax) {
         flag = 2;
+        t = a.max_steps;
         break;
       }
       if (n <= kFew) {
@@ -1012,26 +1377,39 @@ struct Decoder {
         flag = misc[5];
         break;
       }
-      int mark[4];
-      if (n <= g.sparse_max) {
-        move_listed<true>(n, t, mark);
-        sync();
-        if (!LARGE && misc[3]) break;
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-          if (mark[q] >= 0) F[mark[q]] = 0;
-        n = advance(t + 1, true);
-      } else {
-        const int nl = mark_dense(t);
-        if (nl) {
-          move_listed<false>(nl, t, mark);
+      Strip p;
+      int mine = 0, pos = 0, todo = n, r0 = 0;
+      if (!listed) {
+        p = strip();
+        mine = mark_dense(t, p);
+        pos = places(mine);
+        todo = next_counter();
+      }
+      bool moved = false;
+#pragma unroll 1
+      for (; r0 < todo; r0 += g.list_cap) {
+        if (!listed) {
+          list_open(t, p, mine, pos, r0);
           sync();
         }
-        if (!LARGE && misc[3]) break;
-        n = apply_dense(t);
-        for (int w = tid; w < 2 * g.nws; w += NT) F[w] = 0;
-        if (n) advance(t + 1, n <= g.sparse_max);
+        moved = sync_or(move_listed(min(todo - r0, g.list_cap), t, listed));
       }
+      if (!LARGE && misc[3]) break;
+      if (listed) {
+        if ((t & kEpochs) == kEpochs) {
+          zero(table, g.tmask + 1);
+          sync();
+        }
+      } else {
+        moved = false;
+        const int left = apply_dense(t, p, moved);
+        if (left == n) moved = sync_or(moved);
+        else moved = true;
+        n = left;
+        listed = n <= g.sparse_max;
+        if (listed) zero(table, g.tmask + 1);
+      }
+      still = watch && !moved ? still + 1 : 0;
       ++t;
     }
     if (!LARGE && misc[3]) {
@@ -1041,7 +1419,16 @@ struct Decoder {
       return;
     }
     // ---- correction, homology, steps, flag
+    if (!LARGE && g.c_global) {
+      // the bytes will take the place of the correction's words
+#pragma unroll 2
+      for (int w = tid; w < 2 * g.nws; w += NT) ring[w] = __ldcg(C + w);
+      C = ring;
+      sync();
+    }
+#pragma unroll 1
     for (int y = tid; y < L; y += NT) wx ^= (int)(C[y << lws] & 1u);
+#pragma unroll 1
     for (int j = tid; j <= lastw; j += NT) wy ^= __popc(C[g.nws + j]) & 1;
     wx = __reduce_xor_sync(kFull, wx);
     wy = __reduce_xor_sync(kFull, wy);
@@ -1052,7 +1439,10 @@ struct Decoder {
       wx = misc[6];
       wy = misc[7];
     }
-    store_bits<NT>(outC, 2 * L, L, lws, C, tid);
+    if ((L & 15) == 0 && (reinterpret_cast<uintptr_t>(outC) & 15) == 0)
+      store_rows<NT>(outC, 2 * L, L, lws, C, tid);
+    else
+      store_flat(outC, 2 * L, L, lws, C, tid, NT);
     if (tid == 0) {
       a.out_steps[shot] = t;
       if (a.from_sigma) {

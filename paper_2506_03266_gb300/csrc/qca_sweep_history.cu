@@ -1,15 +1,21 @@
 // Host side and kernels of the history sweep (qca_history.cuh).
 //
-// Up to L = 256 everything a shot needs is in one CTA's shared memory: the last
-// 4 to 8 syndrome bitmaps, the correction, the flipped-link maps and the anyon
-// list; older syndromes go to the shot's own correction block, which is not
-// written before the shot ends (16 bitmaps of L^2 / 8 bytes fit its 2 L^2).  A
-// shot that needs a still older one (all anyons of a region far apart while
-// others elsewhere linger) is
-// left pending, and the sweep with message planes decodes it in a second
-// launch, which otherwise only looks for pending shots.  Above L = 256 the
-// bitmaps live in a slot of a cached workspace that holds all 85 syndromes a
-// message can come from.
+// Up to L = 256 the last 4 to 8 syndrome bitmaps and the anyon list are in the
+// shared memory of the shot's CTA; older syndromes go to the shot's own
+// correction block, which is not written before the shot ends, as bitmaps while
+// the anyons are many and as lists of sites afterwards, so that every shot of
+// random noise keeps all 85 syndromes a message can come from.  A shot that has
+// too many large old ones (a syndrome with a part that stays dense for dozens of
+// steps and a part that is sparse) is left pending, and the sweep with message
+// planes decodes it in a second launch, which otherwise only looks for pending
+// shots.  Above L = 256 the bitmaps live in a slot of a cached workspace that
+// holds all 85.
+//
+// What bounds it: instruction issue at 20 to 24 warps per SM (2 of 4 slots used,
+// L = 256), about 160 thousand warp instructions per shot, half of them the
+// anyon searches; instruction fetch for the small sizes, whose warps are all at
+// different places of the code.  L = 256, p = 0.05, 20 000 shots: 4.8 ms, against
+// 55 ms for the sweep over message planes; floor by bytes 0.77 ms.
 #include <algorithm>
 #include <atomic>
 #include <mutex>
@@ -22,20 +28,23 @@ namespace {
 
 using namespace hist;
 
-template <int NT, bool LARGE>
+template <int NT, bool LARGE, bool PLAIN>
 __global__ void __launch_bounds__(NT, NT == 32 ? 24 : (NT == 1024 ? 1 : 768 / NT))
     history_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ Geom g,
                    uint32_t* ws, size_t slot_words) {
   extern __shared__ __align__(16) uint32_t sm[];
   uint32_t* base = LARGE ? ws + (size_t)blockIdx.x * slot_words : sm;
   for (int64_t k = blockIdx.x; k < a.shots; k += gridDim.x) {
-    Decoder<NT, LARGE> d{a, g};
+    Decoder<NT, LARGE, PLAIN> d{a, g};
     d.ring = base;
     d.C = base + g.o_C;
     d.F = base + g.o_F;
     d.list = sm + g.o_list;
-    d.few = reinterpret_cast<typename Decoder<NT, LARGE>::Ent*>(sm + g.o_few);
+    d.table = sm + g.o_table;
+    d.snap = sm + g.o_snap;
+    d.few = reinterpret_cast<typename Decoder<NT, LARGE, PLAIN>::Ent*>(sm + g.o_few);
     d.misc = reinterpret_cast<int*>(sm + g.o_misc);
+    d.nset = reinterpret_cast<uint16_t*>(sm + g.o_misc + 8);
     d.shot = a.shot_list ? (int64_t)a.shot_list[k] : k;
     d.tid = threadIdx.x;
     d.lane = threadIdx.x & 31;
@@ -45,9 +54,13 @@ __global__ void __launch_bounds__(NT, NT == 32 ? 24 : (NT == 1024 ? 1 : 768 / NT
   }
 }
 
-// Threads per shot: a warp up to L = 64 (no block barriers), then about eight
-// bitmap words per thread.
-int threads_for(int L) { return L <= 64 ? 32 : (L <= 128 ? 128 : (L <= 256 ? 256 : 1024)); }
+// Threads per shot: a warp up to L = 64 (no block barriers).  Above, four warps:
+// the steps with few anyons leave most of a larger CTA idle, so more and smaller
+// CTAs per SM are better (L = 256: 256 threads 5.4 ms per 20 000 shots at three
+// CTAs per SM, 128 threads at the same three 6.3 ms, at six 4.8 ms).  What lets
+// six fit at L = 256 is keeping the correction and the dense steps' link maps in
+// the shot's (L2-resident) correction block instead of shared memory.
+int threads_for(int L) { return L <= 64 ? 32 : (L <= 256 ? 128 : 1024); }
 
 bool make_hist_geom(int L, int m_max, Geom& g, int& threads, size_t& smem, size_t& slot_words) {
   if (L < 8 || L > QCA_MAX_L) return false;
@@ -58,32 +71,52 @@ bool make_hist_geom(int L, int m_max, Geom& g, int& threads, size_t& smem, size_
   g.lws = 0;
   while ((1 << g.lws) < wpr) ++g.lws;
   g.nws = L << g.lws;
+  g.nslot = (g.nws + 3) & ~3;
   g.kmax = (m_max - 1) / 3;
+  g.kthread = std::min(4, (L - 7) / 6);
   const int K = L <= 128 ? 8 : 4;
   g.kmask = K - 1;
-  g.spill = g.kmax > K - 2 ? 16 : 0;
-  // the dense pass costs about as much as searching half an anyon per word
-  g.sparse_max = std::max(kFew, std::min(4 * threads, g.nws / 2));
-  g.list_cap = std::max(g.nws / 2, g.sparse_max) + 64;
-  if (large) g.list_cap = std::min(g.list_cap, 8192);
+  g.spill = g.kmax > K - 2;
+  g.c_global = !large && L > 128;
+  // a dense pass costs about as much as searching half an anyon per word (L = 32,
+  // p = 0.06: 0.80 ms per 20 000 shots, 0.87 at a quarter); above L = 128 the
+  // smaller list and crossing table let one more CTA fit (L = 256: 4.8 against
+  // 5.8 ms)
+  g.sparse_max = std::max(kFew, L <= 128 ? g.nws / 2 : g.nws / 4);
+  if (large) g.sparse_max = std::min(g.sparse_max, 4096);
+  g.list_cap = g.sparse_max;
+  int tsize = 1;
+  while (tsize < g.sparse_max) tsize *= 2;
+  g.tmask = tsize - 1;
   const int few = large ? kFewWords<true> : kFewWords<false>;
+  // the crossing table and the few-anyon mode's sets are never in use at once
+  int o = 0, region = std::max(few, tsize);
   if (large) {
     g.o_C = kLargeRing * g.nws;
     g.o_F = g.o_C + 2 * g.nws;
     slot_words = (size_t)g.o_F + 2 * g.nws;
-    g.o_few = 0;
-    g.o_list = few;
-    g.o_misc = g.o_list + g.list_cap;
   } else {
-    // the few-anyon mode's sets take the link maps' place
-    g.o_C = K * g.nws;
-    g.o_F = (g.o_C + 2 * g.nws + 3) & ~3;
-    g.o_few = g.o_F;
-    g.o_list = g.o_F + std::max(2 * g.nws, few);
-    g.o_misc = g.o_list + g.list_cap;
+    o = K * g.nslot;
+    g.o_C = g.o_F = 0;
+    if (!g.c_global) {
+      g.o_C = o;
+      o = (o + 2 * g.nws + 3) & ~3;
+    }
     slot_words = 0;
   }
-  smem = (size_t)(g.o_misc + 8) * 4;
+  g.o_table = g.o_few = o;
+  o += (region + 3) & ~3;
+  // the snapshots are taken when the bitmaps are no longer needed
+  if (!large && K * g.nslot >= 2 * few) {
+    g.o_snap = 0;
+  } else {
+    g.o_snap = o;
+    o += 2 * few;
+  }
+  g.o_list = o;
+  o += g.list_cap;
+  g.o_misc = o;
+  smem = (size_t)(o + 8 + 64) * 4;  // counters, archived set sizes
   return true;
 }
 
@@ -106,10 +139,15 @@ struct HistWorkspace {
 std::mutex g_hws_mu;
 HistWorkspace g_hws[64];
 
-template <int NT>
+// The default rules have a kernel of their own.
+bool plain_rules(const DecodeArgs& a) {
+  return a.move_thr == 0 && a.tie_order == QCA_TIE_LEX && a.balance_rule == QCA_BALANCE_STAY;
+}
+
+template <int NT, bool PLAIN>
 int launch_small(const DecodeArgs& a, const Geom& g, size_t smem, int dev, cudaStream_t stream) {
   static std::atomic<int> have[64];
-  auto kern = history_kernel<NT, false>;
+  auto kern = history_kernel<NT, false, PLAIN>;
   if (int rc = allow_smem(kern, smem, have, dev)) return rc;
   // a CTA per shot: the hardware hands out shots as CTAs retire
   const int64_t grid = std::min<int64_t>(a.shots, 1 << 30);
@@ -117,11 +155,12 @@ int launch_small(const DecodeArgs& a, const Geom& g, size_t smem, int dev, cudaS
   return cuda_fail(cudaGetLastError(), "history sweep launch");
 }
 
+template <bool PLAIN>
 int launch_large(const DecodeArgs& a, const Geom& g, size_t smem, size_t slot_words, int dev,
                  cudaStream_t stream) {
   constexpr int NT = 1024;
   static std::atomic<int> have[64];
-  auto kern = history_kernel<NT, true>;
+  auto kern = history_kernel<NT, true, PLAIN>;
   if (int rc = allow_smem(kern, smem, have, dev)) return rc;
   int sms = 0, per_sm = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -181,11 +220,17 @@ int launch_history(const DecodeArgs& a, cudaStream_t stream) {
     set_error("device index %d out of range", dev);
     return QCA_ERR_UNSUPPORTED;
   }
+  const bool plain = plain_rules(a);
   switch (threads) {
-    case 32: return launch_small<32>(a, g, smem, dev, stream);
-    case 128: return launch_small<128>(a, g, smem, dev, stream);
-    case 256: return launch_small<256>(a, g, smem, dev, stream);
-    default: return launch_large(a, g, smem, slot_words, dev, stream);
+    case 32:
+      return plain ? launch_small<32, true>(a, g, smem, dev, stream)
+                   : launch_small<32, false>(a, g, smem, dev, stream);
+    case 128:
+      return plain ? launch_small<128, true>(a, g, smem, dev, stream)
+                   : launch_small<128, false>(a, g, smem, dev, stream);
+    default:
+      return plain ? launch_large<true>(a, g, smem, slot_words, dev, stream)
+                   : launch_large<false>(a, g, smem, slot_words, dev, stream);
   }
 }
 
