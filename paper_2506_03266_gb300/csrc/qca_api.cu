@@ -102,9 +102,7 @@ int decode_path(int L, int v, int m_max) {
   return fast_path_for(L, v, m_max);
 }
 
-// The sweeps that keep the message fields: the on-chip, large-lattice or
-// generic one.
-static int launch_planes(const DecodeArgs& a, cudaStream_t stream) {
+int launch_planes(const DecodeArgs& a, cudaStream_t stream) {
   int path = decode_path(a.L, a.v, a.m_max);
   // The on-chip and large-lattice kernels read the input and write the
   // correction as 32-bit words.  A caller array or shot block off a 4-byte

@@ -87,11 +87,30 @@ __device__ __forceinline__ uint32_t row_bits_wrapped(const uint32_t* row, int wp
   return n >= 32 ? v : v & ((1u << n) - 1u);
 }
 
-// Any anyon within `reach` columns of x in a bitmap row.
+// The same without wrap: columns below 0 or from L on are 0 (0 - n < c < L).
+__device__ __forceinline__ uint32_t row_bits_clipped(const uint32_t* row, int wpr, int L, int c,
+                                                     int n) {
+  const int s = max(c, 0), w = s >> 5;
+  uint32_t v = 0;
+  if (s < L) {
+    v = __funnelshift_r(row[w], w + 1 < wpr ? row[w + 1] : 0u, s & 31);
+    if (c < 0) v <<= -c;
+  }
+  return n >= 32 ? v : v & ((1u << n) - 1u);
+}
+
+// Any anyon within `reach` columns of x in a bitmap row; OPEN: a row that does
+// not wrap.
+template <bool OPEN>
 __device__ __forceinline__ uint32_t row_any(const uint32_t* row, int wpr, int L, int x,
                                             int reach) {
   uint32_t any = 0;
-  if (2 * reach + 1 >= L) {
+  if (OPEN) {
+    const int hi = min(x + reach, L - 1);
+#pragma unroll 1
+    for (int c = max(x - reach, 0); c <= hi; c += 32)
+      any |= row_bits_clipped(row, wpr, L, c, min(32, hi - c + 1));
+  } else if (2 * reach + 1 >= L) {
 #pragma unroll 1
     for (int w = 0; w < wpr; ++w) any |= row[w];
   } else {
@@ -115,24 +134,33 @@ __device__ __forceinline__ uint32_t slice_limit(int m_max, int k) {
 
 // Slice k of the anyon at (x, y) by one thread, from the bitmap of sigma_{t-k}:
 // the (6k + 7) x (6k + 7) neighbourhood, a row window per row; needs 6k + 7 <=
-// 31 and <= L.
+// 31 and <= L.  OPEN: rows and columns outside the lattice are empty.
+template <bool OPEN>
 __device__ __forceinline__ uint32_t slice_thread(const uint32_t* sig, int lws, int L, int x, int y,
                                                  int k) {
   const int wpr = 1 << lws;
   const int r = 3 * k + 3, n = 2 * r + 1;
-  const int s = wrap_lo(x - r, L);
+  const int s = OPEN ? max(x - r, 0) : wrap_lo(x - r, L);
   const int w0 = s >> 5, sh = s & 31;
   const int w1 = min(w0 + 1, wpr - 1);
   const int sl = w0 < wpr - 1 ? 32 - sh : 32;  // 1 .. 32
-  const int n0 = s + n > L ? L - s : 0;        // columns before the wrap, if any
+  // columns before the wrap, if any; OPEN: columns left of the lattice
+  const int n0 = OPEN ? s - (x - r) : (s + n > L ? L - s : 0);
   const uint32_t mask = (1u << n) - 1u;
-  int yy = wrap_lo(y - r, L);
+  int yy = OPEN ? y - r : wrap_lo(y - r, L);
   auto next = [&]() {  // bit i: column x - r + i of the next row
+    if (OPEN && (unsigned)yy >= (unsigned)L) {
+      ++yy;
+      return 0u;
+    }
     const uint32_t* row = sig + (yy << lws);
     uint32_t v = (row[w0] >> sh) | __funnelshift_lc(0u, row[w1], sl);
-    if (n0) v |= row[0] << n0;  // the bits past column L - 1 are 0
+    if (OPEN)
+      v <<= n0;
+    else if (n0)
+      v |= row[0] << n0;  // the bits past column L - 1 are 0
     ++yy;
-    if (yy == L) yy = 0;
+    if (!OPEN && yy == L) yy = 0;
     return v & mask;
   };
   // rows y - r .. y + r; the distances' cone sections across the rows are
@@ -162,21 +190,26 @@ __device__ __forceinline__ uint32_t slice_thread(const uint32_t* sig, int lws, i
 // fields (three columns on either side), six lanes for the y fields' rows.  For
 // the far slices, which few anyons reach: a function of its own, since the
 // kernel is bound by instruction fetch when every use is a copy.
+template <bool OPEN>
 static __device__ __noinline__ uint32_t slice_warp(const uint32_t* sig, int lws, int L, int x, int y,
                                                int k, int lane) {
   const int wpr = 1 << lws;
   const int r = 3 * k + 3;
-  const int nrows = min(2 * r + 1, L);
-  const int half = nrows == L ? (L - 1) >> 1 : r;
-  const int cl = wrap_lo(x - r % L, L);              // columns x - 3k - 3 ..
-  const int cr = wrap_hi(x + (3 * k + 1) % L, L);    // columns x + 3k + 1 ..
+  const int nrows = OPEN ? 2 * r + 1 : min(2 * r + 1, L);
+  const int half = nrows == 2 * r + 1 ? r : (L - 1) >> 1;
+  const int cl = OPEN ? x - r : wrap_lo(x - r % L, L);                  // columns x - 3k - 3 ..
+  const int cr = OPEN ? x + r - 2 : wrap_hi(x + (3 * k + 1) % L, L);    // columns x + 3k + 1 ..
   uint32_t m = 0;
 #pragma unroll 1
   for (int i = lane; i < nrows; i += 32) {
     const int j = i - half;
+    if (OPEN && (unsigned)(y + j) >= (unsigned)L) continue;
     const uint32_t* row = sig + (wrap_hi(wrap_lo(y + j, L), L) << lws);
-    const uint32_t l = row_bits_wrapped(row, wpr, L, cl, 3);  // d = 3, 2, 1
-    const uint32_t q = row_bits_wrapped(row, wpr, L, cr, 3);  // d = 1, 2, 3
+    // d = 3, 2, 1 and d = 1, 2, 3
+    const uint32_t l = OPEN ? (cl > -3 ? row_bits_clipped(row, wpr, L, cl, 3) : 0u)
+                            : row_bits_wrapped(row, wpr, L, cl, 3);
+    const uint32_t q = OPEN ? row_bits_clipped(row, wpr, L, cr, 3)
+                            : row_bits_wrapped(row, wpr, L, cr, 3);
     uint32_t h = ((l >> 2) & 1u) | ((q << 1) & 2u) | ((l << 3) & 0x10u) | ((q << 4) & 0x20u) |
                  ((l << 8) & 0x100u) | ((q << 7) & 0x200u);
     const int aj = (j < 0 ? -j : j) - 3 * k;  // |j| <= 3k + d
@@ -185,23 +218,28 @@ static __device__ __noinline__ uint32_t slice_warp(const uint32_t* sig, int lws,
   }
   if (lane < 6) {
     const int d = lane < 3 ? lane + 1 : lane - 2;
-    const int reach = 3 * k + d, dr = reach % L;
-    const int yy = lane < 3 ? wrap_lo(y - dr, L) : wrap_hi(y + dr, L);
-    m |= row_any(sig + (yy << lws), wpr, L, x, reach) << (4 * (d - 1) + (lane < 3 ? 2 : 3));
+    const int reach = 3 * k + d, dr = OPEN ? reach : reach % L;
+    int yy = lane < 3 ? y - dr : y + dr;
+    if (!OPEN) yy = wrap_hi(wrap_lo(yy, L), L);
+    if (!OPEN || (unsigned)yy < (unsigned)L)
+      m |= row_any<OPEN>(sig + (yy << lws), wpr, L, x, reach) << (4 * (d - 1) + (lane < 3 ? 2 : 3));
   }
   return __reduce_or_sync(kFull, m);
 }
 
 // Slice k of the anyon at (xa, ya) against one anyon (xb, yb) of sigma_{t-k}, for
-// slices within half the torus (3k + 3 <= (L - 1) / 2): the larger of the two
-// coordinate distances decides.
+// slices within half the torus (3k + 3 <= (L - 1) / 2; OPEN: any slice): the
+// larger of the two coordinate distances decides.
+template <bool OPEN>
 __device__ __forceinline__ uint32_t slice_near(int xa, int ya, int xb, int yb, int L, int k) {
   const int half = L >> 1;
   int sx = xa - xb, sy = ya - yb;
-  if (sx > half) sx -= L;
-  if (sx < -half) sx += L;
-  if (sy > half) sy -= L;
-  if (sy < -half) sy += L;
+  if (!OPEN) {
+    if (sx > half) sx -= L;
+    if (sx < -half) sx += L;
+    if (sy > half) sy -= L;
+    if (sy < -half) sy += L;
+  }
   const int ax = abs(sx), ay = abs(sy), d = max(ax, ay), e = d - 3 * k - 1;
   if ((unsigned)e >= 3u) return 0;
   return ((ax == d ? (sx > 0 ? 1u : 2u) : 0u) | (ay == d ? (sy > 0 ? 4u : 8u) : 0u)) << (4 * e);
@@ -225,6 +263,7 @@ __device__ __forceinline__ uint32_t slice_pair(int xa, int ya, int xb, int yb, i
 }
 
 // The same against all n anyons of an archived set, by a whole warp.
+template <bool OPEN>
 static __device__ __noinline__ uint32_t slice_list(const uint16_t* set, int n, int L, int x, int y,
                                                    int k, int lane) {
   const int c = (3 * k + 1) % L;
@@ -232,7 +271,8 @@ static __device__ __noinline__ uint32_t slice_list(const uint16_t* set, int n, i
 #pragma unroll 1
   for (int i = lane; i < n; i += 32) {
     const uint32_t e = set[i];
-    m |= slice_pair(x, y, (int)(e & 0xFFu), (int)(e >> 8), L, k, c);
+    m |= OPEN ? slice_near<true>(x, y, (int)(e & 0xFFu), (int)(e >> 8), L, k)
+              : slice_pair(x, y, (int)(e & 0xFFu), (int)(e >> 8), L, k, c);
   }
   return __reduce_or_sync(kFull, m);
 }
@@ -425,7 +465,12 @@ static __device__ __noinline__ int orbit_stop(int t, int P, int max_steps) {
 
 // PLAIN: lexicographic ties, a balanced axis stays, no random moves (the
 // default rules); the other forms read the rules from the arguments.
-template <int NT, bool LARGE, bool PLAIN>
+// OPEN (with PLAIN only): the lattice with open boundaries (Def. "message passing
+// automaton with open boundaries"): no wrap; the columns x = 0 and x = L - 1 hold
+// no anyons and no messages, send m^{+x} and m^{-x} into the bulk in every
+// sub-step and absorb anyons; only the links between bulk sites and those to the
+// two columns exist.
+template <int NT, bool LARGE, bool PLAIN, bool OPEN = false>
 struct Decoder {
   using Ent = typename std::conditional<LARGE, uint32_t, uint16_t>::type;
   // crossing table: bits of a link (word of the link maps and bit), steps it
@@ -592,6 +637,17 @@ struct Decoder {
 
   __device__ __forceinline__ uint32_t site(int x, int y) const { return (uint32_t)(y * g.L + x); }
 
+  // OPEN: hits of slice k from the two rough columns.
+  __device__ __forceinline__ uint32_t edges(int x, int k) const {
+    if (!OPEN) return 0u;
+    const int l = x - 3 * k - 1, r = g.L - 2 - x - 3 * k;
+    return ((unsigned)l < 3u ? 1u << (4 * l) : 0u) | ((unsigned)r < 3u ? 2u << (4 * r) : 0u);
+  }
+  // OPEN: whether column x can hold anyons.
+  __device__ __forceinline__ bool bulk(int x) const {
+    return !OPEN || (x > 0 && x < g.L - 1);
+  }
+
   // One slice of the anyon at (x, y) by the whole warp, wherever the syndrome is.
   __device__ __forceinline__ uint32_t far_slice(int x, int y, int t, int k) const {
     const int s = t - k;
@@ -600,14 +656,14 @@ struct Decoder {
     if (LARGE || s >= oldest()) {
       sig = slot(s);
     } else if (nset[s & 127] != kNoSet) {
-      m = slice_list(ar.sets + (s % kArchiveSets) * ar.cap, nset[s & 127], g.L, x, y, k, lane);
+      m = slice_list<OPEN>(ar.sets + (s % kArchiveSets) * ar.cap, nset[s & 127], g.L, x, y, k, lane);
     } else if (s >= ar.gone - ar.nb) {
       sig = ar.bitmaps + (s % ar.nb) * g.nws;
     } else {
       misc[3] = 1;  // the shot needs a syndrome that is no longer kept
     }
-    if (sig) m = slice_warp(sig, g.lws, g.L, x, y, k, lane);
-    return m & slice_limit(a.m_max, k);
+    if (sig) m = slice_warp<OPEN>(sig, g.lws, g.L, x, y, k, lane);
+    return (m | edges(x, k)) & slice_limit(a.m_max, k);
   }
   // Slices from k on by the whole warp; returns the first slice's hits (0:
   // nothing heard) and its index in k.
@@ -705,7 +761,8 @@ struct Decoder {
         y = e >> 16;
 #pragma unroll 1
         for (;; ++k) {
-          m = slice_thread(slot(t - k), g.lws, g.L, x, y, k) & slice_limit(a.m_max, k);
+          m = slice_thread<OPEN>(slot(t - k), g.lws, g.L, x, y, k) | edges(x, k);
+          m &= slice_limit(a.m_max, k);
           if (m || k >= lastt) break;
         }
       }
@@ -752,7 +809,7 @@ struct Decoder {
               first_crossing((uint32_t)w << 5 | (__ffs(bit) - 1), t)) {
             atomicXor(&C[w], bit);
             atomicXor(&sn[(y << g.lws) + (x >> 5)], 1u << (x & 31));
-            atomicXor(&sn[wn], 1u << (nx & 31));
+            if (bulk(nx)) atomicXor(&sn[wn], 1u << (nx & 31));
           }
         }
       }
@@ -768,7 +825,8 @@ struct Decoder {
     int jl, jr;         // lanes of the words to the left and to the right
     int sl, top;        // bit of the left word that is column x - 1 of this word's first
                         // column, bit of this word that is its last column
-    uint32_t valid;     // this word's columns
+    uint32_t valid;     // this word's columns that can hold anyons
+    bool on;            // not a padding word
     int y0, y1;         // rows
   };
   __device__ __forceinline__ Strip strip() const {
@@ -782,6 +840,9 @@ struct Decoder {
     p.sl = p.j == 0 ? lastb : 31;
     p.top = p.j == lastw ? lastb : 31;
     p.valid = p.j < lastw ? kFull : (p.j == lastw ? kFull >> (31 - lastb) : 0u);
+    if (OPEN && p.j == 0) p.valid &= ~1u;
+    if (OPEN && p.j == lastw) p.valid &= ~(1u << lastb);
+    p.on = p.j <= lastw;
     p.y0 = min((tid >> lws) * H, g.L);
     p.y1 = min(p.y0 + H, g.L);
     return p;
@@ -806,9 +867,16 @@ struct Decoder {
     uint32_t *fxp = map_x(t) + p.j, *fyp = map_y(t) + p.j;
     const int L = g.L, lws = g.lws, H = strip_rows();
     const Keys key = keys_of(t);
-    const bool on = p.valid != 0 && p.y0 < L;
+    const bool on = p.on && p.y0 < L;
     int n = 0, y = p.y0;
-    auto row = [&](int r) { return on ? sig[wrap_hi(wrap_lo(r, L), L) << lws] : 0u; };
+    auto row = [&](int r) {
+      if (OPEN && (unsigned)r >= (unsigned)L) return 0u;
+      return on ? sig[wrap_hi(wrap_lo(r, L), L) << lws] : 0u;
+    };
+    // OPEN: bits of the columns next to the rough ones (which hold no anyons, so
+    // the shifts need no clipping)
+    const uint32_t first = OPEN && p.j == 0 ? 2u : 0u;
+    const uint32_t last = OPEN && (L - 2) >> 5 == p.j ? 1u << ((L - 2) & 31) : 0u;
     // rows y - 1 (u), y (c), y + 1 (d), each with its shifted copies
     uint32_t u = row(y - 1), c = row(y);
     uint32_t ul = from_left(u, p), ur = from_right(u, p);
@@ -819,8 +887,8 @@ struct Decoder {
     for (int i = 0; i <= H; ++i, ++y) {
       const uint32_t d = row(y + 1);
       const uint32_t dl = from_left(d, p), dr = from_right(d, p);
-      const uint32_t px = ul | cl | dl;  // anyon in column x - 1
-      const uint32_t mx = ur | cr | dr;  // in column x + 1
+      const uint32_t px = ul | cl | dl | first;  // anyon in column x - 1
+      const uint32_t mx = ur | cr | dr | last;   // in column x + 1
       const uint32_t py = u | ul | ur, my = d | dl | dr;
       uint32_t todo = c & ~(px | mx | py | my);
       uint32_t mpy = c & my & ~py;  // moves +y
@@ -892,7 +960,7 @@ struct Decoder {
     const uint32_t *fxp = map_x(t) + p.j, *fyp = map_y(t) + p.j;
     uint32_t *cx = C + p.j, *cy = C + g.nws + p.j;
     const int lws = g.lws, H = strip_rows();
-    const bool on = p.valid != 0 && p.y0 < g.L;
+    const bool on = p.on && p.y0 < g.L;
     int n = 0;
     if (!on && p.y0 < g.L) {  // padding words stay 0
 #pragma unroll 1
@@ -946,11 +1014,11 @@ struct Decoder {
     Ent b = first;
     uint32_t m = 0;
     int q = 0;
-    if (near) {
+    if (OPEN || near) {
 #pragma unroll 1
       do {
         const uint32_t yx = dec(b);
-        m |= slice_near(x, y, (int)(yx & 0xFFFFu), (int)(yx >> 16), g.L, k);
+        m |= slice_near<OPEN>(x, y, (int)(yx & 0xFFFFu), (int)(yx >> 16), g.L, k);
         if (++q == kFew) break;
         b = e[q];
       } while (b != first);
@@ -965,7 +1033,7 @@ struct Decoder {
         b = e[q];
       } while (b != first);
     }
-    return m & slice_limit(a.m_max, k);
+    return (m | edges(x, k)) & slice_limit(a.m_max, k);
   }
   // Writes the anyons with alive set (np on lanes 0 .. n - 1) as the set of step
   // t, sorted; returns the anyon of lane i < number in pos.
@@ -1019,8 +1087,8 @@ struct Decoder {
         if (k <= lim) {
           const Ent* set = set_of(t - k);
           const uint32_t b0 = dec(set[0]), b1 = dec(set[1]);
-          m = slice_near(xa, ya, (int)(b0 & 0xFFFFu), (int)(b0 >> 16), g.L, k) |
-              slice_near(xa, ya, (int)(b1 & 0xFFFFu), (int)(b1 >> 16), g.L, k);
+          m = slice_near<false>(xa, ya, (int)(b0 & 0xFFFFu), (int)(b0 >> 16), g.L, k) |
+              slice_near<false>(xa, ya, (int)(b1 & 0xFFFFu), (int)(b1 >> 16), g.L, k);
         }
         const uint32_t seg = (__ballot_sync(kFull, m != 0) >> (lane & 16)) & 0xFFFFu;
         const uint32_t mm = __shfl_sync(kFull, m, (lane & 16) | ((__ffs(seg) - 1) & 15));
@@ -1045,7 +1113,10 @@ struct Decoder {
       // (literal ties may ask for a distance of the next slice)
       if (!__all_sync(kFull, hm != 0 && !(literal() && !(hm & 0xFFu) && !(h0 & 10u)))) break;
       int dir = direction(h0, h1, PLAIN ? QCA_TIE_LEX : a.tie_order);
-      if (dir >= 5) dir = 0;
+      if (dir >= 5)
+        dir = balance_random()
+                  ? draw_balance(dir, key_of(a.balance_key, a.shot_offset + shot, t), site(xa, ya))
+                  : 0;
       const uint32_t np = dir ? site_after(xa, ya, dir) : pa;
       const uint32_t q0 = __shfl_sync(kFull, np, 0), q1 = __shfl_sync(kFull, np, 16);
       const bool swap = q0 == p1 && q1 == p0;
@@ -1086,7 +1157,7 @@ struct Decoder {
     // the two snapshots' steps (-1: none), when the next ones are due
     int t_kept = -1, t_moving = -1, due_kept = 0, due_moving = 0, interval = 0;
     int n_before = 0, t_stop = -1, flag = 0;
-    const int near = (g.L - 1) / 6;  // slices within half the torus
+    const int near = OPEN ? 1 << 20 : (g.L - 1) / 6;  // slices within half the torus
     int t_pair = 1 << 30;            // first step with two anyons
     uint32_t pos = lane < n ? list[lane] : 0u;
     pos = write_set(t, (1u << n) - 1u, pos, n);
@@ -1097,11 +1168,11 @@ struct Decoder {
         t = a.max_steps;
         break;
       }
+      if (n == 2 && t_pair > t) t_pair = t;
       if (watch && t_stop < 0) {
         if (n != n_before) {
           // the number of anyons changed: a new orbit, if it is one
           n_before = n;
-          if (n == 2) t_pair = t;
           t_kept = t_moving = -1;
           due_moving = max(t, tf) + g.kmax + 1;
           due_kept = due_moving + g.kmax + 1;
@@ -1134,11 +1205,13 @@ struct Decoder {
           __syncwarp();
         }
       }
-      if (watch && n == 2 && t > t_pair) {
+      if (!OPEN && !moves_random() && n == 2 && t > t_pair) {
         const int t1 = pair_steps(
             t, t_pair, pos, n, near, t_stop < 0, t_kept, t_moving,
-            min(a.max_steps,
-                t_stop >= 0 ? t_stop : (t_kept < 0 ? min(due_kept, due_moving) : due_moving)));
+            !watch ? a.max_steps
+                   : min(a.max_steps, t_stop >= 0 ? t_stop
+                                                  : (t_kept < 0 ? min(due_kept, due_moving)
+                                                                : due_moving)));
         if (t1 != t) {
           t = t1;
           continue;
@@ -1179,7 +1252,8 @@ struct Decoder {
           uint32_t m = 0;
           const int k = kb + kk;
           if (kk < 2 && k <= lastt && ai < n && !hm)
-            m = slice_thread(slot(t - k), g.lws, g.L, xa, ya, k) & slice_limit(a.m_max, k);
+            m = (slice_thread<OPEN>(slot(t - k), g.lws, g.L, xa, ya, k) | edges(xa, k)) &
+                slice_limit(a.m_max, k);
           const uint32_t m0 = __shfl_sync(kFull, m, ai << lgS);
           const uint32_t m1 = __shfl_sync(kFull, m, (ai << lgS) + 1);
           if (!hm && (m0 | m1)) {
@@ -1246,7 +1320,7 @@ struct Decoder {
         }
       }
       if (dir && first) atomicXor(&C[lw], bit);
-      const bool stays = lane < n && !swap;
+      const bool stays = lane < n && !swap && bulk(np & 0xFFFFu);
       if (!stays) np = 0x80000000u | lane;
       int same = 0, lower = 0;
 #pragma unroll 1
@@ -1334,10 +1408,19 @@ struct Decoder {
         uint32_t s = 0;
         if (j <= lastw) {
           const int yu = y == 0 ? L - 1 : y - 1;
-          const uint32_t bx = B[w], by = B[g.nws + w], bu = B[g.nws + (yu << lws) + j];
-          const uint32_t carry = j ? B[w - 1] >> 31 : (B[(y << lws) + lastw] >> lastb) & 1u;
-          s = (bx ^ ((bx << 1) | carry) ^ by ^ bu) &
-              (j == lastw ? kFull >> (31 - lastb) : kFull);
+          uint32_t bx = B[w], by = B[g.nws + w], bu = B[g.nws + (yu << lws) + j];
+          uint32_t carry = j ? B[w - 1] >> 31 : (B[(y << lws) + lastw] >> lastb) & 1u;
+          uint32_t cols = j == lastw ? kFull >> (31 - lastb) : kFull;
+          if (OPEN) {
+            // links that do not exist count for nothing; the rough columns hold no
+            // anyons
+            if (j == 0) carry = 0;
+            if (j == lastw) bx &= ~(1u << lastb), cols &= ~(1u << lastb);
+            if (j == 0) cols &= ~1u;
+            if (y == L - 1) by = 0;
+            if (y == 0) bu = 0;
+          }
+          s = (bx ^ ((bx << 1) | carry) ^ by ^ bu) & cols;
           if (j == 0) wx ^= (int)(bx & 1u);
           if (y == 0) wy ^= __popc(by) & 1;
         }
@@ -1415,7 +1498,10 @@ struct Decoder {
     if (!LARGE && misc[3]) {
       // the whole CTA leaves together (misc[3] was read behind a barrier); the
       // banded or generic sweep decodes the shot afterwards
-      if (tid == 0) a.out_steps[shot] = kStepsPending;
+      if (tid == 0) {
+        a.out_steps[shot] = kStepsPending;
+        if (a.pending) atomicAdd(a.pending, 1u);
+      }
       return;
     }
     // ---- correction, homology, steps, flag
@@ -1450,7 +1536,8 @@ struct Decoder {
         a.out_cut[2 * shot + 1] = (uint8_t)wy;
         if (a.out_exhausted) a.out_exhausted[shot] = (uint8_t)(flag == 2);
       } else {
-        a.out_flag[shot] = (uint8_t)(flag == 2 ? 2 : ((wx | wy) ? 1 : 0));
+        // (the open lattice has one cut, between columns 0 and 1)
+        a.out_flag[shot] = (uint8_t)(flag == 2 ? 2 : ((OPEN ? wx : wx | wy) ? 1 : 0));
       }
     }
   }

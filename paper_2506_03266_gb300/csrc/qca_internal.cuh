@@ -54,6 +54,9 @@ struct DecodeArgs {
   int bytewise;
   // Decode only the shots whose out_steps is kStepsPending (the others are done).
   int only_pending;
+  // Optional count of them: the history sweep adds to it, and the sweeps that
+  // follow have nothing to do where it is 0.
+  unsigned int* pending;
 };
 
 // out_steps of a shot that the history sweep leaves to the sweeps with message
@@ -159,6 +162,15 @@ bool four_cta_chosen(int L);
 bool history_takes(int L, int v);
 bool history_may_leave_pending(int L);
 int launch_history(const DecodeArgs& a, cudaStream_t stream);
+// Open boundaries, default rules, v = 3, 8 <= L <= 256; may leave shots pending.
+int launch_history_open(const DecodeArgs& a, cudaStream_t stream);
+// The same for shots of several sizes (at most kHistoryMixSizes, all of the same
+// history_threads): sizes[c] is the size of the shots a.shot_list[start[c] ..
+// start[c + 1]).
+constexpr int kHistoryMixSizes = 16;
+int history_threads(int L);  // 0 above L = 256 or below 8
+int launch_history_mixed(const DecodeArgs& a, const int* sizes, const int64_t* start, int nsizes,
+                         cudaStream_t stream);
 int history_workspace_release();
 // Large-lattice kernel (cluster of 8 CTAs per shot, state in global memory).
 int tiled_path_for(int L, int v, int m_max);  // 1 if it takes (L, v, m_max)
@@ -170,6 +182,8 @@ int generic_forced(int L);  // qca_set_kernel_path(L, 0) is in effect
 int decode_path(int L, int v, int m_max);
 bool path_forced(int L);  // a kernel path or form was chosen for L by the caller
 int launch_decode(const DecodeArgs& a, cudaStream_t stream);
+// The sweeps that keep the message fields (on-chip, large-lattice or generic).
+int launch_planes(const DecodeArgs& a, cudaStream_t stream);
 // Mixed lattice sizes in one persistent launch (on-chip sweep): the group
 // size of a lattice size in it (0 two-CTA pair, else 512, 256, 128 or 64
 // threads; -1 not on the on-chip sweep), and the launch over items queued by

@@ -914,6 +914,7 @@ __global__ void __launch_bounds__(CL == 1 ? 1024 : (CL == 2 ? 512 : 256), CL == 
                                      (size_t)((g.cap + 7) & ~7) * 2);
   const int nclusters = gridDim.x / CL;
   const int cid = blockIdx.x / CL;
+  if (a.only_pending && a.pending && *a.pending == 0) return;  // (every CTA of the launch)
   // Work: static (cluster c takes c, c + nclusters, ...) or, with a queue,
   // dynamic (rank 0 of the cluster takes the next index and shares it).
   auto next_work = [&](int64_t prev) -> int64_t {
@@ -1120,6 +1121,10 @@ __global__ void __launch_bounds__(kMixThreads, 1) mixed_kernel(MixArgs m) {
   cg::cluster_group cluster = cg::this_cluster();
   const int csize = (int)cluster.num_blocks();
   const int rank = (int)cluster.block_rank();
+  if (m.a.only_pending && *m.a.pending == 0) return;  // (every CTA of the launch)
+  auto done = [&](int64_t shot) {
+    return m.a.only_pending && m.a.out_steps[shot] != kStepsPending;
+  };
   long long k = -1;
   // ---- pair items: both CTAs of the cluster on one shot
   if (m.n_pair > 0 && csize == 2) {
@@ -1134,7 +1139,10 @@ __global__ void __launch_bounds__(kMixThreads, 1) mixed_kernel(MixArgs m) {
         k = (rank == 0) ? kk : -1;
         break;
       }
-      decode_shot<2, 2>(m.a, m.geom[m.item_class[kk]], smem, m.a.shot_list[kk], whole);
+      const int64_t shot = m.a.shot_list[kk];
+      const bool skip = done(shot);
+      cluster.sync();  // both CTAs have read the shot's state before one writes it
+      if (!skip) decode_shot<2, 2>(m.a, m.geom[m.item_class[kk]], smem, shot, whole);
     }
   }
   // ---- every other item: groups of 512, 256, 128 or 64 threads
@@ -1159,7 +1167,10 @@ __global__ void __launch_bounds__(kMixThreads, 1) mixed_kernel(MixArgs m) {
       }
       continue;
     }
-    if (m.geom[c].L > 128)  // two plane words per lane
+    const bool skip = done(m.a.shot_list[k]);
+    G.sync();  // all have read the shot's state before one writes it
+    if (skip) {
+    } else if (m.geom[c].L > 128)  // two plane words per lane
       decode_shot<1, 2>(m.a, m.geom[c], smem + (size_t)(gofs / 64) * m.slice_bytes,
                         m.a.shot_list[k], G);
     else

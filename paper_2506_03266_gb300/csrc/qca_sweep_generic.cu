@@ -39,6 +39,7 @@ __global__ void __launch_bounds__(kThreads) sweep_generic_kernel(DecodeArgs a, u
   uint8_t* fl = dir + LL;            // [L][L] bit0: e_x flipped, bit1: e_y flipped
   __shared__ int s_red[2];
 
+  if (a.only_pending && a.pending && *a.pending == 0) return;
   __shared__ int64_t s_next;
   // static work (CTA b takes b, b + gridDim.x, ...) or a dynamic queue
   auto next_work = [&](int64_t prev) -> int64_t {

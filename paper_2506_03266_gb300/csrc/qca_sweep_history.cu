@@ -16,6 +16,8 @@
 // anyon searches; instruction fetch for the small sizes, whose warps are all at
 // different places of the code.  L = 256, p = 0.05, 20 000 shots: 4.8 ms, against
 // 55 ms for the sweep over message planes; floor by bytes 0.77 ms.
+#include <string.h>
+
 #include <algorithm>
 #include <atomic>
 #include <mutex>
@@ -28,21 +30,21 @@ namespace {
 
 using namespace hist;
 
-template <int NT, bool LARGE, bool PLAIN>
+template <int NT, bool LARGE, bool PLAIN, bool OPEN>
 __global__ void __launch_bounds__(NT, NT == 32 ? 24 : (NT == 1024 ? 1 : 768 / NT))
     history_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ Geom g,
                    uint32_t* ws, size_t slot_words) {
   extern __shared__ __align__(16) uint32_t sm[];
   uint32_t* base = LARGE ? ws + (size_t)blockIdx.x * slot_words : sm;
   for (int64_t k = blockIdx.x; k < a.shots; k += gridDim.x) {
-    Decoder<NT, LARGE, PLAIN> d{a, g};
+    Decoder<NT, LARGE, PLAIN, OPEN> d{a, g};
     d.ring = base;
     d.C = base + g.o_C;
     d.F = base + g.o_F;
     d.list = sm + g.o_list;
     d.table = sm + g.o_table;
     d.snap = sm + g.o_snap;
-    d.few = reinterpret_cast<typename Decoder<NT, LARGE, PLAIN>::Ent*>(sm + g.o_few);
+    d.few = reinterpret_cast<typename Decoder<NT, LARGE, PLAIN, OPEN>::Ent*>(sm + g.o_few);
     d.misc = reinterpret_cast<int*>(sm + g.o_misc);
     d.nset = reinterpret_cast<uint16_t*>(sm + g.o_misc + 8);
     d.shot = a.shot_list ? (int64_t)a.shot_list[k] : k;
@@ -52,6 +54,41 @@ __global__ void __launch_bounds__(NT, NT == 32 ? 24 : (NT == 1024 ? 1 : 768 / NT
     d.run();
     d.sync();  // the next shot reuses the state
   }
+}
+
+// Shots of several sizes: CTA b takes the b-th shot from the end of the list,
+// which is grouped by increasing size, so that the large shots start first.
+struct MixArgs {
+  DecodeArgs a;
+  int nsizes;
+  int64_t first[kHistoryMixSizes];  // list index of each size's first shot
+  int64_t end;
+  Geom geom[kHistoryMixSizes];
+};
+
+template <int NT, bool PLAIN>
+__global__ void __launch_bounds__(NT, NT == 32 ? 24 : 768 / NT)
+    history_mixed_kernel(const __grid_constant__ MixArgs m) {
+  extern __shared__ __align__(16) uint32_t sm[];
+  const int64_t k = m.end - 1 - blockIdx.x;
+  int c = 0;
+  while (c + 1 < m.nsizes && k >= m.first[c + 1]) ++c;
+  const Geom& g = m.geom[c];
+  Decoder<NT, false, PLAIN> d{m.a, g};
+  d.ring = sm;
+  d.C = sm + g.o_C;
+  d.F = nullptr;
+  d.list = sm + g.o_list;
+  d.table = sm + g.o_table;
+  d.snap = sm + g.o_snap;
+  d.few = reinterpret_cast<uint16_t*>(sm + g.o_few);
+  d.misc = reinterpret_cast<int*>(sm + g.o_misc);
+  d.nset = reinterpret_cast<uint16_t*>(sm + g.o_misc + 8);
+  d.shot = m.a.shot_list[k];
+  d.tid = threadIdx.x;
+  d.lane = threadIdx.x & 31;
+  d.warp = threadIdx.x >> 5;
+  d.run();
 }
 
 // Threads per shot: a warp up to L = 64 (no block barriers).  Above, four warps:
@@ -144,10 +181,10 @@ bool plain_rules(const DecodeArgs& a) {
   return a.move_thr == 0 && a.tie_order == QCA_TIE_LEX && a.balance_rule == QCA_BALANCE_STAY;
 }
 
-template <int NT, bool PLAIN>
+template <int NT, bool PLAIN, bool OPEN = false>
 int launch_small(const DecodeArgs& a, const Geom& g, size_t smem, int dev, cudaStream_t stream) {
   static std::atomic<int> have[64];
-  auto kern = history_kernel<NT, false, PLAIN>;
+  auto kern = history_kernel<NT, false, PLAIN, OPEN>;
   if (int rc = allow_smem(kern, smem, have, dev)) return rc;
   // a CTA per shot: the hardware hands out shots as CTAs retire
   const int64_t grid = std::min<int64_t>(a.shots, 1 << 30);
@@ -155,12 +192,21 @@ int launch_small(const DecodeArgs& a, const Geom& g, size_t smem, int dev, cudaS
   return cuda_fail(cudaGetLastError(), "history sweep launch");
 }
 
+template <int NT, bool PLAIN>
+int launch_mix(const MixArgs& m, size_t smem, int64_t shots, int dev, cudaStream_t stream) {
+  static std::atomic<int> have[64];
+  auto kern = history_mixed_kernel<NT, PLAIN>;
+  if (int rc = allow_smem(kern, smem, have, dev)) return rc;
+  kern<<<(unsigned)shots, NT, smem, stream>>>(m);
+  return cuda_fail(cudaGetLastError(), "history sweep launch (mixed sizes)");
+}
+
 template <bool PLAIN>
 int launch_large(const DecodeArgs& a, const Geom& g, size_t smem, size_t slot_words, int dev,
                  cudaStream_t stream) {
   constexpr int NT = 1024;
   static std::atomic<int> have[64];
-  auto kern = history_kernel<NT, true, PLAIN>;
+  auto kern = history_kernel<NT, true, PLAIN, false>;
   if (int rc = allow_smem(kern, smem, have, dev)) return rc;
   int sms = 0, per_sm = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -232,6 +278,67 @@ int launch_history(const DecodeArgs& a, cudaStream_t stream) {
       return plain ? launch_large<true>(a, g, smem, slot_words, dev, stream)
                    : launch_large<false>(a, g, smem, slot_words, dev, stream);
   }
+}
+
+int launch_history_open(const DecodeArgs& a, cudaStream_t stream) {
+  Geom g;
+  int threads;
+  size_t smem, slot_words;
+  if (a.v != 3 || a.L > 256 || !make_hist_geom(a.L, a.m_max, g, threads, smem, slot_words)) {
+    set_error("no open-boundary history sweep for L=%d v=%d", a.L, a.v);
+    return QCA_ERR_UNSUPPORTED;
+  }
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return cuda_fail(e, "cudaGetDevice");
+  if (dev < 0 || dev >= 64) {
+    set_error("device index %d out of range", dev);
+    return QCA_ERR_UNSUPPORTED;
+  }
+  return threads == 32 ? launch_small<32, true, true>(a, g, smem, dev, stream)
+                       : launch_small<128, true, true>(a, g, smem, dev, stream);
+}
+
+int history_threads(int L) { return L >= 8 && L <= 256 ? threads_for(L) : 0; }
+
+int launch_history_mixed(const DecodeArgs& a, const int* sizes, const int64_t* start, int nsizes,
+                         cudaStream_t stream) {
+  const int64_t shots = nsizes > 0 ? start[nsizes] - start[0] : 0;
+  if (shots == 0) return QCA_OK;
+  if (nsizes > kHistoryMixSizes || shots >= (int64_t)1 << 31) {
+    set_error("history sweep: %d sizes, %lld shots in one launch", nsizes, (long long)shots);
+    return QCA_ERR_UNSUPPORTED;
+  }
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return cuda_fail(e, "cudaGetDevice");
+  if (dev < 0 || dev >= 64) {
+    set_error("device index %d out of range", dev);
+    return QCA_ERR_UNSUPPORTED;
+  }
+  MixArgs m;
+  memset(&m, 0, sizeof(m));
+  m.a = a;
+  m.nsizes = nsizes;
+  m.end = start[nsizes];
+  size_t smem = 0;
+  int threads = 0;
+  for (int c = 0; c < nsizes; ++c) {
+    size_t s, slot;
+    m.first[c] = start[c];
+    if (!make_hist_geom(sizes[c], a.m_max, m.geom[c], threads, s, slot) ||
+        threads != history_threads(sizes[0])) {
+      set_error("no mixed history sweep for L=%d", sizes[c]);
+      return QCA_ERR_UNSUPPORTED;
+    }
+    smem = std::max(smem, s);
+  }
+  const bool plain = plain_rules(a);
+  if (threads == 32)
+    return plain ? launch_mix<32, true>(m, smem, shots, dev, stream)
+                 : launch_mix<32, false>(m, smem, shots, dev, stream);
+  return plain ? launch_mix<128, true>(m, smem, shots, dev, stream)
+               : launch_mix<128, false>(m, smem, shots, dev, stream);
 }
 
 int history_workspace_release() {

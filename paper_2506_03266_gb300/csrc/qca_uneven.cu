@@ -195,8 +195,8 @@ int qca_uneven_plan_create(const int32_t* L_host, int64_t shots, int64_t* offset
   if (shots > 0) {
     e = cudaMalloc(&p->d_list, sizeof(int32_t) * shots);
     if (e == cudaSuccess) e = cudaMalloc(&p->d_offsets, sizeof(int64_t) * shots);
-    // one counter per size, and the mixed queue's after them
-    if (e == cudaSuccess) e = cudaMalloc(&p->d_counters, sizeof(unsigned) * (nc + 1));
+    // one counter per size, after them the mixed queue's and the pending shots'
+    if (e == cudaSuccess) e = cudaMalloc(&p->d_counters, sizeof(unsigned) * (nc + 2));
     if (e == cudaSuccess)
       e = cudaMemcpy(p->d_list, list.data(), sizeof(int32_t) * shots, cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
@@ -302,28 +302,97 @@ int qca_decode_uneven_async(qca_uneven_plan_t p, const uint8_t* errors, int max_
   qca_default_config(&c);
   if (cfg) c = *cfg;
   cudaStream_t st = (cudaStream_t)stream;
-  // the mixed-size launch takes the queued sizes unless the per-size form is
-  // chosen, or the options leave the on-chip sweep (v != 3, m_max < 3) or
-  // change a planned group size (tuning overrides)
-  bool mixed = p->mode == 0 && p->m_items > 0 && c.v == 3;
+  // The packed batch decodes from the syndrome history (v = 3) where no kernel
+  // was chosen for a size: one launch over all sizes of the same CTA shape, for
+  // the shapes of at most 64 (a warp per shot) and 65 to 256 sites side by side;
+  // then the sweeps with message planes take what was left pending (usually
+  // nothing, and they return at once).  In the per-size form, and for every other
+  // size, each size has launches of its own on a forked stream.
+  cudaError_t e = cudaMemsetAsync(p->d_counters, 0, sizeof(unsigned) * (p->sizes.size() + 2), st);
+  if (e != cudaSuccess) return cuda_fail(e, "uneven decode counters");
+  DecodeArgs base;
+  int rc = fill_decode_args(base, errors, p->sizes[0], 0, max_steps, rng_seed, &c);
+  if (rc) return rc;
+  base.out_C = out_correction;
+  base.out_steps = out_steps;
+  base.out_flag = out_logical_fail;
+  base.offsets = p->d_offsets;
+  if ((rc = check_aligned(out_steps, 4, "out_steps"))) return rc;
+  const size_t ns = p->sizes.size();
+  std::vector<char> done(ns, 0);
+  // runs of consecutive sizes with the same CTA shape
+  struct Run {
+    size_t lo, hi;
+  };
+  std::vector<Run> runs;
+  for (size_t i = 0; p->mode == 0 && i < ns; ++i) {
+    const int th = history_threads(p->sizes[i]);
+    if (!th || !history_takes(p->sizes[i], c.v) || path_forced(p->sizes[i])) continue;
+    done[i] = 1;
+    if (!runs.empty() && runs.back().hi == i && i - runs.back().lo < kHistoryMixSizes &&
+        history_threads(p->sizes[runs.back().lo]) == th) {
+      runs.back().hi = i + 1;
+    } else {
+      runs.push_back({i, i + 1});
+    }
+  }
+  const size_t others = ns - std::count(done.begin(), done.end(), 1);
+  // side streams fork before the first launch
+  const bool fork = others > 0 || runs.size() > 1;
+  if (fork) {
+    e = cudaEventRecord(p->fork, st);
+    if (e != cudaSuccess) return cuda_fail(e, "uneven decode fork");
+  }
+  auto on_side = [&](size_t i) {
+    e = cudaStreamWaitEvent(p->side[i], p->fork, 0);
+    return e == cudaSuccess ? QCA_OK : cuda_fail(e, "uneven decode fork wait");
+  };
+  auto join = [&](size_t i) {
+    e = cudaEventRecord(p->join[i], p->side[i]);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(st, p->join[i], 0);
+    return e == cudaSuccess ? QCA_OK : cuda_fail(e, "uneven decode join");
+  };
+  // the largest sizes first, on the caller's stream
+  for (size_t q = runs.size(); q-- > 0;) {
+    const Run& r = runs[q];
+    const bool main = q + 1 == runs.size();
+    if (!main && (rc = on_side(r.lo))) return rc;
+    DecodeArgs a = base;
+    a.shots = p->start[r.hi - 1] + p->count[r.hi - 1] - p->start[r.lo];
+    a.shot_list = p->d_list;
+    a.pending = p->d_counters + ns + 1;
+    std::vector<int64_t> start(p->start.begin() + r.lo, p->start.begin() + r.hi);
+    start.push_back(p->start[r.hi - 1] + p->count[r.hi - 1]);
+    rc = launch_history_mixed(a, p->sizes.data() + r.lo, start.data(), (int)(r.hi - r.lo),
+                              main ? st : p->side[r.lo]);
+    if (rc) return rc;
+  }
+  for (size_t i = 0; i < ns; ++i) {
+    if (done[i]) continue;
+    if ((rc = on_side(i))) return rc;
+    DecodeArgs a = base;
+    a.L = p->sizes[i];
+    a.shots = p->count[i];
+    a.shot_list = p->d_list + p->start[i];
+    a.queue = p->d_counters + i;
+    a.bytewise = p->bytewise[i];
+    if ((rc = launch_decode(a, p->side[i]))) return rc;
+    if ((rc = join(i))) return rc;
+  }
+  for (size_t q = 0; q + 1 < runs.size(); ++q)
+    if ((rc = join(runs[q].lo))) return rc;
+  // ---- shots left pending
+  bool mixed = !runs.empty() && p->m_items > 0;
   for (size_t i = 0; mixed && i < p->msizes.size(); ++i)
     mixed = mixed_group_threads(p->msizes[i], c.m_max) == p->mgroup[i];
-  cudaError_t e = cudaMemsetAsync(p->d_counters, 0, sizeof(unsigned) * (p->sizes.size() + 1), st);
-  if (e != cudaSuccess) return cuda_fail(e, "uneven decode counters");
-  // the side streams fork before the mixed-size launch, so that the sizes
-  // outside its queue take SMs as its CTAs retire
-  e = cudaEventRecord(p->fork, st);
-  if (e != cudaSuccess) return cuda_fail(e, "uneven decode fork");
   if (mixed) {
-    DecodeArgs a;
-    int rc = fill_decode_args(a, errors, p->msizes[0], p->m_items, max_steps, rng_seed, &c);
-    if (rc) return rc;
-    a.out_C = out_correction;
-    a.out_steps = out_steps;
-    a.out_flag = out_logical_fail;
+    DecodeArgs a = base;
+    a.L = p->msizes[0];
+    a.shots = p->m_items;
     a.shot_list = p->d_mitems;
-    a.offsets = p->d_offsets;
-    a.queue = p->d_counters + p->sizes.size();
+    a.queue = p->d_counters + ns;
+    a.only_pending = 1;
+    a.pending = p->d_counters + ns + 1;
     int64_t n_pair = 0;
     for (size_t i = 0; i < p->mgroup.size(); ++i)
       if (p->mgroup[i] == 0) n_pair += p->mcount[i];
@@ -331,25 +400,16 @@ int qca_decode_uneven_async(qca_uneven_plan_t p, const uint8_t* errors, int max_
                       n_pair, p->m_items, st);
     if (rc) return rc;
   }
-  for (size_t i = 0; i < p->sizes.size(); ++i) {
-    if (mixed && p->in_mixed[i]) continue;
-    e = cudaStreamWaitEvent(p->side[i], p->fork, 0);
-    if (e != cudaSuccess) return cuda_fail(e, "uneven decode fork wait");
-    DecodeArgs a;
-    int rc = fill_decode_args(a, errors, p->sizes[i], p->count[i], max_steps, rng_seed, &c);
-    if (rc) return rc;
-    a.out_C = out_correction;
-    a.out_steps = out_steps;
-    a.out_flag = out_logical_fail;
+  for (size_t i = 0; i < ns; ++i) {
+    if (!done[i] || (mixed && p->in_mixed[i])) continue;
+    DecodeArgs a = base;
+    a.L = p->sizes[i];
+    a.shots = p->count[i];
     a.shot_list = p->d_list + p->start[i];
-    a.offsets = p->d_offsets;
-    a.queue = p->d_counters + i;
     a.bytewise = p->bytewise[i];
-    rc = launch_decode(a, p->side[i]);
-    if (rc) return rc;
-    e = cudaEventRecord(p->join[i], p->side[i]);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(st, p->join[i], 0);
-    if (e != cudaSuccess) return cuda_fail(e, "uneven decode join");
+    a.only_pending = 1;
+    a.pending = p->d_counters + ns + 1;
+    if ((rc = launch_planes(a, st))) return rc;
   }
   return QCA_OK;
 }

@@ -49,6 +49,7 @@ struct VariantArgs {
   uint8_t* out_C;
   int32_t* out_steps;
   uint8_t* out_flag;
+  int only_pending;  // decode only the shots whose out_steps is kStepsPending
 };
 
 __device__ __forceinline__ int vwrap(int i, int L) { return i < 0 ? i + L : (i >= L ? i - L : i); }
@@ -113,6 +114,12 @@ __global__ void __launch_bounds__(kVThreads) variant_kernel(VariantArgs a, uint8
   uint8_t* fl = dir + LL;           // [L][L] bit0 e_x flipped, bit1 e_y flipped
   __shared__ int s_red;
   for (int64_t shot = blockIdx.x; shot < a.shots; shot += gridDim.x) {
+    if (a.only_pending) {
+      // the shots the history sweep left; all threads read the state first
+      const bool done = a.out_steps[shot] != kStepsPending;
+      __syncthreads();
+      if (done) continue;
+    }
     const uint8_t* N = a.in + shot * 2 * (int64_t)LL;
     int any = 0;
     SitePos pi(L);
@@ -393,6 +400,7 @@ int variant_args(VariantArgs& a, const uint8_t* noise, int L, int64_t shots, int
   a.out_C = out_C;
   a.out_steps = out_steps;
   a.out_flag = out_flag;
+  a.only_pending = 0;
   return QCA_OK;
 }
 
@@ -416,6 +424,15 @@ int qca_decode_open_batch_async(const uint8_t* noise, int L, int64_t shots, int 
     return QCA_ERR_UNSUPPORTED;
   }
   if (shots == 0) return QCA_OK;
+  if (history_takes(L, a.v) && L <= 256) {
+    DecodeArgs h;
+    if ((rc = fill_decode_args(h, noise, L, shots, max_steps, 0, cfg))) return rc;
+    h.out_C = out_correction;
+    h.out_steps = out_steps;
+    h.out_flag = out_logical_fail;
+    if ((rc = launch_history_open(h, (cudaStream_t)stream))) return rc;
+    a.only_pending = 1;
+  }
   return launch_variant(kOpen, a, (cudaStream_t)stream);
 }
 
