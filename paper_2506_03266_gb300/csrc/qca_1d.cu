@@ -20,7 +20,10 @@
 // step takes three block barriers.
 // After the last step N xor C is constant on the ring; its value is the
 // decoded logical value.
-#include "qca_internal.cuh"
+#include <algorithm>
+#include <atomic>
+
+#include "qca_history_1d.cuh"
 
 namespace qca {
 
@@ -41,22 +44,6 @@ __global__ void sample_1d_kernel(int L, int64_t shot0, int64_t shots, uint64_t t
     out[i] = splitmix64(ks ^ (uint64_t)r) < thr ? 1 : 0;
   }
 }
-
-struct Args1D {
-  const uint8_t* in;
-  int L;
-  int64_t shots;
-  int max_steps;
-  int v;
-  int m_max;
-  uint64_t move_thr;
-  uint64_t move_key;
-  int64_t shot_offset;
-  uint8_t* out_C;
-  int32_t* out_steps;
-  uint8_t* out_flag;
-  uint8_t* out_maj;
-};
 
 // i mod L: one correction covers every offset of a ring of at least 8 sites
 // (offsets are at most v = 8); shorter rings take the remainder
@@ -175,6 +162,53 @@ __global__ void __launch_bounds__(k1DThreads) decode_1d_kernel(Args1D a) {
   }
 }
 
+template <int NT>
+__global__ void __launch_bounds__(NT)
+    ring_history_kernel(const __grid_constant__ Args1D a, int W, int depth) {
+  extern __shared__ __align__(16) uint32_t rsm[];
+  hist::RingDecoder<NT> d{a};
+  d.W = W;
+  d.depth = depth;
+  d.ring = rsm;
+  d.xch = rsm + depth * W;
+  d.misc = reinterpret_cast<int*>(d.xch + 2 * W);
+  d.tid = threadIdx.x;
+  d.lane = threadIdx.x & 31;
+  d.run(blockIdx.x);
+}
+
+// The history form of the ring: L from 64 up, one thread per 32 sites, where the
+// ring's history fits shared memory (every size at v = 3).  Returns whether it
+// takes the call, and its result in rc.
+bool launch_ring_history(const Args1D& a, cudaStream_t stream, int& rc) {
+  const int W = (a.L + 31) / 32;
+  const int depth = (int)std::min<int64_t>((a.m_max - 1) / a.v, a.max_steps) + 2;
+  const size_t smem = ((size_t)depth * W + 2 * W + 4) * 4;
+  if (a.L < 64 || W > 512 || smem > 220 * 1024 || a.shots >= (int64_t)1 << 31) return false;
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  rc = cuda_fail(e, "cudaGetDevice");
+  if (rc || dev < 0 || dev >= 64) return rc != 0;
+  auto go = [&](auto kern, int nt, std::atomic<int>* have) {
+    if (smem > 48 * 1024 && !have[dev].load()) {
+      rc = cuda_fail(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          220 * 1024), "ring decode smem attribute");
+      if (rc) return;
+      have[dev].store(1);
+    }
+    kern<<<(unsigned)a.shots, nt, smem, stream>>>(a, W, depth);
+    rc = cuda_fail(cudaGetLastError(), "ring decode launch");
+  };
+  static std::atomic<int> have[3][64];
+  if (W <= 32)
+    go(ring_history_kernel<32>, 32, have[0]);
+  else if (W <= 128)
+    go(ring_history_kernel<128>, 128, have[1]);
+  else
+    go(ring_history_kernel<512>, 512, have[2]);
+  return true;
+}
+
 uint64_t thr_1d(double p) {
   if (!(p > 0.0)) return 0;
   if (p >= 1.0) return UINT64_MAX;
@@ -246,6 +280,8 @@ int qca_decode_1d_batch_async(const uint8_t* noise, int L, int64_t shots, int ma
   a.out_steps = out_steps;
   a.out_flag = out_flag;
   a.out_maj = out_majority_flag;
+  int rc = QCA_OK;
+  if (launch_ring_history(a, (cudaStream_t)stream, rc)) return rc;
   const size_t smem = 8 * (size_t)L;
   cudaError_t e = cudaFuncSetAttribute(decode_1d_kernel,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

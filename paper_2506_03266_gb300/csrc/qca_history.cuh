@@ -296,9 +296,6 @@ __device__ __forceinline__ int direction(uint32_t h0, uint32_t h1, int tie_order
 }
 
 // The counter draws, out of line: options that most calls leave off.
-struct Keys {
-  uint64_t move, bal;
-};
 static __device__ __noinline__ uint64_t key_of(uint64_t key, int64_t shot, int t) {
   return move_step_key(key, shot, t);
 }
@@ -678,21 +675,23 @@ struct Decoder {
     return m;
   }
 
-  __device__ __forceinline__ Keys keys_of(int t) const {
-    Keys q{0, 0};
-    if (moves_random()) q.move = key_of(a.move_key, a.shot_offset + shot, t);
-    if (balance_random()) q.bal = key_of(a.balance_key, a.shot_offset + shot, t);
-    return q;
+  __device__ __forceinline__ uint64_t move_key_of(int t) const {
+    return moves_random() ? key_of(a.move_key, a.shot_offset + shot, t) : 0;
+  }
+  // A balanced axis (5 x, 6 y) of the anyon at (x, y) at step t, resolved.
+  __device__ __forceinline__ int balanced(int code, int x, int y, int t) const {
+    if (!balance_random()) return 0;
+    return draw_balance(code, key_of(a.balance_key, a.shot_offset + shot, t), site(x, y));
   }
   // The move of the anyon at (x, y) that hears h0 (and h1 at the next distance).
-  __device__ __forceinline__ int move_of(const Keys& key, int x, int y, uint32_t h0,
+  __device__ __forceinline__ int move_of(uint64_t move_key, int x, int y, int t, uint32_t h0,
                                          uint32_t h1) const {
     int dir = h0 ? direction(h0, h1, PLAIN ? QCA_TIE_LEX : a.tie_order) : 0;
-    if (dir >= 5) dir = balance_random() ? draw_balance(dir, key.bal, site(x, y)) : 0;
     if (moves_random()) {
-      const int d = draw_move(key.move, a.move_thr, site(x, y));
-      if (d) dir = d;
+      const int d = draw_move(move_key, a.move_thr, site(x, y));
+      if (d) return d;
     }
+    if (dir >= 5) dir = balanced(dir, x, y, t);
     return dir;
   }
   // Hits at the smallest distance of a slice's hits, and at the next one (0
@@ -746,7 +745,7 @@ struct Decoder {
     bool moved = false;
     const uint32_t* sig = slot(t);
     uint32_t* sn = slot(t + 1);
-    const Keys key = keys_of(t);
+    const uint64_t key = move_key_of(t);
     const int last = min(t, g.kmax);
     const int lastt = min(min(last, g.kthread), t - oldest());
 #pragma unroll 1
@@ -793,7 +792,7 @@ struct Decoder {
           if (lane == src) h1 = mm & 15u;
         }
       }
-      const int dir = act ? move_of(key, x, y, h0, h1) : 0;
+      const int dir = act ? move_of(key, x, y, t, h0, h1) : 0;
       if (dir) {
         moved = true;
         uint32_t bit;
@@ -866,7 +865,6 @@ struct Decoder {
     uint32_t* open = slot(t + 1) + p.j;
     uint32_t *fxp = map_x(t) + p.j, *fyp = map_y(t) + p.j;
     const int L = g.L, lws = g.lws, H = strip_rows();
-    const Keys key = keys_of(t);
     const bool on = p.on && p.y0 < L;
     int n = 0, y = p.y0;
     auto row = [&](int r) {
@@ -905,13 +903,13 @@ struct Decoder {
 #pragma unroll 1
         for (uint32_t b = xs & px & mx; b; b &= b - 1) {
           const int q = __ffs(b) - 1;
-          if (draw_balance(5, key.bal, site((p.j << 5) + q, wrap_hi(y, L))) == 1) mpx |= 1u << q;
+          if (balanced(5, (p.j << 5) + q, wrap_hi(y, L), t) == 1) mpx |= 1u << q;
           else mmx |= 1u << q;
         }
 #pragma unroll 1
         for (uint32_t b = c & my & py; b; b &= b - 1) {
           const int q = __ffs(b) - 1;
-          if (draw_balance(6, key.bal, site((p.j << 5) + q, wrap_hi(y, L))) == 3) mpy |= 1u << q;
+          if (balanced(6, (p.j << 5) + q, wrap_hi(y, L), t) == 3) mpy |= 1u << q;
           else mmy |= 1u << q;
         }
       }
@@ -1080,7 +1078,8 @@ struct Decoder {
       const uint32_t pa = second ? p1 : p0;
       const int xa = pa & 0xFFFFu, ya = pa >> 16;
       const int lim = min(klim, t - t_pair);
-      uint32_t hm = 0;
+      uint32_t hm = 0, hn = 0;  // hits of the first slice with any, of the one after it
+      bool next = false;        // hn is known
 #pragma unroll 1
       for (int k = kk; k - kk <= lim; k += 16) {
         uint32_t m = 0;
@@ -1091,7 +1090,15 @@ struct Decoder {
               slice_near<false>(xa, ya, (int)(b1 & 0xFFFFu), (int)(b1 >> 16), g.L, k);
         }
         const uint32_t seg = (__ballot_sync(kFull, m != 0) >> (lane & 16)) & 0xFFFFu;
-        const uint32_t mm = __shfl_sync(kFull, m, (lane & 16) | ((__ffs(seg) - 1) & 15));
+        const int f = (__ffs(seg) - 1) & 15;
+        const uint32_t mm = __shfl_sync(kFull, m, (lane & 16) | f);
+        if (!PLAIN) {
+          const uint32_t mn = __shfl_sync(kFull, m, (lane & 16) | ((f + 1) & 15));
+          if (!hm && seg && f < 15 && k - kk + f < lim) {
+            hn = mn;
+            next = true;
+          }
+        }
         if (!hm && seg) hm = mm;
         if (__all_sync(kFull, hm != 0)) break;
       }
@@ -1111,12 +1118,13 @@ struct Decoder {
       uint32_t h0 = 0, h1 = 0;
       if (hm) nearest(hm, h0, h1);
       // (literal ties may ask for a distance of the next slice)
-      if (!__all_sync(kFull, hm != 0 && !(literal() && !(hm & 0xFFu) && !(h0 & 10u)))) break;
+      if (literal() && !(hm & 0xFFu) && !(h0 & 10u)) {
+        h1 = hn & 15u;
+        if (!next) hm = 0;
+      }
+      if (!__all_sync(kFull, hm != 0)) break;
       int dir = direction(h0, h1, PLAIN ? QCA_TIE_LEX : a.tie_order);
-      if (dir >= 5)
-        dir = balance_random()
-                  ? draw_balance(dir, key_of(a.balance_key, a.shot_offset + shot, t), site(xa, ya))
-                  : 0;
+      if (dir >= 5) dir = 0;
       const uint32_t np = dir ? site_after(xa, ya, dir) : pa;
       const uint32_t q0 = __shfl_sync(kFull, np, 0), q1 = __shfl_sync(kFull, np, 16);
       const bool swap = q0 == p1 && q1 == p0;
@@ -1205,13 +1213,11 @@ struct Decoder {
           __syncwarp();
         }
       }
-      if (!OPEN && !moves_random() && n == 2 && t > t_pair) {
+      if (!OPEN && watch && n == 2 && t > t_pair) {
         const int t1 = pair_steps(
             t, t_pair, pos, n, near, t_stop < 0, t_kept, t_moving,
-            !watch ? a.max_steps
-                   : min(a.max_steps, t_stop >= 0 ? t_stop
-                                                  : (t_kept < 0 ? min(due_kept, due_moving)
-                                                                : due_moving)));
+            min(a.max_steps,
+                t_stop >= 0 ? t_stop : (t_kept < 0 ? min(due_kept, due_moving) : due_moving)));
         if (t1 != t) {
           t = t1;
           continue;
@@ -1300,8 +1306,8 @@ struct Decoder {
       h0 = __shfl_sync(kFull, h0, (lane << lgS) & 31);
       h1 = __shfl_sync(kFull, h1, (lane << lgS) & 31);
       const int x = pos & 0xFFFFu, y = pos >> 16;
-      const Keys key = keys_of(t);
-      const int dir = lane < n ? move_of(key, x, y, h0, h1) : 0;
+      const uint64_t key = move_key_of(t);
+      const int dir = lane < n ? move_of(key, x, y, t, h0, h1) : 0;
       uint32_t np = pos, bit = 0;
       int lw = 0;
       if (dir) {

@@ -120,3 +120,52 @@ def test_unaligned_blocks():
             torch.cuda.synchronize()
             same([x.cpu().numpy() for x in (C, steps, flag)], ref, f"L{L} off {off}")
             assert int(out[:off].sum()) == 0 and int(out[off + 8 * n:].sum()) == 0
+
+
+@pytest.mark.parametrize("L", [63, 64, 65, 95, 96, 127, 1024, 1025, 4096, 4099, 16384])
+def test_ring_history_against_oracle(L):
+    shots = 40 if L < 2000 else 4
+    for p, v, m_max, p_move in [(0.3, 3, 255, 0.1), (0.2, 3, 255, 0.0), (0.2, 2, 9, 0.0),
+                                (0.25, 8, 255, 0.05), (0.2, 1, 255, 0.0)]:
+        N = oracle.sample_errors_1d(L, shots, p, seed=L)
+        got = qca.decode_1d_batch(torch.from_numpy(N).cuda(), max_steps=60, v=v, m_max=m_max,
+                                  p_move=p_move, rng_seed=3)
+        C, s, f, m = [x.cpu().numpy() for x in got]
+        thr = oracle.prob_threshold(p_move) if p_move else 0
+        for i in range(shots):
+            Co, so, fo, mo = oracle.decode_shot_1d(N[i], v=v, m_max=m_max, max_steps=60,
+                                                   move_thr=thr, seed=3, shot=i)
+            assert (s[i], f[i], m[i]) == (so, fo, mo), (L, p, v, m_max, p_move, i)
+            np.testing.assert_array_equal(C[i], Co)
+
+
+@pytest.mark.parametrize("L", [8, 9, 16, 31, 33, 64, 65, 96, 130, 200, 256])
+def test_open_history_against_oracle(L):
+    """Tile and word edges of the open lattice, and caps that cut a slice."""
+    shots = 24 if L <= 64 else 3
+    for p, m_max in [(0.03, 255), (0.08, 255), (0.08, 2), (0.08, 7)]:
+        N = oracle.sample_errors(L, shots, p, seed=L)
+        got = qca.decode_open_batch(torch.from_numpy(N).cuda(), max_steps=80, m_max=m_max)
+        C, s, f = [x.cpu().numpy() for x in got]
+        for i in range(shots if L <= 64 else 1):
+            Co, so, fo = oracle.open_decode_shot(N[i], m_max=m_max, max_steps=80)
+            assert (s[i], f[i]) == (so, fo), (L, p, m_max, i)
+            np.testing.assert_array_equal(C[i], Co)
+
+
+def test_mixed_sizes_with_odd_ones_and_both_cta_shapes():
+    rng = np.random.default_rng(3)
+    Ls = rng.choice(np.array([9, 15, 24, 33, 48, 64, 65, 81, 96, 128, 130, 192, 255, 256, 257, 7, 10,
+                              11, 12, 13, 14, 18, 19, 20, 21, 22, 23, 25], dtype=np.int32), 300)
+    plan = qca.UnevenPlan(Ls)
+    N = plan.sample(np.full(len(Ls), oracle.prob_threshold(0.05), dtype=np.uint64), seed=2)
+    C, s, f = plan.decode(N, max_steps=200)
+    torch.cuda.synchronize()
+    for i in rng.permutation(len(Ls))[:120]:
+        L = int(Ls[i])
+        n = N[plan.offsets[i]: plan.offsets[i] + 2 * L * L].view(1, 2, L, L).contiguous()
+        ref = decode(n, path=0, max_steps=200)
+        c = C[plan.offsets[i]: plan.offsets[i] + 2 * L * L].view(2, L, L).cpu().numpy()
+        assert (int(s[i]), int(f[i])) == (ref[1][0], ref[2][0]), (i, L)
+        np.testing.assert_array_equal(c, ref[0][0])
+    plan.close()
