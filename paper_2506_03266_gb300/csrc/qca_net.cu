@@ -27,6 +27,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <mutex>
 #include <vector>
 
 #include "qca_internal.cuh"
@@ -64,6 +65,34 @@ __global__ void syndrome_kernel(const uint8_t* __restrict__ N, int L, int64_t sh
     sig[i] = n[r] ^ n[y * L + wrapL(x - 1, L)] ^ n[LL + r] ^ n[LL + wrapL(y - 1, L) * L + x];
   }
 }
+
+// The same, 16 sites per thread and access (L a multiple of 16, arrays on a
+// 16-byte boundary): bound by its 3 bytes per site instead of by a site's index
+// arithmetic (16.4 M sites: 60 -> 9 us).
+__global__ void syndrome16_kernel(const uint8_t* __restrict__ N, int L, int64_t shots,
+                                  uint8_t* __restrict__ sig) {
+  const uint32_t vpr = (uint32_t)L >> 4, vps = vpr * (uint32_t)L;  // vectors per row, per shot
+  const int64_t LL = (int64_t)L * L;
+  for (int64_t s = blockIdx.y; s < shots; s += gridDim.y) {
+    const uint8_t* n = N + s * 2 * LL;
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < vps; i += gridDim.x * blockDim.x) {
+      const uint32_t y = i / vpr, x = (i - y * vpr) << 4;
+      const uint32_t yu = y == 0 ? L - 1 : y - 1;
+      const uint4 ex = *reinterpret_cast<const uint4*>(n + (size_t)y * L + x);
+      const uint32_t left = n[(size_t)y * L + (x == 0 ? L - 1 : x - 1)];
+      const uint4 ey = *reinterpret_cast<const uint4*>(n + LL + (size_t)y * L + x);
+      const uint4 eu = *reinterpret_cast<const uint4*>(n + LL + (size_t)yu * L + x);
+      uint4 v;
+      v.x = ex.x ^ ((ex.x << 8) | left) ^ ey.x ^ eu.x;
+      v.y = ex.y ^ __funnelshift_l(ex.x, ex.y, 8) ^ ey.y ^ eu.y;
+      v.z = ex.z ^ __funnelshift_l(ex.y, ex.z, 8) ^ ey.z ^ eu.z;
+      v.w = ex.w ^ __funnelshift_l(ex.z, ex.w, 8) ^ ey.w ^ eu.w;
+      *reinterpret_cast<uint4*>(sig + s * LL + (size_t)y * L + x) = v;
+    }
+  }
+}
+
+int launch_syndrome(const uint8_t* N, int L, int64_t shots, uint8_t* sig, cudaStream_t st);
 
 // First-step direction of every anyon (0 +x, 1 -x, 2 +y, 3 -y, 4 none; 255 no
 // anyon).  With empty fields, three applications of A^(D) leave in m^{s a}_r
@@ -1768,8 +1797,17 @@ __global__ void bias_grad_kernel(const __nv_bfloat16* __restrict__ d, int64_t S,
   __shared__ float red[8][32];
   const int c = threadIdx.x & 31, row = threadIdx.x >> 5;
   float acc = 0.f;
-  for (int64_t s = blockIdx.x * 8 + row; s < S; s += (int64_t)gridDim.x * 8)
-    acc += __bfloat162float(d[s * 32 + c]);
+  // (eight loads in flight, added in order: 22 -> 13 us per 262 144 sites)
+  const int64_t step = (int64_t)gridDim.x * 8;
+  int64_t s = blockIdx.x * 8 + row;
+  for (; s + 7 * step < S; s += 8 * step) {
+    __nv_bfloat16 v[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) v[q] = d[(s + q * step) * 32 + c];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) acc += __bfloat162float(v[q]);
+  }
+  for (; s < S; s += step) acc += __bfloat162float(d[s * 32 + c]);
   red[row][c] = acc;
   __syncthreads();
   if (row == 0) {
@@ -1779,33 +1817,62 @@ __global__ void bias_grad_kernel(const __nv_bfloat16* __restrict__ d, int64_t S,
   }
 }
 
-// out[i] = sum over p = 0 .. nparts - 1, in that order, of part[p * stride + i]:
-// the per-CTA partial sums of a gradient added in a fixed order, so that a
-// training run repeats bit for bit.
-__global__ void reduce_parts_kernel(const float* __restrict__ part, int nparts, int stride, int n,
+// The per-CTA partial sums of all gradients of a step, in the order they are
+// made: weights and bias of layers 4 .. 1.  Entry k has parts_k rows of stride_k
+// floats at part + at_k; the sum of the rows' first n_k columns goes to out + to_k.
+constexpr int kGradSets = 8;
+struct GradSets {
+  int64_t at[kGradSets];
+  int parts[kGradSets], stride[kGradSets], n[kGradSets], to[kGradSets];
+};
+
+// out[to + i] = sum over p = 0 .. parts - 1, in that order, of part[at + p * stride
+// + i]: a fixed order, so that a training run repeats bit for bit.  Bound by the
+// latency of the loads, so 32 of them are in flight, and one launch takes all the
+// sets of a step (eight launches with one load in flight took 200 us per step).
+__global__ void reduce_parts_kernel(const float* __restrict__ part,
+                                    const __grid_constant__ GradSets g, int total,
                                     float* __restrict__ out) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    float v = 0.f;
-    for (int q = 0; q < nparts; ++q) v += part[(size_t)q * stride + i];
-    out[i] = v;
+  int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= total) return;
+  int k = 0;
+  while (i >= g.n[k]) i -= g.n[k++];
+  const float* p = part + g.at[k] + i;
+  const int parts = g.parts[k], stride = g.stride[k];
+  float v = 0.f;
+  int q = 0;
+  for (; q + 32 <= parts; q += 32) {
+    float w[32];
+#pragma unroll
+    for (int r = 0; r < 32; ++r) w[r] = p[(size_t)(q + r) * stride];
+#pragma unroll
+    for (int r = 0; r < 32; ++r) v += w[r];
   }
+  for (; q < parts; ++q) v += p[(size_t)q * stride];
+  out[g.to[k] + i] = v;
 }
 
 constexpr int kWgChunk = 64;   // sites staged per round
-constexpr int kWgPitch = 36;   // words per staged row (64 sites = 32 words, padded)
+constexpr int kWgStage = 10 * kWgChunk * 64;  // bytes of a stage: dout and nine taps of in
 
 // dW[co][ci][tap] += sum over the CTA's sites s of dout[s][co] in[nb(s, tap)][ci]
 // (nb: the circular neighbour of s at tap offset (ky - 1, kx - 1)); dout and in
 // bf16 NHWC [S][32]; only co < CO_REAL, ci < CI_REAL are written (param layout
 // [co][CI_REAL][9]).  256 threads: warp w owns output channels 16 (w / 4) ..
 // +15 and the n-tiles 9 (w % 4) .. +8 of the 36 (tap, 8-channel block) tiles.
+//
+// Both operands have the sum index (the site) as their slow one, so the sites
+// are staged as they lie, 64 bytes each, by cp.async into two stages, and
+// ldmatrix.trans hands the fragments over transposed; the 16-byte groups of a
+// site are permuted by its index so that the eight rows of a matrix fall into
+// different banks.  (Transposing by 2-byte stores into one stage, with no copy in
+// flight during the MMAs, took 81 us per 262 144 sites; this form 39 us.)
 template <int CO_REAL, int CI_REAL>
 __global__ void __launch_bounds__(256) wgrad_mma_kernel(const __nv_bfloat16* __restrict__ dout,
                                                         const __nv_bfloat16* __restrict__ in,
                                                         int L, int64_t S, int64_t chunk,
                                                         float* __restrict__ part) {
-  __shared__ uint32_t sD[32 * kWgPitch];       // [co][site pair]
-  __shared__ uint32_t sI[9 * 32 * kWgPitch];   // [tap][ci][site pair]
+  extern __shared__ __align__(128) uint8_t wg_smem[];  // [2][dout, tap 0 .. 8][site][64 bytes]
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int g = lane >> 2, t = lane & 3;
   const int mt = warp >> 2, nt0 = (warp & 3) * 9;
@@ -1814,57 +1881,79 @@ __global__ void __launch_bounds__(256) wgrad_mma_kernel(const __nv_bfloat16* __r
   float acc[9][4];
 #pragma unroll
   for (int k = 0; k < 9; ++k) acc[k][0] = acc[k][1] = acc[k][2] = acc[k][3] = 0.f;
-  __nv_bfloat16* sDh = reinterpret_cast<__nv_bfloat16*>(sD);
-  __nv_bfloat16* sIh = reinterpret_cast<__nv_bfloat16*>(sI);
-  for (int64_t base = s_begin; base < s_end; base += kWgChunk) {
-    __syncthreads();
-    // stage: thread (site j, octet o) transposes 8 channels of dout and of the
-    // nine neighbours of site base + j
-    {
-      const int j = tid >> 2, o = tid & 3;
-      const int64_t s = base + j;
-      const bool ok = s < s_end;
-      uint4 v = make_uint4(0, 0, 0, 0);
-      if (ok) v = *reinterpret_cast<const uint4*>(dout + s * 32 + o * 8);
-      const __nv_bfloat16* vh = reinterpret_cast<const __nv_bfloat16*>(&v);
+  const uint32_t smem0 = (uint32_t)__cvta_generic_to_shared(wg_smem);
+  // stage: thread (site j, octet o) copies 8 channels of dout and of the nine
+  // neighbours of site base + j (zeros past the end)
+  auto stage = [&](int64_t base, int buf) {
+    const int j = tid >> 2, o = tid & 3;
+    const int64_t s = base + j;
+    const bool ok = s < s_end;
+    const uint32_t dst = smem0 + buf * kWgStage + j * 64 + ((o ^ ((j >> 1) & 3)) << 4);
+    const int bytes = ok ? 16 : 0;
+    auto copy = [&](uint32_t to, const __nv_bfloat16* from) {
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(to), "l"(from),
+                   "r"(bytes)
+                   : "memory");
+    };
+    int64_t shot = 0;
+    int x = 0, y = 0;
+    if (ok) {
+      shot = s / LL;
+      const int r = (int)(s - shot * LL);
+      y = r / L;
+      x = r - y * L;
+    }
+    copy(dst, dout + (ok ? s * 32 + o * 8 : 0));
 #pragma unroll
-      for (int k = 0; k < 8; ++k) sDh[(o * 8 + k) * (2 * kWgPitch) + j] = vh[k];
-      int64_t shot = 0;
-      int x = 0, y = 0;
-      if (ok) {
-        shot = s / LL;
-        const int r = (int)(s - shot * LL);
-        x = r % L;
-        y = r / L;
-      }
-#pragma unroll
-      for (int tap = 0; tap < 9; ++tap) {
-        uint4 u = make_uint4(0, 0, 0, 0);
-        if (ok) {
-          const int xx = wrapL(x + tap % 3 - 1, L), yy = wrapL(y + tap / 3 - 1, L);
-          u = *reinterpret_cast<const uint4*>(in + (shot * LL + (int64_t)yy * L + xx) * 32 + o * 8);
-        }
-        const __nv_bfloat16* uh = reinterpret_cast<const __nv_bfloat16*>(&u);
-#pragma unroll
-        for (int k = 0; k < 8; ++k) sIh[((tap * 32) + o * 8 + k) * (2 * kWgPitch) + j] = uh[k];
-      }
+    for (int tap = 0; tap < 9; ++tap) {
+      const int xx = wrapL(x + tap % 3 - 1, L), yy = wrapL(y + tap / 3 - 1, L);
+      copy(dst + (tap + 1) * kWgChunk * 64,
+           in + (ok ? (shot * LL + (int64_t)yy * L + xx) * 32 + o * 8 : 0));
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  // address of the 16-byte group (site, octet) of one operand in a stage
+  auto group = [&](uint32_t op, int site, int octet) {
+    return op + site * 64 + ((octet ^ ((site >> 1) & 3)) << 4);
+  };
+  if (s_begin < s_end) stage(s_begin, 0);
+  int buf = 0;
+  for (int64_t base = s_begin; base < s_end; base += kWgChunk, buf ^= 1) {
+    if (base + kWgChunk < s_end) {
+      stage(base + kWgChunk, buf ^ 1);
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+    } else {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
     }
     __syncthreads();
+    const uint32_t sD = smem0 + buf * kWgStage, sI = sD + kWgChunk * 64;
 #pragma unroll
     for (int ks = 0; ks < kWgChunk / 16; ++ks) {
+      // A: sites 16 ks .. + 15 by channels 16 mt .. + 15, in four 8 x 8 matrices
+      // (lane: row lane & 7 of matrix lane >> 3; matrix bit 0 = channels + 8, bit 1
+      // = sites + 8)
       uint32_t a[4];
-      const uint32_t* ar = sD + (mt * 16 + g) * kWgPitch + ks * 8 + t;
-      a[0] = ar[0];
-      a[1] = ar[8 * kWgPitch];
-      a[2] = ar[4];
-      a[3] = ar[8 * kWgPitch + 4];
+      const int mi = lane >> 3, mr = lane & 7;
+      const uint32_t aa = group(sD, ks * 16 + ((mi >> 1) << 3) + mr, mt * 2 + (mi & 1));
+      asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                   : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3])
+                   : "r"(aa)
+                   : "memory");
 #pragma unroll
       for (int k = 0; k < 9; ++k) {
-        const int ntile = nt0 + k, tap = ntile >> 2, ci = (ntile & 3) * 8 + g;
-        const uint32_t* br = sI + (tap * 32 + ci) * kWgPitch + ks * 8 + t;
-        mma_bf16(acc[k], a, br[0], br[4]);
+        const int ntile = nt0 + k, tap = ntile >> 2;
+        // B: the same sites by 8 input channels of the tap (lanes 0 .. 15 give rows)
+        uint32_t b0, b1;
+        const uint32_t ba =
+            group(sI + tap * kWgChunk * 64, ks * 16 + (mi & 1) * 8 + mr, ntile & 3);
+        asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0, %1}, [%2];"
+                     : "=r"(b0), "=r"(b1)
+                     : "r"(ba)
+                     : "memory");
+        mma_bf16(acc[k], a, b0, b1);
       }
     }
+    __syncthreads();  // the stage is free for the copies of the round after next
   }
   // rows g, g + 8 (output channels), columns 2t, 2t + 1 (input channels) of each tile
 #pragma unroll
@@ -1934,6 +2023,22 @@ __global__ void capture_kernel(const void* __restrict__ src, int form,
   }
 }
 
+int grid_for(int64_t items, int threads);
+
+int launch_syndrome(const uint8_t* N, int L, int64_t shots, uint8_t* sig, cudaStream_t st) {
+  const uintptr_t at = reinterpret_cast<uintptr_t>(N) | reinterpret_cast<uintptr_t>(sig);
+  if (L % 16 == 0 && at % 16 == 0) {
+    const int64_t vps = (int64_t)L * L / 16;
+    const dim3 grid((unsigned)std::min<int64_t>((vps + 255) / 256, 64),
+                    (unsigned)std::min<int64_t>(shots, 32768));
+    syndrome16_kernel<<<grid, (unsigned)std::min<int64_t>(256, ((vps + 31) / 32) * 32), 0, st>>>(
+        N, L, shots, sig);
+  } else {
+    syndrome_kernel<<<grid_for(shots * (int64_t)L * L, 256), 256, 0, st>>>(N, L, shots, sig);
+  }
+  return QCA_OK;
+}
+
 int grid_for(int64_t items, int threads) {
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
@@ -1943,6 +2048,68 @@ int grid_for(int64_t items, int threads) {
   if (b > cap) b = cap;
   return (int)(b < 1 ? 1 : b);
 }
+
+// Device buffers of one training batch of S sites.
+// Gradient reductions split the sites into at most kGradParts CTAs, a number
+// fixed by the batch size alone (not by the device), and add the CTAs' partial
+// sums in order.
+constexpr int kGradParts = 256;
+// columns of all sets of partial sums (the bias sums are 32 wide)
+constexpr int kGradPartCols = 9 * 32 * (4 + 32 + 32 + 2) + 4 * 32;
+
+struct TrainBufs {
+  int64_t S = 0;                   // sites of the batch
+  int64_t have = 0;                // sites the buffers hold
+  uint8_t* bytes = nullptr;        // sig, dir, lab
+  __nv_bfloat16* h = nullptr;      // x0, a1, a2, a3, dz, g1, g2: bf16 NHWC [S][32] each
+  float* z = nullptr;              // logits fp32 [B][4][L][L]
+  __nv_bfloat16* wt = nullptr;     // backward-data weights [3][9][32][32]
+  float* loss = nullptr;           // the loss and, after it, the count of labelled sites
+  float* part = nullptr;           // per-CTA gradient partial sums, all sets
+  uint8_t* sig() const { return bytes; }
+  uint8_t* dir() const { return bytes + S; }
+  uint8_t* lab() const { return bytes + 2 * S; }
+  __nv_bfloat16* act(int k) const { return h + (size_t)k * S * 32; }
+  // buffers for `sites` sites, kept if they are large enough
+  int alloc(int64_t sites) {
+    S = sites;
+    if (sites <= have) return QCA_OK;
+    release();
+    cudaError_t e = cudaMalloc(&bytes, 3 * S);
+    if (e == cudaSuccess) e = cudaMalloc(&h, sizeof(__nv_bfloat16) * 7 * 32 * S);
+    if (e == cudaSuccess) e = cudaMalloc(&z, sizeof(float) * 4 * S);
+    if (e == cudaSuccess) e = cudaMalloc(&wt, sizeof(__nv_bfloat16) * 3 * 9 * 32 * 32);
+    if (e == cudaSuccess) e = cudaMalloc(&part, sizeof(float) * kGradParts * kGradPartCols);
+    if (e == cudaSuccess) e = cudaMalloc(&loss, sizeof(float) + sizeof(unsigned int));
+    if (e != cudaSuccess) release();
+    have = e == cudaSuccess ? sites : 0;
+    return cuda_fail(e, "training buffers");
+  }
+  unsigned int* count() const { return reinterpret_cast<unsigned int*>(loss + 1); }
+  void release() {
+    cudaFree(bytes);
+    cudaFree(h);
+    cudaFree(z);
+    cudaFree(wt);
+    cudaFree(part);
+    cudaFree(loss);
+    bytes = nullptr;
+    h = nullptr;
+    z = nullptr;
+    wt = nullptr;
+    part = nullptr;
+    loss = nullptr;
+    have = 0;
+  }
+  TrainBufs() = default;
+  TrainBufs(const TrainBufs&) = delete;
+  TrainBufs& operator=(const TrainBufs&) = delete;
+  ~TrainBufs() { release(); }
+};
+
+// Most sites (about 490 bytes each) whose training buffers a net keeps from one
+// gradient call for the next: 1 GiB.
+constexpr int64_t kKeptSites = (int64_t)1 << 21;
 
 }  // namespace
 
@@ -1973,6 +2140,9 @@ struct qca_net_s {
   unsigned int* err = nullptr;   // device word: a tensor-core wait timed out
   __nv_bfloat16* lut = nullptr;  // layer-1 outputs per 3 x 3 anyon pattern [512][32]
   uint8_t* lut8 = nullptr;        // the same in e4m3 at the layer-1 activation scale
+  // buffers of qca_net_gradients, one call at a time
+  std::mutex grad_mu;
+  TrainBufs grad_bufs;
   // inference workspace
   uint8_t* ws = nullptr;
   size_t ws_bytes = 0;
@@ -2067,41 +2237,6 @@ int qca_net_set_params(qca_net_t n, const float* host, int64_t count) {
 
 namespace {
 
-// Device buffers of one training batch of S sites.
-// Gradient reductions split the sites into at most kGradParts CTAs, a number
-// fixed by the batch size alone (not by the device), and add the CTAs' partial
-// sums in order.
-constexpr int kGradParts = 256;
-
-struct TrainBufs {
-  int64_t S = 0;
-  uint8_t* bytes = nullptr;        // sig, dir, lab
-  __nv_bfloat16* h = nullptr;      // x0, a1, a2, a3, dz, g1, g2: bf16 NHWC [S][32] each
-  float* z = nullptr;              // logits fp32 [B][4][L][L]
-  __nv_bfloat16* wt = nullptr;     // backward-data weights [3][9][32][32]
-  float* part = nullptr;           // per-CTA gradient partial sums [kGradParts][9216]
-  uint8_t* sig() const { return bytes; }
-  uint8_t* dir() const { return bytes + S; }
-  uint8_t* lab() const { return bytes + 2 * S; }
-  __nv_bfloat16* act(int k) const { return h + (size_t)k * S * 32; }
-  int alloc(int64_t sites) {
-    S = sites;
-    cudaError_t e = cudaMalloc(&bytes, 3 * S);
-    if (e == cudaSuccess) e = cudaMalloc(&h, sizeof(__nv_bfloat16) * 7 * 32 * S);
-    if (e == cudaSuccess) e = cudaMalloc(&z, sizeof(float) * 4 * S);
-    if (e == cudaSuccess) e = cudaMalloc(&wt, sizeof(__nv_bfloat16) * 3 * 9 * 32 * 32);
-    if (e == cudaSuccess) e = cudaMalloc(&part, sizeof(float) * kGradParts * 9 * 32 * 32);
-    return cuda_fail(e, "training buffers");
-  }
-  ~TrainBufs() {
-    cudaFree(bytes);
-    cudaFree(h);
-    cudaFree(z);
-    cudaFree(wt);
-    cudaFree(part);
-  }
-};
-
 // Forward and backward of one batch whose syndromes (bufs.sig) and labels
 // (bufs.lab) are in place: n->grads receives the gradient of the mean
 // smoothed cross-entropy over the labelled sites, *loss that loss.
@@ -2116,9 +2251,27 @@ int train_forward_backward(qca_net_s* n, const TrainBufs& b, int L, int batch,
   chunk = ((chunk + kWgChunk - 1) / kWgChunk) * kWgChunk;
   const int gW = (int)((S + chunk - 1) / chunk);
   const int gB = (int)std::min<int64_t>(kGradParts, (S + 255) / 256);
-  auto reduce = [&](int nparts, int stride, int n, float* out) {
-    reduce_parts_kernel<<<(n + 255) / 256, 256>>>(b.part, nparts, stride, n, out);
+  // place of the next set of partial sums
+  GradSets sets;
+  int nsets = 0, total = 0;
+  int64_t at = 0;
+  auto place = [&](int nparts, int stride, int n, int to) {
+    sets.at[nsets] = at;
+    sets.parts[nsets] = nparts;
+    sets.stride[nsets] = stride;
+    sets.n[nsets] = n;
+    sets.to[nsets] = to;
+    ++nsets;
+    total += n;
+    float* p = b.part + at;
+    at += (int64_t)nparts * stride;
+    return p;
   };
+  for (auto kern : {wgrad_mma_kernel<4, 32>, wgrad_mma_kernel<32, 32>, wgrad_mma_kernel<32, 2>}) {
+    cudaError_t e =
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * kWgStage);
+    if (e != cudaSuccess) return cuda_fail(e, "weight gradient smem attribute");
+  }
   __nv_bfloat16 *x0 = b.act(0), *a1 = b.act(1), *a2 = b.act(2), *a3 = b.act(3), *dz = b.act(4),
                 *g1 = b.act(5), *g2 = b.act(6);
   // weights of this step: bf16 forward copies, mirrored backward copies
@@ -2136,29 +2289,26 @@ int train_forward_backward(qca_net_s* n, const TrainBufs& b, int L, int batch,
                                            nullptr, b.z, nullptr, nullptr, nullptr);
   loss_grad_nhwc_kernel<<<gS, 256>>>(b.z, b.lab(), L, batch, count, dz, loss);
   // backward: layer 4, 3, 2 (weights, bias, masked input gradient), layer 1
-  float* G = n->grads;
-  wgrad_mma_kernel<4, 32><<<gW, 256>>>(dz, a3, L, S, chunk, b.part);
-  reduce(gW, 4 * 32 * 9, 4 * 32 * 9, G + kW3);
-  bias_grad_kernel<4><<<gB, 256>>>(dz, S, b.part);
-  reduce(gB, 32, 4, G + kB3);
+  const size_t ws = 2 * kWgStage;
+  wgrad_mma_kernel<4, 32><<<gW, 256, ws>>>(dz, a3, L, S, chunk,
+                                           place(gW, 4 * 32 * 9, 4 * 32 * 9, kW3));
+  bias_grad_kernel<4><<<gB, 256>>>(dz, S, place(gB, 32, 4, kB3));
   conv_mma_kernel<4, kGradMasked><<<gm, 128>>>(dz, b.wt + 2 * 9 * 32 * 32, nullptr, L, batch, g1,
                                                nullptr, nullptr, nullptr, a3);
-  wgrad_mma_kernel<32, 32><<<gW, 256>>>(g1, a2, L, S, chunk, b.part);
-  reduce(gW, 32 * 32 * 9, 32 * 32 * 9, G + kW2);
-  bias_grad_kernel<32><<<gB, 256>>>(g1, S, b.part);
-  reduce(gB, 32, 32, G + kB2);
+  wgrad_mma_kernel<32, 32><<<gW, 256, ws>>>(g1, a2, L, S, chunk,
+                                            place(gW, 32 * 32 * 9, 32 * 32 * 9, kW2));
+  bias_grad_kernel<32><<<gB, 256>>>(g1, S, place(gB, 32, 32, kB2));
   conv_mma_kernel<4, kGradMasked><<<gm, 128>>>(g1, b.wt + 9 * 32 * 32, nullptr, L, batch, g2,
                                                nullptr, nullptr, nullptr, a2);
-  wgrad_mma_kernel<32, 32><<<gW, 256>>>(g2, a1, L, S, chunk, b.part);
-  reduce(gW, 32 * 32 * 9, 32 * 32 * 9, G + kW1);
-  bias_grad_kernel<32><<<gB, 256>>>(g2, S, b.part);
-  reduce(gB, 32, 32, G + kB1);
+  wgrad_mma_kernel<32, 32><<<gW, 256, ws>>>(g2, a1, L, S, chunk,
+                                            place(gW, 32 * 32 * 9, 32 * 32 * 9, kW1));
+  bias_grad_kernel<32><<<gB, 256>>>(g2, S, place(gB, 32, 32, kB1));
   conv_mma_kernel<4, kGradMasked><<<gm, 128>>>(g2, b.wt, nullptr, L, batch, g1, nullptr, nullptr,
                                                nullptr, a1);
-  wgrad_mma_kernel<32, 2><<<gW, 256>>>(g1, x0, L, S, chunk, b.part);
-  reduce(gW, 32 * 2 * 9, 32 * 2 * 9, G + kW0);
-  bias_grad_kernel<32><<<gB, 256>>>(g1, S, b.part);
-  reduce(gB, 32, 32, G + kB0);
+  wgrad_mma_kernel<32, 2><<<gW, 256, ws>>>(g1, x0, L, S, chunk,
+                                           place(gW, 32 * 2 * 9, 32 * 2 * 9, kW0));
+  bias_grad_kernel<32><<<gB, 256>>>(g1, S, place(gB, 32, 32, kB0));
+  reduce_parts_kernel<<<(total + 127) / 128, 128>>>(b.part, sets, total, n->grads);
   return cuda_fail(cudaGetLastError(), "training kernels");
 }
 
@@ -2233,34 +2383,27 @@ int qca_net_gradients(qca_net_t n, const uint8_t* noise, int L, int batch, float
     return QCA_ERR_ARG;
   }
   const int64_t S = (int64_t)batch * L * L;
-  TrainBufs b;
+  // allocating and freeing the buffers took as long as half the kernels, so the
+  // net keeps them, up to a bound
+  std::lock_guard<std::mutex> lk(n->grad_mu);
+  TrainBufs& b = n->grad_bufs;
   int rc = b.alloc(S);
   if (rc) return rc;
-  float* dl = nullptr;
-  unsigned int* cnt = nullptr;
-  cudaError_t e = cudaMalloc(&dl, sizeof(float));
-  if (e == cudaSuccess) e = cudaMalloc(&cnt, sizeof(unsigned int));
-  if (e == cudaSuccess) e = cudaMemset(dl, 0, sizeof(float));
-  if (e == cudaSuccess) e = cudaMemset(cnt, 0, sizeof(unsigned int));
-  if (e != cudaSuccess) {
-    cudaFree(dl);
-    cudaFree(cnt);
-    return cuda_fail(e, "qca_net_gradients allocation");
-  }
+  cudaError_t e = cudaMemsetAsync(b.loss, 0, sizeof(float) + sizeof(unsigned int), nullptr);
+  if (e != cudaSuccess) return cuda_fail(e, "qca_net_gradients");
   const int gS = grid_for(S, 256);
-  syndrome_kernel<<<gS, 256>>>(noise, L, batch, b.sig());
+  launch_syndrome(noise, L, batch, b.sig(), nullptr);
   first_dir_kernel<<<gS, 256>>>(b.sig(), L, batch, b.dir());
   mutual_label_kernel<<<gS, 256>>>(b.dir(), L, batch, b.lab());
-  count_labelled_kernel<<<gS, 256>>>(b.lab(), (int)S, cnt);
-  rc = train_forward_backward(n, b, L, batch, cnt, dl);
+  count_labelled_kernel<<<gS, 256>>>(b.lab(), (int)S, b.count());
+  rc = train_forward_backward(n, b, L, batch, b.count(), b.loss);
   if (rc == QCA_OK) rc = cuda_fail(cudaDeviceSynchronize(), "qca_net_gradients");
   if (rc == QCA_OK)
     rc = cuda_fail(cudaMemcpy(host_grads, n->grads, sizeof(float) * kParams, cudaMemcpyDeviceToHost),
                    "gradient copy");
   if (rc == QCA_OK && host_loss)
-    rc = cuda_fail(cudaMemcpy(host_loss, dl, sizeof(float), cudaMemcpyDeviceToHost), "loss copy");
-  cudaFree(dl);
-  cudaFree(cnt);
+    rc = cuda_fail(cudaMemcpy(host_loss, b.loss, sizeof(float), cudaMemcpyDeviceToHost), "loss copy");
+  if (b.have > kKeptSites) b.release();
   return rc;
 }
 
@@ -2275,7 +2418,7 @@ int qca_net_labels_async(const uint8_t* noise, int L, int64_t shots, uint8_t* ou
   const int64_t n = shots * (int64_t)L * L;
   uint8_t* sig = scratch;
   uint8_t* dir = scratch + n;
-  syndrome_kernel<<<grid_for(n, 256), 256, 0, st>>>(noise, L, shots, sig);
+  launch_syndrome(noise, L, shots, sig, st);
   first_dir_kernel<<<grid_for(n, 256), 256, 0, st>>>(sig, L, shots, dir);
   mutual_label_kernel<<<grid_for(n, 256), 256, 0, st>>>(dir, L, shots, out_labels);
   return cuda_fail(cudaGetLastError(), "label kernels");
@@ -2341,7 +2484,7 @@ int net_run(qca_net_s* n, const uint8_t* noise, int L, int64_t shots, float* log
         reinterpret_cast<__nv_bfloat16*>(n->ws + ((2 * S + 255) & ~(int64_t)255));
     __nv_bfloat16* actB = actA + S * 32;
     const uint8_t* Nc = noise + c0s * 2 * LL;
-    syndrome_kernel<<<grid_for(S, 256), 256, 0, st>>>(Nc, L, m, sig);
+    launch_syndrome(Nc, L, m, sig, st);
     const int64_t tiles = (S + 15) / 16;
     const int gm = grid_for(tiles * 32, 128);
     if (n->precision == 1 && n->use_tc == 2 && L % kTcM == 0 && L % kTcStrip == 0) {
