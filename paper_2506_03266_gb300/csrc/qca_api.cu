@@ -121,7 +121,7 @@ int launch_decode(const DecodeArgs& a, cudaStream_t stream) {
   // caller chose a kernel for the size
   if (!history_takes(a.L, a.v) || path_forced(a.L)) return launch_planes(a, stream);
   int rc = launch_history(a, stream);
-  if (rc || !history_may_leave_pending(a.L)) return rc;
+  if (rc || !history_may_leave_pending(a.L, a.shots)) return rc;
   DecodeArgs rest = a;
   rest.only_pending = 1;
   rest.queue = nullptr;

@@ -134,8 +134,10 @@ __device__ __forceinline__ uint32_t slice_limit(int m_max, int k) {
 
 // Slice k of the anyon at (x, y) by one thread, from the bitmap of sigma_{t-k}:
 // the (6k + 7) x (6k + 7) neighbourhood, a row window per row; needs 6k + 7 <=
-// 31 and <= L.  OPEN: rows and columns outside the lattice are empty.
-template <bool OPEN>
+// 31 and <= L.  OPEN: rows and columns outside the lattice are empty.  ROWS: rows
+// whose loads are in flight together (1 in shared memory, where short code is
+// worth more; 6 in global memory, whose latency it would otherwise pay per row).
+template <bool OPEN, int ROWS>
 __device__ __forceinline__ uint32_t slice_thread(const uint32_t* sig, int lws, int L, int x, int y,
                                                  int k) {
   const int wpr = 1 << lws;
@@ -167,8 +169,19 @@ __device__ __forceinline__ uint32_t slice_thread(const uint32_t* sig, int lws, i
   // |j| <= 3k + 1, 3k + 2, 3k + 3
   const uint32_t u3 = next(), u2 = next(), u1 = next();
   uint32_t v1 = u1;
+  int i = n - 6;  // 1 + 6k
+  if (ROWS > 1) {
 #pragma unroll 1
-  for (int i = 0; i < n - 6; ++i) v1 |= next();
+    for (; i >= ROWS; i -= ROWS) {
+      uint32_t v[ROWS];
+#pragma unroll
+      for (int q = 0; q < ROWS; ++q) v[q] = next();
+#pragma unroll
+      for (int q = 0; q < ROWS; ++q) v1 |= v[q];
+    }
+  }
+#pragma unroll 1
+  for (; i > 0; --i) v1 |= next();
   const uint32_t d1 = next(), d2 = next(), d3 = next();
   v1 |= d1;
   const uint32_t v2 = v1 | u2 | d2, v3 = v2 | u3 | d3;
@@ -474,6 +487,7 @@ struct Decoder {
   // tells apart
   static constexpr int kIdBits = LARGE ? 21 : 17;
   static constexpr int kEpochs = LARGE ? 1023 : 16383;
+  static constexpr int kRowsAhead = LARGE ? 4 : 2;  // rows of a strip in flight
 
   const DecodeArgs& a;
   const Geom& g;
@@ -597,10 +611,12 @@ struct Decoder {
       return 0;
     }
     int n = 0;
-#pragma unroll 2
-    for (int i = tid; i < n4; i += NT) {
+    uint32_t some = 0;  // which of this thread's groups hold anyons (at most 32 of them)
+#pragma unroll 4
+    for (int i = tid, q = 0; i < n4; i += NT, ++q) {
       const uint4 v = cur[i];
       nxt[i] = v;
+      if (v.x | v.y | v.z | v.w) some |= 1u << q;
       n += __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w);
     }
     int pos = places(n);
@@ -608,9 +624,9 @@ struct Decoder {
       uint16_t* set = ar.sets + (LARGE ? 0 : (s % kArchiveSets) * ar.cap);
       const int wsm = (1 << g.lws) - 1;
 #pragma unroll 1
-      for (int i = tid; i < n4; i += NT) {
+      for (; some; some &= some - 1) {
+        const int i = tid + (__ffs(some) - 1) * NT;
         const uint4 v = cur[i];
-        if (!(v.x | v.y | v.z | v.w)) continue;
         const uint32_t q4[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -749,8 +765,14 @@ struct Decoder {
     const int last = min(t, g.kmax);
     const int lastt = min(min(last, g.kthread), t - oldest());
 #pragma unroll 1
-    for (int i0 = tid - lane; i0 < n; i0 += NT) {
-      const int i = i0 + lane;
+    for (int i0 = 0; i0 < n; i0 += NT) {
+      // a warp searches its far anyons one after the other: few anyons are spread
+      // over the warps (L = 256, p = 0.08: 6.8 -> 5.6 ms per 2000 shots), many are
+      // packed, so that fewer warps run the near slices (L = 256, p = 0.05: 4.9 ->
+      // 4.8 ms per 20 000 shots)
+      const bool spread = LARGE || n <= NT / 2;
+      const int i = i0 + (spread ? lane * (NT / 32) + warp : tid);
+      if (i0 + (spread ? warp : tid - lane) >= n) break;
       const bool act = i < n;
       int x = 0, y = 0, k = 0;
       uint32_t m = 0;
@@ -760,7 +782,7 @@ struct Decoder {
         y = e >> 16;
 #pragma unroll 1
         for (;; ++k) {
-          m = slice_thread<OPEN>(slot(t - k), g.lws, g.L, x, y, k) | edges(x, k);
+          m = slice_thread<OPEN, LARGE ? 6 : 1>(slot(t - k), g.lws, g.L, x, y, k) | edges(x, k);
           m &= slice_limit(a.m_max, k);
           if (m || k >= lastt) break;
         }
@@ -880,10 +902,12 @@ struct Decoder {
     uint32_t ul = from_left(u, p), ur = from_right(u, p);
     uint32_t cl = from_left(c, p), cr = from_right(c, p);
     uint32_t up = 0;  // +y moves of the row before
+    uint32_t ahead = row(y + 1);
     // one row more than the strip has: its -y moves cross the last row's links
 #pragma unroll 1
     for (int i = 0; i <= H; ++i, ++y) {
-      const uint32_t d = row(y + 1);
+      const uint32_t d = ahead;
+      if (i < H) ahead = row(y + 2);  // (loaded a row early)
       const uint32_t dl = from_left(d, p), dr = from_right(d, p);
       const uint32_t px = ul | cl | dl | first;  // anyon in column x - 1
       const uint32_t mx = ur | cr | dr | last;   // in column x + 1
@@ -965,7 +989,7 @@ struct Decoder {
       for (int y = p.y0; y < p.y1; ++y) sn[y << lws] = 0;
     }
     uint32_t fu = on ? fyp[wrap_lo(p.y0 - 1, g.L) << lws] : 0u;
-#pragma unroll 2
+#pragma unroll kRowsAhead
     for (int y = p.y0; y < p.y0 + H; ++y) {
       const bool in = on && y < p.y1;
       const int o = y << lws;
@@ -1198,6 +1222,7 @@ struct Decoder {
         const bool keep = t_kept < 0 && t >= due_kept;
         if (keep || t >= due_moving) {
           // (kFewRing entries cover the kmax + 1 <= 85 sets ending at t)
+          __syncwarp();  // every lane has compared with the snapshot it replaces
 #pragma unroll 1
           for (int i = lane; i < kFewRing * kWords; i += 32) {
             if (keep) snap[i] = now[i];
@@ -1258,7 +1283,7 @@ struct Decoder {
           uint32_t m = 0;
           const int k = kb + kk;
           if (kk < 2 && k <= lastt && ai < n && !hm)
-            m = (slice_thread<OPEN>(slot(t - k), g.lws, g.L, xa, ya, k) | edges(xa, k)) &
+            m = (slice_thread<OPEN, LARGE ? 6 : 1>(slot(t - k), g.lws, g.L, xa, ya, k) | edges(xa, k)) &
                 slice_limit(a.m_max, k);
           const uint32_t m0 = __shfl_sync(kFull, m, ai << lgS);
           const uint32_t m1 = __shfl_sync(kFull, m, (ai << lgS) + 1);
@@ -1435,8 +1460,11 @@ struct Decoder {
       }
     }
     n = total(n);
-    if (!LARGE && tid < 4 * (g.kmask + 1) && g.nws + (tid & 3) < g.nslot)
-      ring[(tid >> 2) * g.nslot + g.nws + (tid & 3)] = 0;  // the slots' last words
+    if (!LARGE && g.nws < g.nslot) {  // the slots' last words
+#pragma unroll 1
+      for (int i = tid; i < 4 * (g.kmask + 1); i += NT)
+        if (g.nws + (i & 3) < g.nslot) ring[(i >> 2) * g.nslot + g.nws + (i & 3)] = 0;
+    }
     int t = 0, flag = 0;
     bool listed = n <= g.sparse_max;
     if (listed || a.max_steps == 0) {  // else the first dense step writes it

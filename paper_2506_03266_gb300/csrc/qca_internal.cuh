@@ -160,7 +160,7 @@ bool four_cta_chosen(int L);
 // History sweep (v = 3, 8 <= L <= 1024): whether it takes the call, whether it
 // may leave shots pending (up to L = 256), and the launch.
 bool history_takes(int L, int v);
-bool history_may_leave_pending(int L);
+bool history_may_leave_pending(int L, int64_t shots);
 int launch_history(const DecodeArgs& a, cudaStream_t stream);
 // Open boundaries, default rules, v = 3, 8 <= L <= 256; may leave shots pending.
 int launch_history_open(const DecodeArgs& a, cudaStream_t stream);
