@@ -40,45 +40,29 @@ MAX_STEPS = 4096
 METRIC = "shot-decodes/s and site-updates/s at L=256,p=0.05 (plain vs net+CA, same p_log)"
 UNIT = "shot-decodes/s"
 
-# Integer-ALU roofline of the sweep: the fused
-# v = 3 message update costs 16 min/compare lane-ops per site-update (4 fields x
-# (3 two-input mins of the width-7 cone window + 1 clamp)); the ALU pipe issues
-# 64 32-bit instructions / clk / SM (qca_probe_peaks measures min.u16x2, lop3
-# and min.u32 all at this rate; reported as "probe"), each carrying
-# 2 16-bit lanes; 152 SMs at the 2070 MHz maximum SM clock.
-ALU_OPS_PER_SITE_UPDATE = 16
-ALU_PEAK_LANE_OPS = 152 * 64 * 2 * 2.070e9
+# Byte roofline of the decoders: a shot's links (or ring) are read once and its
+# correction, steps and flag written once; the state in between stays on chip or
+# in L2.  The peak is the measured copy bandwidth of the card.
+def hbm_roofline(nbytes, seconds, **more):
+    peak = 6800.0
+    try:
+        with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as f:
+            peak = float(json.load(f)["hbm_gbs"])
+    except (OSError, ValueError, KeyError):
+        pass
+    achieved = nbytes / seconds / 1e9
+    return dict({"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
+                 "frac": achieved / peak, "traffic": None,
+                 "note": "link bytes in, correction, steps and flags out, once each; the kernel "
+                         "is bound by instruction issue"}, **more)
 
-# Shared-memory roofline of the same sweep (the second fraction): with the
-# width-7 window in registers, a step reads and writes each of a site's four
-# field bytes once, 8 B per site-update, against 128 B/clk/SM.
-SMEM_BYTES_PER_SITE_UPDATE = 8
+
+# Shared-memory bandwidth, the bound of the literal desynchronised sweep.
 SMEM_PEAK = 152 * 128 * 2.070e9
 
 # A message grows by at most v = 3 per step, so the m_max = 255 cap can only act
 # on shots that run longer than this many steps.
 CAP_REACH_STEPS = (255 + 2) // 3
-
-# DRAM traffic of the dominant kernel per decoded shot at L = 256, p = 0.05
-# (dram__bytes_read.sum + dram__bytes_write.sum of one launch over 4000 shots,
-# profiles/fast_kernel_L256_p005_full.md), valid only for the kernel source
-# whose SHA-256 prefix is recorded with it; reported as null otherwise.
-TRAFFIC_PER_SHOT = {"sha256_prefixes": ("5e1dbd7f441ad48a",), "L": 256,
-                    "p": 0.05, "bytes_per_shot": (525.402112e6 + 479.698944e6) / 4000}
-
-
-def traffic_per_launch(L, p, shots):
-    import hashlib
-    src = os.path.join(ROOT, "paper_2506_03266_gb300", "csrc", "qca_sweep_fast.cu")
-    try:
-        sha = hashlib.sha256(open(src, "rb").read()).hexdigest()[:16]
-    except OSError:
-        return None
-    t = TRAFFIC_PER_SHOT
-    if sha not in t["sha256_prefixes"] or L != t["L"] or p != t["p"]:
-        return None
-    return t["bytes_per_shot"] * shots
-
 
 def executed_site_updates(steps, flags, L):
     """Site-updates the sweep executed: the sum of steps x L^2 over the shots
@@ -357,12 +341,11 @@ def run_uneven(args, rank, world, local):
     del C_default
     site_updates = executed_site_updates(steps_h, fail_h, L_s)
     value = shots / (ms_per_step / 1e3)
-    achieved = ALU_OPS_PER_SITE_UPDATE * site_updates / (ms_per_step / 1e3)
     per_size = {int(s): {"shots": int((L_s == s).sum()),
                          "p_log": float((fail_h[L_s == s] > 0).mean()),
                          "mean_steps": float(steps_h[L_s == s].mean())} for s in np.unique(L_s)}
     line = {
-        "metric": "shot-decodes/s (uneven batch of mixed L, one persistent launch, "
+        "metric": "shot-decodes/s (uneven batch of mixed L, one launch per CTA shape, "
                   "one CUDA-graph replay per step)",
         "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": ms_per_step, "higher_is_better": True,
@@ -377,11 +360,11 @@ def run_uneven(args, rank, world, local):
                               "ms_per_step": per_size_ms, "identical_outputs": same,
                               "note": "one persistent launch per size on forked streams, "
                                       "same noise, not graph-captured"},
-        "roofline": {"bound": "alu", "achieved": achieved / 1e9,
-                     "peak": ALU_PEAK_LANE_OPS / 1e9, "unit": "Glane-op/s",
-                     "frac": achieved / ALU_PEAK_LANE_OPS, "traffic": None},
+        "roofline": hbm_roofline(4 * float(np.sum(L_s.astype(np.float64) ** 2)) + 5 * shots,
+                                 ms_per_step / 1e3),
         "clocks": clk,
-        "gpu_launches": args.steps,  # one mixed-size sweep launch per step
+        # a launch per CTA shape (two) and one for shots left pending
+        "gpu_launches": 3 * args.steps,
     }
     if rank == 0:
         print(json.dumps(line), flush=True)
@@ -664,7 +647,6 @@ def run_large(args, rank, world, local):
         return
     ms_per_step = timed["ms_per_step"]
     kernel_s = statistics.mean(timed["kernel_ms"]) / 1e3
-    achieved = ALU_OPS_PER_SITE_UPDATE * site_updates / kernel_s
     line = {
         "metric": "shot-decodes/s of the plain automaton at L=1024, p=0.05 (large-lattice "
                   "kernel), with the FP8 net + automaton compared at p=0.05 and 0.07",
@@ -683,9 +665,8 @@ def run_large(args, rank, world, local):
                              "final_loss": float(np.mean(losses[-50:]))},
                    "fp8_activation_scales": [float(x) for x in scales]},
         "comparison": results,
-        "roofline": {"bound": "alu", "achieved": achieved / 1e9, "peak": ALU_PEAK_LANE_OPS / 1e9,
-                     "unit": "Glane-op/s", "frac": achieved / ALU_PEAK_LANE_OPS, "traffic": None,
-                     "kernel_ms": statistics.mean(timed["kernel_ms"])},
+        "roofline": hbm_roofline((4 * L * L + 5) * shots, kernel_s,
+                                 kernel_ms=statistics.mean(timed["kernel_ms"])),
         "clocks": timed["clocks"],
         "gpu_launches": args.steps,
         "e2e": None,
@@ -702,8 +683,6 @@ def run_large(args, rank, world, local):
 # (syndrome byte, move byte; the fields are still in registers), feedback (two
 # move bytes, flip byte, correction read/write) and the syndrome update (two
 # flip bytes, syndrome read/write).
-SMEM_BYTES_PER_SITE_UPDATE_1D = 21
-SMEM_PEAK_BYTES = 152 * 128 * 2.070e9  # 128 B/clk/SM at the maximum SM clock
 
 
 def run_1d(args, rank, world, local):
@@ -773,7 +752,6 @@ def run_1d(args, rank, world, local):
             dist.destroy_process_group()
         return
     kernel_s = statistics.mean(kernel_ms) / 1e3
-    achieved = SMEM_BYTES_PER_SITE_UPDATE_1D * site_updates / kernel_s
     line = {
         "metric": "shot-decodes/s of the 1D repetition-code automaton (L=1024, p=0.3, "
                   "10 % random moves)",
@@ -792,10 +770,7 @@ def run_1d(args, rank, world, local):
                     "mean_steps": float(steps_h.mean()),
                     "p99_steps": float(np.percentile(steps_h, 99)),
                     "tdec_vs_L": tdec},
-        "roofline": {"bound": "smem", "achieved": achieved / 1e9, "peak": SMEM_PEAK_BYTES / 1e9,
-                     "unit": "GB/s", "frac": achieved / SMEM_PEAK_BYTES, "traffic": None,
-                     "note": f"{SMEM_BYTES_PER_SITE_UPDATE_1D} shared-memory bytes per "
-                             "site-update against 128 B/clk/SM"},
+        "roofline": hbm_roofline((2 * L + 6) * shots, ms_per_step / 1e3),
         "clocks": clk, "gpu_launches": args.steps, "e2e": None, "cpu_baseline": None,
     }
     print(json.dumps(line), flush=True)
@@ -892,13 +867,14 @@ def run_variant(args, rank, world, local):
                    "L": L, "p": p, "shots_per_gpu": shots,
                    "l2": "each CTA's state slot is reused across its shots"},
         "decoder": stats,
-        "roofline": {"bound": "smem", "achieved": smem_achieved / 1e9, "peak": SMEM_PEAK / 1e9,
-                     "unit": "GB/s", "frac": smem_achieved / SMEM_PEAK, "traffic": None,
-                     "note": (f"{per_unit} shared-memory bytes per site-"
-                              f"{'update' if open_ else 'tick'}: each message sub-step reads and "
-                              "writes a site's four field bytes once; literal per-site kernel, "
-                              "one launch per step")},
-        "clocks": clk, "gpu_launches": args.steps, "e2e": None, "cpu_baseline": None,
+        "roofline": hbm_roofline((4 * L * L + 5) * shots, ms_per_step / 1e3) if open_ else {
+            "bound": "smem", "achieved": smem_achieved / 1e9, "peak": SMEM_PEAK / 1e9,
+            "unit": "GB/s", "frac": smem_achieved / SMEM_PEAK, "traffic": None,
+            "note": f"{per_unit} shared-memory bytes per site-tick: a message sub-step reads and "
+                    "writes a site's four field bytes once; literal per-site kernel"},
+        # open: the decode and the look for shots left pending
+        "clocks": clk, "gpu_launches": (2 if open_ else 1) * args.steps, "e2e": None,
+        "cpu_baseline": None,
     }
     print(json.dumps(line), flush=True)
     if dist is not None:
@@ -980,12 +956,9 @@ def run_sweep(args, rank, world, local):
                    "shots_per_point": shots,
                    "l2": "each point's input is read once per decode; L >= 64 inputs exceed L2"},
         "points": points,
-        "roofline": {"bound": "alu",
-                     "achieved": ALU_OPS_PER_SITE_UPDATE * tot_su / (tot_ms / 1e3) / 1e9,
-                     "peak": ALU_PEAK_LANE_OPS / 1e9, "unit": "Glane-op/s",
-                     "frac": ALU_OPS_PER_SITE_UPDATE * tot_su / (tot_ms / 1e3) / ALU_PEAK_LANE_OPS,
-                     "traffic": None},
-        "clocks": clk, "gpu_launches": len(points), "e2e": None, "cpu_baseline": None,
+        "roofline": hbm_roofline(sum((4 * q["L"] ** 2 + 5) * shots for q in points),
+                                 tot_ms / 1e3),
+        "clocks": clk, "gpu_launches": 2 * len(points), "e2e": None, "cpu_baseline": None,
     }
     print(json.dumps(line), flush=True)
     if dist is not None:
@@ -1138,7 +1111,8 @@ def main():
     clk = clocks.stop()
     total_ms = t_start.elapsed_time(t_end)
     kernel_ms = [a.elapsed_time(b) for a, b in evs]
-    launches = args.steps  # one sweep-kernel launch per decode call
+    # per call: the decode and, up to L = 256, the look for shots left pending
+    launches = args.steps * (2 if 8 <= L <= 256 else 1)
 
     steps_h = steps.cpu()
     fail_h = fail.cpu()
@@ -1262,15 +1236,6 @@ def main():
         return
 
     kernel_s = statistics.mean(kernel_ms) / 1e3
-    achieved = ALU_OPS_PER_SITE_UPDATE * site_updates / kernel_s
-    # the two denominators measured on this device (untimed, after the timed
-    # region): min.u16x2 issue rate and shared-memory load bandwidth
-    pk = qca.probe_peaks()
-    smem_achieved = SMEM_BYTES_PER_SITE_UPDATE * site_updates / kernel_s
-    probe = dict(pk, frac_alu_of_probe=achieved / pk["min16x2_lane_ops_per_s"],
-                 frac_smem_of_probe=smem_achieved / pk["smem_bytes_per_s"],
-                 note="microbenchmarks of the roofline denominators (qca_probe_peaks); "
-                      "roofline.peak stays the value derived from unit counts and clock")
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": ms_per_step, "higher_is_better": True,
@@ -1283,17 +1248,8 @@ def main():
                     "p99_steps": float(torch.quantile(steps_h.float(), 0.99)),
                     "max_steps_seen": int(steps_h.max()),
                     "shots_beyond_cap_reach": int((steps_h > CAP_REACH_STEPS).sum())},
-        "roofline": {"bound": "alu", "achieved": achieved / 1e9, "peak": ALU_PEAK_LANE_OPS / 1e9,
-                     "unit": "Glane-op/s", "frac": achieved / ALU_PEAK_LANE_OPS,
-                     "traffic": traffic_per_launch(L, args.p, shots),
-                     "kernel_ms": statistics.mean(kernel_ms)},
-        "roofline_smem": {"bound": "smem",
-                          "achieved": smem_achieved / 1e9,
-                          "peak": SMEM_PEAK / 1e9, "unit": "GB/s",
-                          "frac": smem_achieved / SMEM_PEAK,
-                          "note": "second fraction of the same kernel: 8 B of shared memory "
-                                  "per site-update; the ALU fraction is the higher, binding one"},
-        "probe": probe,
+        "roofline": hbm_roofline((4 * L * L + 5) * shots, kernel_s,
+                                 kernel_ms=statistics.mean(kernel_ms)),
         "clocks": clk,
         "gpu_launches": launches,
         "e2e": e2e,
