@@ -230,8 +230,8 @@ typedef struct qca_uneven_plan_s* qca_uneven_plan_t;
 int qca_uneven_plan_create(const int32_t* L_host, int64_t shots, int64_t* offsets_host,
                            int64_t* total_bytes, qca_uneven_plan_t* out_plan);
 int qca_uneven_plan_destroy(qca_uneven_plan_t plan);
-/* Launch form of qca_decode_uneven_async for this plan: 0 (default) one
- * mixed-size persistent launch, 1 one persistent launch per size. */
+/* Launch form of qca_decode_uneven_async for this plan: 0 (default) launches over
+ * many sizes at once, 1 launches per size. */
 int qca_uneven_plan_set_mode(qca_uneven_plan_t plan, int mode);
 /* Device array of the plan's block offsets (int64 [shots]), owned by the plan. */
 int qca_uneven_plan_offsets_device(qca_uneven_plan_t plan, const int64_t** offsets_device);
@@ -244,22 +244,13 @@ int qca_sample_errors_uneven_async(const int32_t* L_dev, const int64_t* offsets_
                                    uint8_t* out_errors, void* stream);
 
 /* Decode a packed uneven batch.  Default (mode 0 of qca_uneven_plan_set_mode):
- * one persistent launch for the shots of every size the on-chip sweep takes
- * (multiples of 4 up to 128 and of 8 up to 256, blocks on a 4-byte boundary;
- * the 8 largest such sizes), queued pairs first, then by group size, then
- * largest L first.
- * Clusters of two CTAs take the shots with L > 192; every other size is
- * decoded by a group of 512, 256 or 128 threads (the smallest that fits), a
- * 512-thread CTA halving into up to four groups as the queue reaches smaller
- * sizes; each takes its next shot when the last one is done (work stealing
- * across sizes; every shot retires after its own number of steps); shots of
- * other sizes go to per-size launches on streams forked from `stream` before
- * it, which run beside it.  Mode 1: one persistent launch per
- * size, each on a stream forked from and joined to `stream`, so that the sizes
- * run side by side.  Only kernel launches, memset and
- * event operations are enqueued, so the call can be captured in a CUDA graph
- * once one uncaptured call has sized the library's workspaces.  Outputs are
- * bit-identical to decoding each shot with qca_decode_batch in either mode. */
+ * with v = 3, one launch for all sizes from 8 to 64, one for all from 65 to 256
+ * (odd ones included, shots of the largest size first), and one that decodes the
+ * shots these left pending (usually none); other sizes and speeds go to launches
+ * per size on streams forked from `stream` and joined back to it, which run
+ * beside them.  Mode 1: launches per size for every size.  The outputs are the
+ * same in both modes, and both can be captured in a CUDA graph.  Calls of one
+ * plan that overlap on the GPU race on its work counters. */
 int qca_decode_uneven_async(qca_uneven_plan_t plan, const uint8_t* errors, int max_steps,
                             uint64_t rng_seed, uint8_t* out_correction, int32_t* out_steps,
                             uint8_t* out_logical_fail, const qca_config* cfg, void* stream);
@@ -519,7 +510,10 @@ int qca_net_decode_batch_async(qca_net_t net, const uint8_t* noise, int L, int64
                                int32_t* out_steps, uint8_t* out_logical_fail,
                                const qca_config* cfg, uint8_t* residual_scratch, void* stream);
 
-/* Kernel path chosen for a lattice size: 1 = on-chip fast sweep, 2 = on-chip
+/* Kernel path with stored message fields for a lattice size.  (With v = 3 and L
+ * from 8 up a decode runs from the syndrome history instead, and this path takes
+ * the shots that need a syndrome older than it keeps; a path chosen with
+ * qca_set_kernel_path takes the whole call.)  1 = on-chip fast sweep, 2 = on-chip
  * sweep on a 2-CTA cluster, 3 = large-lattice sweep (8-CTA cluster per shot,
  * state in global memory, bulk-copy staged bands; L a multiple of 128, chosen
  * automatically above 256), 0 = generic sweep with HBM-resident state.

@@ -2,15 +2,13 @@
 //
 // A plan groups the shots by L once (host side) and keeps on the device the
 // shot lists, the byte offsets of every shot's [2][L][L] block in the packed
-// input, and the work counters.  A decode makes one persistent launch of the
-// mixed-size on-chip kernel over every shot whose size it takes (a single
-// queue, largest L first, work stealing across sizes, each shot retiring on
-// its own step count).  Shots of other sizes (or packed off a 4-byte boundary)
-// go to per-size persistent launches of their own kernel on side streams
-// forked from and joined back to the caller's stream (beside the mixed-size
-// launch, which has no dependence on them), and that per-size form
-// can also be chosen for every size (qca_uneven_plan_set_mode).  Either way
-// the decode can be captured in one CUDA graph.
+// input, and the work counters.  A decode (v = 3) makes one launch of the history
+// sweep over all sizes that share a CTA shape, largest L first, and one of the
+// mixed-size on-chip sweep for the shots it left pending (usually none).  Sizes
+// above 256 and below 8, other speeds, and, in the per-size form
+// (qca_uneven_plan_set_mode), every size go to launches of their own on side
+// streams forked from and joined back to the caller's stream.  Either way the
+// decode can be captured in one CUDA graph.
 #include <math.h>
 #include <stdlib.h>
 #include <string.h>
