@@ -91,80 +91,6 @@ __global__ void __launch_bounds__(NT, NT == 32 ? 24 : 768 / NT)
   d.run();
 }
 
-// Threads per shot: a warp up to L = 64 (no block barriers).  Above, four warps:
-// the steps with few anyons leave most of a larger CTA idle, so more and smaller
-// CTAs per SM are better (L = 256: 256 threads 5.4 ms per 20 000 shots at three
-// CTAs per SM, 128 threads at the same three 6.3 ms, at six 4.8 ms).  What lets
-// six fit at L = 256 is keeping the correction and the dense steps' link maps in
-// the shot's (L2-resident) correction block instead of shared memory.
-int threads_for(int L) { return L <= 64 ? 32 : (L <= 256 ? 128 : 1024); }
-
-// Whether a small batch of small lattices keeps all 85 syndromes in shared memory
-// (128 slots, 21 KB at L = 32): the shots are all resident anyway, and the call
-// then has no second launch for pending shots (64 shots of L = 16: 30.7 -> 26.7 us
-// per call on the device).
-constexpr int kAllSlotsL = 32, kAllSlotsShots = 1024;
-bool all_slots(int L, int64_t shots) { return L <= kAllSlotsL && shots <= kAllSlotsShots; }
-
-bool make_hist_geom(int L, int m_max, Geom& g, int& threads, size_t& smem, size_t& slot_words,
-                    bool all = false) {
-  if (L < 8 || L > QCA_MAX_L) return false;
-  const bool large = L > 256;
-  threads = threads_for(L);
-  g.L = L;
-  const int wpr = (L + 31) / 32;
-  g.lws = 0;
-  while ((1 << g.lws) < wpr) ++g.lws;
-  g.nws = L << g.lws;
-  g.nslot = (g.nws + 3) & ~3;
-  g.kmax = (m_max - 1) / 3;
-  g.kthread = std::min(4, (L - 7) / 6);
-  const int K = all ? 128 : (L <= 128 ? 8 : 4);
-  g.kmask = K - 1;
-  g.spill = g.kmax > K - 2;
-  g.c_global = !large && L > 128;
-  // a dense pass costs about as much as searching half an anyon per word (L = 32,
-  // p = 0.06: 0.80 ms per 20 000 shots, 0.87 at a quarter); above L = 128 the
-  // smaller list and crossing table let one more CTA fit (L = 256: 4.8 against
-  // 5.8 ms)
-  g.sparse_max = std::max(kFew, L <= 128 ? g.nws / 2 : g.nws / 4);
-  if (large) g.sparse_max = std::min(g.sparse_max, 4096);
-  g.list_cap = g.sparse_max;
-  int tsize = 1;
-  while (tsize < g.sparse_max) tsize *= 2;
-  g.tmask = tsize - 1;
-  const int few = large ? kFewWords<true> : kFewWords<false>;
-  // the crossing table and the few-anyon mode's sets are never in use at once
-  int o = 0, region = std::max(few, tsize);
-  if (large) {
-    g.o_C = kLargeRing * g.nws;
-    g.o_F = g.o_C + 2 * g.nws;
-    slot_words = (size_t)g.o_F + 2 * g.nws;
-  } else {
-    o = K * g.nslot;
-    g.o_C = g.o_F = 0;
-    if (!g.c_global) {
-      g.o_C = o;
-      o = (o + 2 * g.nws + 3) & ~3;
-    }
-    slot_words = 0;
-  }
-  g.o_table = g.o_few = o;
-  o += (region + 3) & ~3;
-  // the snapshots are taken when the bitmaps are no longer needed
-  if (!large && K * g.nslot >= 2 * few) {
-    g.o_snap = 0;
-  } else {
-    g.o_snap = o;
-    o += 2 * few;
-  }
-  g.o_list = o;
-  o += g.list_cap;
-  g.o_misc = o;
-  smem = (size_t)(o + 8 + 64) * 4;  // counters, archived set sizes
-  return true;
-}
-
 // Shared-memory allowance of one kernel, raised once per device.
 template <class K>
 int allow_smem(K kern, size_t smem, std::atomic<int> (&have)[64], int dev) {

@@ -1,0 +1,55 @@
+"""The history decoder's device code run on the CPU, lane by lane in a drawn
+order, against the oracle: whole outputs, and no lane of a warp or block left
+behind at a collective.  A shot it leaves pending is not compared."""
+import shutil
+
+import numpy as np
+import pytest
+
+import history_emulation as emu
+import oracle
+
+pytestmark = pytest.mark.skipif(shutil.which("g++") is None, reason="no host compiler")
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    oracle.build()
+
+
+def compare_noise(N, **kw):
+    """Decodes noise; every shot that is not pending equals the oracle's.  Returns
+    the number of pending shots."""
+    okw = dict(max_steps=kw.get("max_steps", 400), m_max=kw.get("m_max", 255),
+               move_thr=kw.get("move_thr", 0), seed=kw.get("seed", 0), tie_order=kw.get("tie", 0),
+               balance_rule=kw.get("bal", 0))
+    C, s, f = emu.decode(N, **kw)
+    Co, so, fo = oracle.decode_batch(N, **okw)
+    done = s != emu.PENDING
+    np.testing.assert_array_equal(s[done], so[done])
+    np.testing.assert_array_equal(f[done], fo[done])
+    np.testing.assert_array_equal(C[done], Co[done])
+    return int((~done).sum())
+
+
+def compare_sigma(s, **kw):
+    C, st, ex = emu.decode(s[None], sigma=True, **kw)
+    if st[0] == emu.PENDING:
+        return 1
+    Co, so, fo = oracle.decode_syndrome_shot(s, max_steps=kw.get("max_steps", 400),
+                                             m_max=kw.get("m_max", 255),
+                                             tie_order=kw.get("tie", 0))[:3]
+    assert (int(st[0]), bool(ex[0])) == (so, fo == 2)
+    np.testing.assert_array_equal(C[0], Co)
+    return 0
+
+
+@pytest.mark.parametrize("L,p,shots", [(8, .15, 20), (16, .08, 20), (33, .08, 5), (64, .07, 4),
+                                       (65, .07, 2), (128, .05, 1), (200, .04, 1)])
+def test_noise_against_oracle(L, p, shots):
+    N = oracle.sample_errors(L, shots, p, seed=L)
+    thr = oracle.prob_threshold(0.1)
+    for kw in (dict(), dict(tie=1), dict(bal=1, seed=4), dict(move_thr=thr, tie=1, seed=5)):
+        compare_noise(N, max_steps=150, skew=L % 3, order=L, **kw)
+    if L <= 32:
+        compare_noise(N, max_steps=150, all_slots=True)
