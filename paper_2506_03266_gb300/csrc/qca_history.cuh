@@ -97,8 +97,10 @@ inline bool make_hist_geom(int L, int m_max, Geom& g, int& threads, size_t& smem
   g.kthread = std::min(4, (L - 7) / 6);
   const int K = all ? 128 : (L <= 128 ? 8 : 4);
   g.kmask = K - 1;
-  g.spill = g.kmax > K - 2;
   g.c_global = !large && L > 128;
+  // a listed step t gives up one slot, for sigma_{t+1}, and keeps slices 0 to K - 2;
+  // a dense one whose link maps are in slots gives up two more
+  g.spill = g.kmax > (g.c_global ? K - 2 : K - 4);
   // a dense pass costs about as much as searching half an anyon per word (L = 32,
   // p = 0.06: 0.80 ms per 20 000 shots, 0.87 at a quarter); above L = 128 the
   // smaller list and crossing table let one more CTA fit (L = 256: 4.8 against
@@ -746,7 +748,7 @@ struct Decoder {
       sig = slot(s);
     } else if (nset[s & 127] != kNoSet) {
       m = slice_list<OPEN>(ar.sets + (s % kArchiveSets) * ar.cap, nset[s & 127], g.L, x, y, k, lane);
-    } else if (s >= ar.gone - ar.nb) {
+    } else if (s < ar.gone && s >= ar.gone - ar.nb) {
       sig = ar.bitmaps + (s % ar.nb) * g.nws;
     } else {
       misc[3] = 1;  // the shot needs a syndrome that is no longer kept

@@ -8,6 +8,7 @@ import pytest
 
 import history_emulation as emu
 import oracle
+from history_states import open_noise_of, patch_and_far
 
 pytestmark = pytest.mark.skipif(shutil.which("g++") is None, reason="no host compiler")
 
@@ -53,3 +54,19 @@ def test_noise_against_oracle(L, p, shots):
         compare_noise(N, max_steps=150, skew=L % 3, order=L, **kw)
     if L <= 32:
         compare_noise(N, max_steps=150, all_slots=True)
+
+
+@pytest.mark.parametrize("L", [64, 96, 128])
+@pytest.mark.parametrize("m_max", [15, 16, 18, 19, 21, 22])
+def test_caps_around_the_slots(L, m_max):
+    """Caps whose oldest slice is about the oldest syndrome that dense and listed
+    steps keep in slots; the correction holds 0xFF before."""
+    rng = np.random.default_rng(100 * L + m_max)
+    for i in range(6):
+        s = patch_and_far(L, rng, 1 + i % 5)
+        compare_sigma(s, max_steps=70, m_max=m_max, tie=i & 1, order=i)
+    N = open_noise_of(patch_and_far(L, rng, 4))
+    C, st, f = emu.decode(N[None], max_steps=40, m_max=m_max, open=True)
+    Co, so, fo = oracle.open_decode_shot(N, max_steps=40, m_max=m_max)
+    assert (st[0], f[0]) == (so, fo)
+    np.testing.assert_array_equal(C[0], Co)
