@@ -764,7 +764,8 @@ struct Decoder {
 #pragma unroll 1
     for (; k <= last; ++k) {
       m = far_slice(x, y, t, k);
-      if (m || (!LARGE && misc[3])) break;
+      // (other warps set the flag at any time: one vote, so that the warp stays together)
+      if (m || (!LARGE && __any_sync(kFull, *(volatile int*)&misc[3]))) break;
     }
     return m;
   }

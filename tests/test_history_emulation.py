@@ -70,3 +70,12 @@ def test_caps_around_the_slots(L, m_max):
     Co, so, fo = oracle.open_decode_shot(N, max_steps=40, m_max=m_max)
     assert (st[0], f[0]) == (so, fo)
     np.testing.assert_array_equal(C[0], Co)
+
+
+@pytest.mark.parametrize("L,far,tie,seed", [(192, 6, 1, 2), (192, 80, 0, 1), (229, 20, 0, 2),
+                                            (256, 20, 1, 1)])
+def test_warps_stay_together_when_a_shot_is_left(L, far, tie, seed):
+    """One warp finds that a syndrome is no longer kept while others search."""
+    s = patch_and_far(L, np.random.default_rng(seed), far)
+    for order in range(10):
+        assert compare_sigma(s, max_steps=130, tie=tie, order=1000 + 17 * order) == 1
