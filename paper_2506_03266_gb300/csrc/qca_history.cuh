@@ -38,8 +38,9 @@ namespace hist {
 
 constexpr int kFew = 8;        // most anyons of the few-anyon mode
 constexpr int kFewRing = 128;  // steps of anyon sets it keeps (more than 85)
-constexpr int kArchiveSets = 86;  // steps of archived sets (more than 85)
-constexpr uint16_t kNoSet = 0xFFFF;
+constexpr int kSteps = 128;    // steps whose place in the archive is known (more than 85)
+// what the archive holds of a step, if not a list of so many anyons
+constexpr uint16_t kNotKept = 0xFFFF, kBitmap = 0xFFFE;
 constexpr int kLargeRing = 88; // syndromes kept per shot above L = 256 (more than 85)
 constexpr uint32_t kFull = 0xffffffffu;
 
@@ -51,7 +52,8 @@ struct Geom {
   int kmask;       // syndromes kept in shared memory, less one (a power of two less one)
   int spill;       // whether syndromes older than those are needed at all
   int kthread;     // oldest slice a single thread can search: min(4, (L - 7) / 6)
-  int c_global;    // correction and link maps are kept in the correction block
+  int c_global;    // the correction is kept in the correction block
+  int f_global;    // and so are the dense steps' link maps
   int kmax;        // oldest slice a message can come from: (m_max - 1) / 3
   int sparse_max;  // most anyons of the listed mode
   int list_cap;    // entries of the anyon list
@@ -97,10 +99,12 @@ inline bool make_hist_geom(int L, int m_max, Geom& g, int& threads, size_t& smem
   g.kthread = std::min(4, (L - 7) / 6);
   const int K = all ? 128 : (L <= 128 ? 8 : 4);
   g.kmask = K - 1;
-  g.c_global = !large && L > 128;
+  // (up to L = 176 six CTAs per SM fit with the correction in shared memory too)
+  g.c_global = !large && L > 176;
+  g.f_global = !large && L > 128;
   // a listed step t gives up one slot, for sigma_{t+1}, and keeps slices 0 to K - 2;
   // a dense one whose link maps are in slots gives up two more
-  g.spill = g.kmax > (g.c_global ? K - 2 : K - 4);
+  g.spill = g.kmax > (g.f_global ? K - 2 : K - 4);
   // a dense pass costs about as much as searching half an anyon per word (L = 32,
   // p = 0.06: 0.80 ms per 20 000 shots, 0.87 at a quarter); above L = 128 the
   // smaller list and crossing table let one more CTA fit (L = 256: 4.8 against
@@ -139,22 +143,27 @@ inline bool make_hist_geom(int L, int m_max, Geom& g, int& threads, size_t& smem
   g.o_list = o;
   o += g.list_cap;
   g.o_misc = o;
-  smem = (size_t)(o + 8 + 64) * 4;  // counters, archived set sizes
+  smem = (size_t)(o + 8 + kSteps) * 4;  // counters; archived sets' sizes and places
   return true;
 }
 
-// Syndromes that have left shared memory, in the shot's correction block (2 L^2
-// bytes, not written before the shot ends): a set of at most `cap` anyons as a
-// list of 16-bit sites, one place for each of the last 86 steps, taken when the
-// set is listed; a larger one as a bitmap, in a ring of nb places.  Anyons
-// never multiply, so the bitmaps are the first syndromes of the shot.  Blocks
-// too small for lists (L < 55) are all bitmaps.
+// Syndromes that have left shared memory, in the part of the shot's correction
+// block (2 L^2 bytes, not written before the shot ends) that the correction and
+// the link maps leave.  It is a ring of 4-byte words: a listed set is written to
+// it as a list of 16-bit sites when it is made, one that was never listed as a
+// bitmap (rows without padding) when it leaves its slot, each right after the one
+// before, over whatever is oldest.  Lists take what they need: of L = 144, p = 0.08,
+// whose sets have 5300, 2600, 1500, 850, 490, 310, 210, 170, 130, ... anyons, six
+// bitmaps and all lists since fit (24 of the 32 KB).  With a place of fixed size for
+// each of 86 lists, three quarters of such shots asked for a set that was gone.
+// A word of the ring always holds the last thing written to it, and whatever a new
+// entry covers is marked as not kept, so a search finds a set whole or not at all.
 struct Archive {
-  uint16_t* sets;     // [kArchiveSets][cap]
-  uint32_t* bitmaps;  // [nb][nws]
-  int cap, nb;
-  int gone;           // one more than the last bitmap's step
-  int next;           // syndromes moved so far
+  uint32_t* words;
+  int size;  // words of the ring
+  int head;  // next free word
+  int next;  // syndromes that have left their slot
+  uint32_t listed;  // bit i: the (i + 1)-th last step was archived as a list
 };
 
 __device__ __forceinline__ int wrap_lo(int i, int L) { return i < 0 ? i + L : i; }
@@ -283,14 +292,14 @@ __device__ __forceinline__ uint32_t slice_thread(const uint32_t* sig, int lws, i
   return m;
 }
 
-// Any slice of the anyon at (x, y) by a whole warp: a lane per row for the x
+// Any slice of the anyon at (x, y) by a whole warp, from a bitmap of wpr words per
+// row: a lane per row for the x
 // fields (three columns on either side), six lanes for the y fields' rows.  For
 // the far slices, which few anyons reach: a function of its own, since the
 // kernel is bound by instruction fetch when every use is a copy.
 template <bool OPEN>
-static __device__ __noinline__ uint32_t slice_warp(const uint32_t* sig, int lws, int L, int x, int y,
+static __device__ __noinline__ uint32_t slice_warp(const uint32_t* sig, int wpr, int L, int x, int y,
                                                int k, int lane) {
-  const int wpr = 1 << lws;
   const int r = 3 * k + 3;
   const int nrows = OPEN ? 2 * r + 1 : min(2 * r + 1, L);
   const int half = nrows == 2 * r + 1 ? r : (L - 1) >> 1;
@@ -301,7 +310,7 @@ static __device__ __noinline__ uint32_t slice_warp(const uint32_t* sig, int lws,
   for (int i = lane; i < nrows; i += 32) {
     const int j = i - half;
     if (OPEN && (unsigned)(y + j) >= (unsigned)L) continue;
-    const uint32_t* row = sig + (wrap_hi(wrap_lo(y + j, L), L) << lws);
+    const uint32_t* row = sig + wrap_hi(wrap_lo(y + j, L), L) * wpr;
     // d = 3, 2, 1 and d = 1, 2, 3
     const uint32_t l = OPEN ? (cl > -3 ? row_bits_clipped(row, wpr, L, cl, 3) : 0u)
                             : row_bits_wrapped(row, wpr, L, cl, 3);
@@ -319,7 +328,7 @@ static __device__ __noinline__ uint32_t slice_warp(const uint32_t* sig, int lws,
     int yy = lane < 3 ? y - dr : y + dr;
     if (!OPEN) yy = wrap_hi(wrap_lo(yy, L), L);
     if (!OPEN || (unsigned)yy < (unsigned)L)
-      m |= row_any<OPEN>(sig + (yy << lws), wpr, L, x, reach) << (4 * (d - 1) + (lane < 3 ? 2 : 3));
+      m |= row_any<OPEN>(sig + yy * wpr, wpr, L, x, reach) << (4 * (d - 1) + (lane < 3 ? 2 : 3));
   }
   return __reduce_or_sync(kFull, m);
 }
@@ -571,13 +580,15 @@ struct Decoder {
   const Geom& g;
   uint32_t* ring;    // [kmask + 1][nws] (LARGE: [kLargeRing][nws])
   uint32_t* C;       // [2][nws] correction
-  uint32_t* F;       // LARGE or c_global: [2][nws] links flipped in a dense step
+  uint32_t* F;       // LARGE or f_global: [2][nws] links flipped in a dense step
   uint32_t* list;    // [list_cap] anyons (y << 16 | x)
   uint32_t* table;   // [tmask + 1] links crossed toward an anyon in a listed step
   Ent* few;          // [kFewRing][kFew]
   uint32_t* snap;    // [2][kFewWords] snapshots of it
   int* misc;         // 0-2 rotating counters, 3 miss, 4 steps, 5 flag, 6-7 cuts
-  uint16_t* nset;    // [128] anyons in the archived set of a step, or kNoSet
+  uint16_t* nset;    // [kSteps] anyons in the archived list of a step, kBitmap or kNotKept
+  uint16_t* place;   // [kSteps] and its first word in the ring
+                     // (entry i of both is written by thread i mod NT alone)
   Archive ar;
   int64_t shot;
   int tid, lane, warp;
@@ -607,7 +618,7 @@ struct Decoder {
   __device__ __forceinline__ int oldest() const { return LARGE ? 0 : ar.next; }
   // x- / y-link map of dense step t: their own place, or the two slots with the
   // oldest syndromes
-  __device__ __forceinline__ bool maps_in_slots() const { return !LARGE && !g.c_global; }
+  __device__ __forceinline__ bool maps_in_slots() const { return !LARGE && !g.f_global; }
   __device__ __forceinline__ uint32_t* map_x(int t) const {
     return maps_in_slots() ? slot(t + 2) : F;
   }
@@ -656,12 +667,34 @@ struct Decoder {
     return __shfl_sync(kFull, base, 31) + incl - n;
   }
 
-  // Makes sigma_s (in its slot) the newest bitmap, and moves the syndrome in the
-  // slot of s + 1 to the archive, in a dense step perhaps also those in the slots
-  // of s + 2 and s + 3, which become the link maps.  listed: copies sigma_s to the
-  // slot of s + 1, where the moves will flip bits, and lists the anyons; returns
-  // their number.  Ends with a barrier.
-  __device__ __forceinline__ int advance(int s, bool listed) {
+  // Words of an archived bitmap, and of the ring's entry i.
+  __device__ __forceinline__ int bitmap_words() const { return g.L * ((g.L + 31) >> 5); }
+  __device__ __forceinline__ int entry_words(int i) const {
+    return nset[i] == kBitmap ? bitmap_words() : (nset[i] + 1) >> 1;
+  }
+  // First word of a new entry of at most n words (the ring has more); marks the
+  // entries that it covers.
+  __device__ __forceinline__ int reserve(int n) {
+    const int at = ar.head + n > ar.size ? 0 : ar.head;
+#pragma unroll 1
+    for (int i = tid; i < kSteps; i += NT)
+      if (nset[i] != kNotKept && place[i] < at + n && place[i] + entry_words(i) > at)
+        nset[i] = kNotKept;
+    return at;
+  }
+  // (by every thread: the one that owns the entry writes it)
+  __device__ __forceinline__ void record(int s, uint16_t what, int at) {
+    if (tid != (s & (kSteps - 1)) % NT) return;
+    nset[s & (kSteps - 1)] = what;
+    place[s & (kSteps - 1)] = (uint16_t)at;
+  }
+
+  // Makes sigma_s (in its slot), of at most n anyons, the newest bitmap, and moves
+  // the syndrome in the slot of s + 1 to the archive, in a dense step perhaps also
+  // those in the slots of s + 2 and s + 3, which become the link maps.  listed:
+  // copies sigma_s to the slot of s + 1, where the moves will flip bits, and lists
+  // the anyons; returns their number.  Ends with a barrier.
+  __device__ __forceinline__ int advance(int s, bool listed, int n) {
     const uint4* cur = reinterpret_cast<const uint4*>(slot(s));
     uint4* nxt = reinterpret_cast<uint4*>(slot(s + 1));
     const int n4 = g.nslot >> 2;
@@ -671,24 +704,31 @@ struct Decoder {
 #pragma unroll 1
       for (; ar.next < end; ++ar.next) {
         const int old = ar.next;
-        if (!g.spill || nset[old & 127] != kNoSet) continue;
-        // (the archive is on a 4-byte boundary)
-        uint32_t* to = ar.bitmaps + (old % ar.nb) * g.nws;
+        if (!g.spill || (ar.listed >> (s - 1 - old)) & 1u) continue;
+        const int at = reserve(bitmap_words());
+        uint32_t* to = ar.words + at;
         const uint32_t* from = slot(old);
+        const int wpr = (g.L + 31) >> 5, wsm = (1 << g.lws) - 1;
 #pragma unroll 2
-        for (int w = tid; w < g.nws; w += NT) to[w] = from[w];
-        ar.gone = old + 1;
+        for (int w = tid; w < g.nws; w += NT)
+          if ((w & wsm) < wpr) to[(w >> g.lws) * wpr + (w & wsm)] = from[w];
+        record(old, kBitmap, at);
+        ar.head = at + bitmap_words();
         any = true;
       }
       if (any) sync();
     }
     tb = s;
+    // a list where it is no longer than the bitmap
+    const bool keep = !LARGE && listed && g.spill && n <= 2 * bitmap_words();
+    if (!LARGE) ar.listed = ar.listed << 1 | (keep ? 1u : 0u);
     if (!listed) {
-      if (!LARGE && tid == 0) nset[s & 127] = kNoSet;
+      if (!LARGE) record(s, kNotKept, 0);
       sync();
       return 0;
     }
-    int n = 0;
+    const int at = keep ? reserve((n + 1) >> 1) : 0;
+    n = 0;
     uint32_t some = 0;  // which of this thread's groups hold anyons (at most 32 of them)
 #pragma unroll 4
     for (int i = tid, q = 0; i < n4; i += NT, ++q) {
@@ -699,7 +739,7 @@ struct Decoder {
     }
     int pos = places(n);
     if (n) {
-      uint16_t* set = ar.sets + (LARGE ? 0 : (s % kArchiveSets) * ar.cap);
+      uint16_t* set = reinterpret_cast<uint16_t*>(ar.words + at);
       const int wsm = (1 << g.lws) - 1;
 #pragma unroll 1
       for (; some; some &= some - 1) {
@@ -715,14 +755,18 @@ struct Decoder {
             const uint32_t e = yx + __ffs(b) - 1;
             b &= b - 1;
             list[pos] = e;
-            if (!LARGE && pos < ar.cap) set[pos] = (uint16_t)((e >> 8) | (e & 0xFFu));
+            if (keep) set[pos] = (uint16_t)((e >> 8) | (e & 0xFFu));
             ++pos;
           }
         }
       }
     }
     const int all = next_counter();
-    if (!LARGE && tid == 0) nset[s & 127] = all <= ar.cap ? (uint16_t)all : kNoSet;
+    if (!LARGE) {
+      // (read from the next step on)
+      record(s, keep ? (uint16_t)all : kNotKept, at);
+      if (keep) ar.head = at + ((all + 1) >> 1);
+    }
     return all;
   }
 
@@ -743,17 +787,23 @@ struct Decoder {
   __device__ __forceinline__ uint32_t far_slice(int x, int y, int t, int k) const {
     const int s = t - k;
     const uint32_t* sig = nullptr;
+    int wpr = 1 << g.lws;
     uint32_t m = 0;
     if (LARGE || s >= oldest()) {
       sig = slot(s);
-    } else if (nset[s & 127] != kNoSet) {
-      m = slice_list<OPEN>(ar.sets + (s % kArchiveSets) * ar.cap, nset[s & 127], g.L, x, y, k, lane);
-    } else if (s < ar.gone && s >= ar.gone - ar.nb) {
-      sig = ar.bitmaps + (s % ar.nb) * g.nws;
     } else {
-      misc[3] = 1;  // the shot needs a syndrome that is no longer kept
+      const int n = nset[s & (kSteps - 1)];
+      const uint32_t* at = ar.words + place[s & (kSteps - 1)];
+      if (n == kNotKept) {
+        misc[3] = 1;
+      } else if (n == kBitmap) {
+        sig = at;
+        wpr = (g.L + 31) >> 5;
+      } else {
+        m = slice_list<OPEN>(reinterpret_cast<const uint16_t*>(at), n, g.L, x, y, k, lane);
+      }
     }
-    if (sig) m = slice_warp<OPEN>(sig, g.lws, g.L, x, y, k, lane);
+    if (sig) m = slice_warp<OPEN>(sig, wpr, g.L, x, y, k, lane);
     return (m | edges(x, k)) & slice_limit(a.m_max, k);
   }
   // Slices from k on by the whole warp; returns the first slice's hits (0:
@@ -1084,7 +1134,7 @@ struct Decoder {
         if (t == 0) {
           cx[o] = fx;
           cy[o] = fy;
-        } else if (maps_in_slots()) {
+        } else if (!LARGE && !g.c_global) {
           cx[o] ^= fx;
           cy[o] ^= fy;
         } else {
@@ -1480,16 +1530,16 @@ struct Decoder {
                                                  ~(uintptr_t)3);
       if (g.c_global) {
         C = reinterpret_cast<uint32_t*>(room);
-        F = C + 2 * g.nws;
-        room += 16 * g.nws;
+        room += 8 * g.nws;
       }
-      const int bytes = 2 * LL - (int)(room - outC), bm = 4 * g.nws;
-      ar.cap = bytes / (4 * kArchiveSets);
-      if (ar.cap < 2 * kFew) ar.cap = 0;
-      ar.nb = (bytes - 2 * kArchiveSets * ar.cap) / bm;
-      ar.bitmaps = reinterpret_cast<uint32_t*>(room);
-      ar.sets = reinterpret_cast<uint16_t*>(room + ar.nb * bm);
-      ar.gone = ar.next = 0;
+      if (g.f_global) {
+        F = reinterpret_cast<uint32_t*>(room);
+        room += 8 * g.nws;
+      }
+      ar.words = reinterpret_cast<uint32_t*>(room);
+      ar.size = (2 * LL - (int)(room - outC)) >> 2;
+      ar.head = ar.next = 0;
+      ar.listed = 0;
     }
     if (tid < 8) misc[tid] = 0;
     ph = 0;
@@ -1557,7 +1607,7 @@ struct Decoder {
     int still = 0;
 #pragma unroll 1
     while (n) {
-      const int nl = advance(t, listed);
+      const int nl = advance(t, listed, n);
       if (listed) n = nl;
       if (n == 0) break;
       if (t >= a.max_steps || still > g.kmax) {

@@ -47,6 +47,7 @@ __global__ void __launch_bounds__(NT, NT == 32 ? 24 : (LARGE ? 1024 / NT : 768 /
     d.few = reinterpret_cast<typename Decoder<NT, LARGE, PLAIN, OPEN>::Ent*>(sm + g.o_few);
     d.misc = reinterpret_cast<int*>(sm + g.o_misc);
     d.nset = reinterpret_cast<uint16_t*>(sm + g.o_misc + 8);
+    d.place = d.nset + kSteps;
     d.shot = a.shot_list ? (int64_t)a.shot_list[k] : k;
     d.tid = threadIdx.x;
     d.lane = threadIdx.x & 31;
@@ -84,6 +85,7 @@ __global__ void __launch_bounds__(NT, NT == 32 ? 24 : 768 / NT)
   d.few = reinterpret_cast<uint16_t*>(sm + g.o_few);
   d.misc = reinterpret_cast<int*>(sm + g.o_misc);
   d.nset = reinterpret_cast<uint16_t*>(sm + g.o_misc + 8);
+  d.place = d.nset + kSteps;
   d.shot = m.a.shot_list[k];
   d.tid = threadIdx.x;
   d.lane = threadIdx.x & 31;

@@ -209,6 +209,7 @@ void lane_body(int tid) {
   d.few = reinterpret_cast<uint16_t*>(g_sm + g_geom.o_few);
   d.misc = reinterpret_cast<int*>(g_sm + g_geom.o_misc);
   d.nset = reinterpret_cast<uint16_t*>(g_sm + g_geom.o_misc + 8);
+  d.place = d.nset + kSteps;
   d.shot = 0;
   d.tid = tid;
   d.lane = tid & 31;

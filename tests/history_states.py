@@ -16,6 +16,19 @@ def patch_and_far(L, rng, far):
     return s
 
 
+def strip_and_far(L, rng, far):
+    """Anyon indicator: a strip of balanced anyons along the lattice that never thins
+    out, and anyons half the torus from it, which ask for more old syndromes than the
+    decoder keeps (from L = 129 on)."""
+    s = np.zeros((L, L), np.uint8)
+    s[:, : L // 4][::2, ::2] = 1
+    for _ in range(far):
+        s[int(rng.integers(L)), int(rng.integers(L // 2, 3 * L // 4))] ^= 1
+    if s.sum() % 2:
+        s[0, 5 * L // 8] ^= 1
+    return s
+
+
 def noise_of(s):
     """Links uint8 [2][L][L] of the torus whose anyons are s (an even number)."""
     L = s.shape[0]

@@ -8,7 +8,7 @@ import pytest
 
 import history_emulation as emu
 import oracle
-from history_states import open_noise_of, patch_and_far
+from history_states import open_noise_of, patch_and_far, strip_and_far
 
 pytestmark = pytest.mark.skipif(shutil.which("g++") is None, reason="no host compiler")
 
@@ -72,10 +72,27 @@ def test_caps_around_the_slots(L, m_max):
     np.testing.assert_array_equal(C[0], Co)
 
 
-@pytest.mark.parametrize("L,far,tie,seed", [(192, 6, 1, 2), (192, 80, 0, 1), (229, 20, 0, 2),
-                                            (256, 20, 1, 1)])
+@pytest.mark.parametrize("L,far,tie,seed", [(129, 80, 0, 3), (129, 80, 1, 1), (229, 80, 0, 2),
+                                            (229, 80, 1, 3)])
 def test_warps_stay_together_when_a_shot_is_left(L, far, tie, seed):
     """One warp finds that a syndrome is no longer kept while others search."""
-    s = patch_and_far(L, np.random.default_rng(seed), far)
+    s = strip_and_far(L, np.random.default_rng(seed), far)
     for order in range(10):
         assert compare_sigma(s, max_steps=130, tie=tie, order=1000 + 17 * order) == 1
+
+
+@pytest.mark.parametrize("L", [129, 136, 144, 152, 160, 176, 177, 208])
+def test_no_shot_of_random_noise_is_left(L):
+    for p in (0.08, 0.12):
+        assert compare_noise(oracle.sample_errors(L, 2, p, seed=L), max_steps=100) == 0
+
+
+@pytest.mark.parametrize("L", [9, 23, 33, 50, 80, 97, 128, 129, 170, 192, 256])
+def test_archive_against_oracle(L):
+    """Sets that stay large while a few anyons ask for old ones: entries of all sizes,
+    the ring's end, and entries that others have covered."""
+    rng = np.random.default_rng(L)
+    for i in range(6):
+        make = strip_and_far if i & 1 or L < 24 else patch_and_far
+        s = make(L, rng, 1 + 3 * i)
+        compare_sigma(s, max_steps=100, tie=i % 3 == 2, skew=i, order=i, m_max=255 - 60 * (i % 3))
