@@ -929,14 +929,16 @@ __global__ void __launch_bounds__(CL == 1 ? 1024 : (CL == 2 ? 512 : 256), CL == 
   };
   auto shot_of = [&](int64_t k) { return a.shot_list ? (int64_t)a.shot_list[k] : k; };
   if (a.only_pending) {
-    // the shots the history sweep left: the threads look at as many shots at a
-    // time (every CTA of a cluster reads a shot's state before it is decoded)
-    for (int64_t k0 = (int64_t)cid * blockDim.x; k0 < a.shots;
-         k0 += (int64_t)nclusters * blockDim.x) {
-      const bool mine = k0 + tid < a.shots && a.out_steps[shot_of(k0 + tid)] == kStepsPending;
+    // the shots the history sweep left, dealt to the clusters one by one as in a full
+    // decode; the threads look at as many of the cluster's shots at a time (every CTA
+    // of a cluster reads a shot's state before it is decoded)
+    const int64_t per = (int64_t)nclusters * blockDim.x;
+    for (int64_t k0 = cid; k0 < a.shots; k0 += per) {
+      const int64_t km = k0 + (int64_t)nclusters * tid;
+      const bool mine = km < a.shots && a.out_steps[shot_of(km)] == kStepsPending;
       if (!__syncthreads_or(mine)) continue;
-      for (int i = 0; i < (int)blockDim.x && k0 + i < a.shots; ++i) {
-        const int64_t shot = shot_of(k0 + i);
+      for (int64_t k = k0; k < a.shots && k < k0 + per; k += nclusters) {
+        const int64_t shot = shot_of(k);
         if (a.out_steps[shot] != kStepsPending) continue;
         Cluster<CL>::sync();  // all have read it
         decode_shot<CL, KW>(a, g, smem, shot, G);
