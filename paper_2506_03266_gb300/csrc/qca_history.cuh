@@ -1017,6 +1017,7 @@ struct Decoder {
     uint32_t *fxp = map_x(t) + p.j, *fyp = map_y(t) + p.j;
     const int L = g.L, lws = g.lws, H = strip_rows();
     const bool on = p.on && p.y0 < L;
+    const uint64_t key = move_key_of(t);
     int n = 0, y = p.y0;
     auto row = [&](int r) {
       if (OPEN && (unsigned)r >= (unsigned)L) return 0u;
@@ -1066,9 +1067,21 @@ struct Decoder {
           else mmy |= 1u << q;
         }
       }
-      if (moves_random()) {  // any anyon may be drawn to move: one by one
-        todo = c;
-        mpx = mmx = mpy = mmy = 0;
+      if (moves_random()) {
+        // a decided anyon may be drawn to move another way (an undecided one draws
+        // when it is searched; searching all of them took L = 256, p = 0.05, 16 shots
+        // 650 us instead of 358)
+#pragma unroll 1
+        for (uint32_t b = c & ~todo; b; b &= b - 1) {
+          const int q = __ffs(b) - 1;
+          const int d = draw_move(key, a.move_thr, site((p.j << 5) + q, wrap_hi(y, L)));
+          if (d == 0) continue;
+          const uint32_t bit = 1u << q;
+          mpx = d == 1 ? mpx | bit : mpx & ~bit;
+          mmx = d == 2 ? mmx | bit : mmx & ~bit;
+          mpy = d == 3 ? mpy | bit : mpy & ~bit;
+          mmy = d == 4 ? mmy | bit : mmy & ~bit;
+        }
       }
       const uint32_t fx = mpx | from_right(mmx, p);
       if (on) {

@@ -56,6 +56,15 @@ def test_noise_against_oracle(L, p, shots):
         compare_noise(N, max_steps=150, all_slots=True)
 
 
+@pytest.mark.parametrize("L", [8, 17, 33, 64, 100, 161])
+def test_random_moves_of_dense_steps(L):
+    """Draws that replace a decided move, a balanced axis and no move."""
+    N = oracle.sample_errors(L, 3 if L < 100 else 1, 0.1, seed=L)
+    for p in (0.02, 0.5, 1.0):
+        for kw in (dict(), dict(bal=1), dict(tie=1), dict(tie=1, bal=1)):
+            compare_noise(N, max_steps=20, move_thr=oracle.prob_threshold(p), seed=9, order=L, **kw)
+
+
 @pytest.mark.parametrize("L", [64, 96, 128])
 @pytest.mark.parametrize("m_max", [15, 16, 18, 19, 21, 22])
 def test_caps_around_the_slots(L, m_max):
