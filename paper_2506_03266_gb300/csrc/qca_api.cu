@@ -118,10 +118,13 @@ int launch_decode(const DecodeArgs& a, cudaStream_t stream) {
   if (a.shots == 0) return QCA_OK;
   if (int rc = check_aligned(a.out_steps, 4, "out_steps")) return rc;
   // v = 3 decodes from the syndrome history at any size from 8 on, unless the
-  // caller chose a kernel for the size
-  if (!history_takes(a.L, a.v) || path_forced(a.L)) return launch_planes(a, stream);
+  // caller chose a kernel for the size, or the correction would overwrite the
+  // input of a shot that is left pending
+  const bool leaves = history_may_leave_pending(a.L, a.shots);
+  if (!history_takes(a.L, a.v) || path_forced(a.L) || (a.in_place && leaves))
+    return launch_planes(a, stream);
   int rc = launch_history(a, stream);
-  if (rc || !history_may_leave_pending(a.L, a.shots)) return rc;
+  if (rc || !leaves) return rc;
   DecodeArgs rest = a;
   rest.only_pending = 1;
   rest.queue = nullptr;
@@ -216,6 +219,8 @@ int qca_decode_batch_async(const uint8_t* syndrome, int L, int64_t shots, int ma
   }
   DecodeArgs a;
   fill_args(a, syndrome, L, shots, max_steps, rng_seed, c);
+  const int64_t block = 2 * (int64_t)L * L * shots;
+  a.in_place = overlap(syndrome, block, out_correction, block);
   a.out_C = out_correction;
   a.out_steps = out_steps;
   a.out_flag = out_logical_fail;
@@ -246,6 +251,8 @@ int qca_decode_syndrome_batch_async(const uint8_t* sigma, int L, int64_t shots, 
   DecodeArgs a;
   fill_args(a, sigma, L, shots, max_steps, rng_seed, c);
   a.from_sigma = 1;
+  const int64_t sites = (int64_t)L * L * shots;
+  a.in_place = overlap(sigma, sites, out_correction, 2 * sites);
   a.out_C = out_correction;
   a.out_steps = out_steps;
   a.out_cut = out_cut_parity;

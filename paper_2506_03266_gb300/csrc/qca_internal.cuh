@@ -54,10 +54,19 @@ struct DecodeArgs {
   int bytewise;
   // Decode only the shots whose out_steps is kStepsPending (the others are done).
   int only_pending;
+  // The correction takes the place of the input (or of a part of it): a shot left
+  // pending could not be decoded again.
+  int in_place;
   // Optional count of them: the history sweep adds to it, and the sweeps that
   // follow have nothing to do where it is 0.
   unsigned int* pending;
 };
+
+// Whether two arrays of na and nb bytes share any.
+inline bool overlap(const void* a, int64_t na, const void* b, int64_t nb) {
+  const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+  return x < y ? y - x < (uintptr_t)na : x - y < (uintptr_t)nb;
+}
 
 // out_steps of a shot that the history sweep leaves to the sweeps with message
 // planes (it needs a syndrome older than the ones it keeps).

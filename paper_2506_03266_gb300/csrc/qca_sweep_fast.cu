@@ -595,6 +595,15 @@ __device__ __forceinline__ void decode_shot(const DecodeArgs& a, const FastGeom&
 
   const int64_t base = shot_offset_of(a, shot);
   const uint8_t* N = a.in + base;
+  // cut parities of N (x, y; rank 0), read with the syndrome: the correction may
+  // be written over N
+  int cutx = 0, cuty = 0;
+  if (rank == 0 && !a.from_sigma) {
+    for (int i = tid; i < L; i += nt) {
+      cutx ^= N[(size_t)i * L];
+      cuty ^= N[LL + i];
+    }
+  }
   // ---- init: bitmaps cleared, sigma measured (every CTA of the cluster holds
   //      the full sigma); the planes are written whole by the first step
   {
@@ -854,7 +863,9 @@ __device__ __forceinline__ void decode_shot(const DecodeArgs& a, const FastGeom&
     ++t;
   }
   // ================= outputs: correction bytes, homology, steps, flag
-  // (each CTA holds the correction of its own rows)
+  // (each CTA holds the correction of its own rows; a shot without anyons has met
+  // no barrier since its partners read N)
+  if (CL > 1 && t == 0) csync();
   uint8_t* outC = a.out_C + correction_offset_of(a, shot);
   const int gpr = L / 4;  // 4-site groups per row
   for (int ax = 0; ax < 2; ++ax) {
@@ -871,7 +882,7 @@ __device__ __forceinline__ void decode_shot(const DecodeArgs& a, const FastGeom&
   // partners' shares below
   csync();
   if (rank == 0) {
-    int wx = 0, wy = 0;
+    int wx = cutx, wy = cuty;
     for (int i = tid; i < L; i += nt) {
       // e_x((0, i)): row i, held by CTA i / rows_local; e_y((i, 0)): row 0, CTA 0
       const int owner = (CL == 1) ? 0 : i / g.rows_local;
@@ -879,10 +890,6 @@ __device__ __forceinline__ void decode_shot(const DecodeArgs& a, const FastGeom&
       const uint32_t by = Cb[cbk + (i >> 5)] >> (i & 31);
       wx ^= (int)(bx & 1);
       wy ^= (int)(by & 1);
-      if (!a.from_sigma) {
-        wx ^= N[(size_t)i * L];
-        wy ^= N[LL + i];
-      }
     }
     if (wx) atomicXor(&misc[1], 1);
     if (wy) atomicXor(&misc[2], 1);

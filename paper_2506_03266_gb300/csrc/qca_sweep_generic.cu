@@ -60,6 +60,12 @@ __global__ void __launch_bounds__(kThreads) sweep_generic_kernel(DecodeArgs a, u
     const int64_t base = shot_offset_of(a, shot);
     const uint8_t* in = a.in + base;
     int any = 0;
+    // cut parities of N, read with the syndrome: the correction may be written over N
+    int wx = 0, wy = 0;
+    for (int i = threadIdx.x; i < L && !a.from_sigma; i += blockDim.x) {
+      wx ^= in[i * L];
+      wy ^= in[LL + i];
+    }
     for (int i = threadIdx.x; i < LL; i += blockDim.x) {
       const int x = i % L, y = i / L;
       uint8_t s;
@@ -155,15 +161,10 @@ __global__ void __launch_bounds__(kThreads) sweep_generic_kernel(DecodeArgs a, u
     }
     // ---- outputs and homology (cut parities of N xor C, or of C alone)
     uint8_t* outC = a.out_C + correction_offset_of(a, shot);
-    int wx = 0, wy = 0;
     for (int i = threadIdx.x; i < 2 * LL; i += blockDim.x) outC[i] = Cc[i];
     for (int i = threadIdx.x; i < L; i += blockDim.x) {
       wx ^= Cc[i * L];       // e_x((0, i))
       wy ^= Cc[LL + i];      // e_y((i, 0))
-      if (!a.from_sigma) {
-        wx ^= in[i * L];
-        wy ^= in[LL + i];
-      }
     }
     if (threadIdx.x == 0) s_red[0] = s_red[1] = 0;
     __syncthreads();

@@ -315,6 +315,7 @@ int qca_decode_uneven_async(qca_uneven_plan_t p, const uint8_t* errors, int max_
   base.out_steps = out_steps;
   base.out_flag = out_logical_fail;
   base.offsets = p->d_offsets;
+  base.in_place = overlap(errors, p->total_bytes, out_correction, p->total_bytes);
   if ((rc = check_aligned(out_steps, 4, "out_steps"))) return rc;
   const size_t ns = p->sizes.size();
   std::vector<char> done(ns, 0);
@@ -325,7 +326,8 @@ int qca_decode_uneven_async(qca_uneven_plan_t p, const uint8_t* errors, int max_
   std::vector<Run> runs;
   for (size_t i = 0; p->mode == 0 && i < ns; ++i) {
     const int th = history_threads(p->sizes[i]);
-    if (!th || !history_takes(p->sizes[i], c.v) || path_forced(p->sizes[i])) continue;
+    if (!th || base.in_place || !history_takes(p->sizes[i], c.v) || path_forced(p->sizes[i]))
+      continue;
     done[i] = 1;
     if (!runs.empty() && runs.back().hi == i && i - runs.back().lo < kHistoryMixSizes &&
         history_threads(p->sizes[runs.back().lo]) == th) {

@@ -122,6 +122,12 @@ __global__ void __launch_bounds__(kVThreads) variant_kernel(VariantArgs a, uint8
     }
     const uint8_t* N = a.in + shot * 2 * (int64_t)LL;
     int any = 0;
+    // cut parities of N, read with the syndrome: the correction may be written over N
+    int wx = 0, wy = 0;
+    for (int i = threadIdx.x; i < L; i += blockDim.x) {
+      wx ^= N[i * L];  // e_x((0, i))
+      if (MODE != kOpen) wy ^= N[LL + i];  // e_y((i, 0))
+    }
     SitePos pi(L);
     for (int i = threadIdx.x; i < LL; i += blockDim.x, pi.next()) {
       const int x = pi.x, y = pi.y;
@@ -268,19 +274,12 @@ __global__ void __launch_bounds__(kVThreads) variant_kernel(VariantArgs a, uint8
     for (int i = threadIdx.x; i < 2 * LL; i += blockDim.x) outC[i] = Cc[i];
     if (threadIdx.x == 0) s_red = 0;
     __syncthreads();
-    int w = 0;
-    if (MODE == kOpen) {
-      for (int y = threadIdx.x; y < L; y += blockDim.x) w ^= N[y * L] ^ Cc[y * L];  // e_x(0, y)
-      if (w) atomicXor(&s_red, 1);
-    } else {
-      int wx = 0, wy = 0;
-      for (int i = threadIdx.x; i < L; i += blockDim.x) {
-        wx ^= N[i * L] ^ Cc[i * L];        // e_x((0, i))
-        wy ^= N[LL + i] ^ Cc[LL + i];      // e_y((i, 0))
-      }
-      if (wx) atomicXor(&s_red, 1);
-      if (wy) atomicXor(&s_red, 2);
+    for (int i = threadIdx.x; i < L; i += blockDim.x) {
+      wx ^= Cc[i * L];
+      if (MODE != kOpen) wy ^= Cc[LL + i];
     }
+    if (wx) atomicXor(&s_red, 1);
+    if (wy) atomicXor(&s_red, 2);
     __syncthreads();
     if (threadIdx.x == 0) {
       a.out_steps[shot] = t;
@@ -424,7 +423,8 @@ int qca_decode_open_batch_async(const uint8_t* noise, int L, int64_t shots, int 
     return QCA_ERR_UNSUPPORTED;
   }
   if (shots == 0) return QCA_OK;
-  if (history_takes(L, a.v) && L <= 256) {
+  const int64_t block = 2 * (int64_t)L * L * shots;
+  if (history_takes(L, a.v) && L <= 256 && !overlap(noise, block, out_correction, block)) {
     DecodeArgs h;
     if ((rc = fill_decode_args(h, noise, L, shots, max_steps, 0, cfg))) return rc;
     h.out_C = out_correction;
