@@ -1023,7 +1023,8 @@ def main():
     ap.add_argument("--max-steps", type=int, default=MAX_STEPS,
                     help="sweep workload: step budget per shot")
     ap.add_argument("--autotune", action="store_true",
-                    help="tune band height and sparse threshold per L before timing")
+                    help="tune the on-chip sweep's band height and sparse threshold per L before "
+                         "timing (with v = 3 it decodes only the shots left pending)")
     args = ap.parse_args()
 
     world = int(os.environ.get("WORLD_SIZE", "1"))

@@ -258,6 +258,9 @@ int qca_decode_uneven_async(qca_uneven_plan_t plan, const uint8_t* errors, int m
                             uint8_t* out_logical_fail, const qca_config* cfg, void* stream);
 
 /* ---- Tuning of the on-chip sweep (per lattice size, process-wide) --------
+ * The settings concern the on-chip sweep alone: with v = 3 and L from 8 up it decodes
+ * only the shots that the history decoder leaves to it, and everything where
+ * qca_set_cluster_ctas chose its four-CTA form (see qca_kernel_path).
  * band_height: rows of one plane a warp segment sweeps (4, 8, 16 or 32; it sets
  * the threads per CTA and so the CTAs per SM); 0 = built-in heuristic (the band
  * whose warp count is nearest 4 up to L = 64, L / 8 above, at most 16; where
@@ -278,9 +281,9 @@ int qca_set_cluster_ctas(int L, int ctas);
 /* Current effective values and the resulting threads per CTA (QCA_ERR_UNSUPPORTED
  * if L has no on-chip kernel). */
 int qca_get_tuning(int L, int* band_height, int* sparse_divisor, int* threads_per_cta);
-/* Time every valid (band_height, sparse_divisor) on `shots` shots of i.i.d.
- * noise p (seed) and keep the fastest as the setting for L.  Allocates
- * temporary device memory; synchronises. */
+/* Time the on-chip sweep with every valid (band_height, sparse_divisor) on `shots`
+ * shots of i.i.d. noise p (seed) and keep the fastest as the setting for L.
+ * Allocates temporary device memory; synchronises. */
 int qca_autotune(int L, int64_t shots, double p, uint64_t seed, int max_steps,
                  int* best_band_height, int* best_sparse_divisor, float* best_ms);
 

@@ -1461,6 +1461,12 @@ int qca_autotune(int L, int64_t shots, double p, uint64_t seed, int max_steps,
   if (e == cudaSuccess) e = cudaEventCreate(&e1);
   int rc = cuda_fail(e, "qca_autotune setup");
   if (rc == QCA_OK) rc = qca_sample_errors_async(L, 0, shots, p, seed, N, st);
+  // the sweep that the settings concern, not the history decoder
+  DecodeArgs args = {};
+  if (rc == QCA_OK) rc = fill_decode_args(args, N, L, shots, max_steps, 0, nullptr);
+  args.out_C = C;
+  args.out_steps = S;
+  args.out_flag = F;
   const int saved_H = g_tune_H[L], saved_div = g_tune_div[L];
   int bH = 0, bD = 0;
   float bms = 1e30f;
@@ -1474,11 +1480,11 @@ int qca_autotune(int L, int64_t shots, double p, uint64_t seed, int max_steps,
     for (int div : {256, 128, 64, 32}) {
       g_tune_div[L] = div;
       // one untimed run, then the median of three timed runs
-      rc = qca_decode_batch_async(N, L, shots, max_steps, 0, C, S, F, nullptr, st);
+      rc = launch_planes(args, st);
       float t[3];
       for (int r = 0; r < 3 && rc == QCA_OK; ++r) {
         cudaEventRecord(e0, st);
-        rc = qca_decode_batch_async(N, L, shots, max_steps, 0, C, S, F, nullptr, st);
+        rc = launch_planes(args, st);
         cudaEventRecord(e1, st);
         e = cudaEventSynchronize(e1);
         if (e != cudaSuccess) rc = cuda_fail(e, "qca_autotune timing");
