@@ -16,6 +16,7 @@
 // anyon searches; instruction fetch for the small sizes, whose warps are all at
 // different places of the code.  L = 256, p = 0.05, 20 000 shots: 4.8 ms, against
 // 55 ms for the sweep over message planes; floor by bytes 0.77 ms.
+#include <stdint.h>
 #include <string.h>
 
 #include <algorithm>
@@ -107,6 +108,7 @@ int allow_smem(K kern, size_t smem, std::atomic<int> (&have)[64], int dev) {
 struct HistWorkspace {
   uint32_t* ptr = nullptr;
   size_t bytes = 0;
+  size_t refused = SIZE_MAX;  // smallest size that could not be allocated since the last release
   cudaEvent_t done = nullptr;
 };
 std::mutex g_hws_mu;
@@ -151,10 +153,10 @@ int launch_large(const DecodeArgs& a, const Geom& g, size_t smem, size_t slot_wo
   int64_t slots = std::min<int64_t>((int64_t)std::max(per_sm, 1) * sms,
                                     (int64_t)((size_t(2) << 30) / (4 * slot_words)));
   slots = std::max<int64_t>(1, std::min<int64_t>(slots, a.shots));
-  const size_t need = 4 * slot_words * (size_t)slots;
+  const size_t slot = 4 * slot_words, need = slot * (size_t)slots;
   std::lock_guard<std::mutex> lk(g_hws_mu);
   HistWorkspace& w = g_hws[dev];
-  if (w.bytes < need) {
+  if (w.bytes < need && (need < w.refused || w.bytes < slot)) {
     if (w.ptr) {
       // the previous workspace may still be in use by queued work on any stream
       e = cudaDeviceSynchronize();
@@ -163,10 +165,19 @@ int launch_large(const DecodeArgs& a, const Geom& g, size_t smem, size_t slot_wo
       w.ptr = nullptr;
       w.bytes = 0;
     }
-    e = cudaMalloc(&w.ptr, need);
+    // where memory is short, fewer shots at a time (L = 1024: 12 MB each)
+    size_t n = (size_t)slots;
+    while ((e = cudaMalloc(&w.ptr, slot * n)) == cudaErrorMemoryAllocation) {
+      cudaGetLastError();
+      w.ptr = nullptr;
+      w.refused = std::min(w.refused, slot * n);
+      if (n == 1) break;
+      n = (n + 1) / 2;
+    }
     if (e != cudaSuccess) return cuda_fail(e, "history workspace allocation");
-    w.bytes = need;
+    w.bytes = slot * n;
   }
+  slots = std::min<int64_t>(slots, (int64_t)(w.bytes / slot));
   if (!w.done) {
     e = cudaEventCreateWithFlags(&w.done, cudaEventDisableTiming);
     if (e != cudaSuccess) return cuda_fail(e, "event creation");
@@ -291,7 +302,9 @@ int history_workspace_release() {
   std::lock_guard<std::mutex> lk(g_hws_mu);
   int dev = 0;
   cudaGetDevice(&dev);
-  if (dev < 0 || dev >= 64 || !g_hws[dev].ptr) return QCA_OK;
+  if (dev < 0 || dev >= 64) return QCA_OK;
+  g_hws[dev].refused = SIZE_MAX;
+  if (!g_hws[dev].ptr) return QCA_OK;
   cudaError_t e = cudaFree(g_hws[dev].ptr);
   g_hws[dev].ptr = nullptr;
   g_hws[dev].bytes = 0;
