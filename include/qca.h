@@ -423,7 +423,9 @@ int qca_net_train(qca_net_t net, int L, int64_t iterations, int batch, double p_
  * first step as for qca_net_train) without updating the weights: host_grads
  * (HOST, count = qca_net_param_count() floats) receives the gradient in the
  * parameter layout, *host_loss (may be NULL) the loss.  Same arithmetic as a
- * training step.  4 <= L <= 128; synchronous. */
+ * training step.  The net keeps its buffers (467 bytes per site and 21 MB) for the
+ * next call up to 2^21 sites, until qca_free_workspace or qca_net_destroy.
+ * 4 <= L <= 128; synchronous. */
 int qca_net_gradients(qca_net_t net, const uint8_t* noise, int L, int batch, float* host_grads,
                       int64_t count, float* host_loss);
 
@@ -536,8 +538,10 @@ int qca_kernel_path(int L, const qca_config* cfg);
  * then unreliable. */
 int qca_set_kernel_path(int L, int path);
 
-/* Release the device workspaces the library caches (generic-kernel state and
- * host-path staging buffers) on the current device. */
+/* Release the device workspaces the library caches on the current device: the
+ * decoders' (the generic sweep's and, above L = 256, the history decoder's up to 2 GiB
+ * each, the large-lattice sweep's), the host path's staging buffers, and the training
+ * buffers that nets keep between gradient calls.  Waits for the work that uses them. */
 int qca_free_workspace(void);
 
 /* Microbenchmarks of the sweep's roofline denominators on the current device

@@ -400,6 +400,7 @@ int qca_free_workspace(void) {
   int rc = generic_workspace_release();
   const int rc2 = tiled_workspace_release(), rc3 = history_workspace_release();
   if (rc == QCA_OK) rc = rc2 ? rc2 : rc3;
+  net_workspace_release();
   std::lock_guard<std::mutex> lk(g_stage_mu);
   int dev = 0;
   cudaGetDevice(&dev);

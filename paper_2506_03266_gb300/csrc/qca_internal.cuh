@@ -181,6 +181,8 @@ int history_threads(int L);  // 0 above L = 256 or below 8
 int launch_history_mixed(const DecodeArgs& a, const int* sizes, const int64_t* start, int nsizes,
                          cudaStream_t stream);
 int history_workspace_release();
+// Training buffers that nets of the current device keep between gradient calls.
+int net_workspace_release();
 // Large-lattice kernel (cluster of 8 CTAs per shot, state in global memory).
 int tiled_path_for(int L, int v, int m_max);  // 1 if it takes (L, v, m_max)
 int launch_tiled(const DecodeArgs& a, cudaStream_t stream);

@@ -2107,7 +2107,7 @@ struct TrainBufs {
   ~TrainBufs() { release(); }
 };
 
-// Most sites (about 490 bytes each) whose training buffers a net keeps from one
+// Most sites (467 bytes each) whose training buffers a net keeps from one
 // gradient call for the next: 1 GiB.
 constexpr int64_t kKeptSites = (int64_t)1 << 21;
 
@@ -2148,6 +2148,31 @@ struct qca_net_s {
   size_t ws_bytes = 0;
 };
 
+namespace {
+
+// All nets, for qca_free_workspace (never destroyed: a net may be closed while the
+// process exits).
+std::mutex& g_nets_mu = *new std::mutex;
+std::vector<qca_net_s*>& g_nets = *new std::vector<qca_net_s*>;
+
+}  // namespace
+
+namespace qca {
+
+int net_workspace_release() {
+  int dev = 0;
+  cudaGetDevice(&dev);
+  std::lock_guard<std::mutex> all(g_nets_mu);
+  for (qca_net_s* n : g_nets) {
+    if (n->device != dev) continue;
+    std::lock_guard<std::mutex> lk(n->grad_mu);  // (no gradient call is under way)
+    n->grad_bufs.release();
+  }
+  return QCA_OK;
+}
+
+}  // namespace qca
+
 extern "C" {
 
 int64_t qca_net_param_count(void) { return kParams; }
@@ -2172,6 +2197,10 @@ int qca_net_create(uint64_t seed, qca_net_t* out) {
   }
   qca_net_s* n = new qca_net_s();
   cudaGetDevice(&n->device);
+  {
+    std::lock_guard<std::mutex> all(g_nets_mu);
+    g_nets.push_back(n);
+  }
   cudaError_t e = cudaMalloc(&n->params, sizeof(float) * kParams);
   if (e == cudaSuccess) e = cudaMalloc(&n->grads, sizeof(float) * kParams);
   if (e == cudaSuccess) e = cudaMalloc(&n->m1, sizeof(float) * kParams);
@@ -2197,6 +2226,10 @@ int qca_net_create(uint64_t seed, qca_net_t* out) {
 
 int qca_net_destroy(qca_net_t n) {
   if (!n) return QCA_OK;
+  {
+    std::lock_guard<std::mutex> all(g_nets_mu);
+    g_nets.erase(std::remove(g_nets.begin(), g_nets.end(), n), g_nets.end());
+  }
   cudaFree(n->params);
   cudaFree(n->grads);
   cudaFree(n->m1);

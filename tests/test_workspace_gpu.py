@@ -40,3 +40,20 @@ def test_large_lattices_with_little_memory():
         assert qca.lib().qca_free_workspace() == 0
     for x, y in zip(out, want):
         assert torch.equal(x, y)
+
+
+def test_training_buffers_are_released():
+    """512 tori of 64 x 64 are 2^21 sites, the most whose buffers a net keeps: 3 bytes,
+    seven times 32 bf16 channels and four floats a site, and some more.  The library
+    gives them back on request, and the next call returns the same gradients (the loss
+    is a sum in no fixed order)."""
+    net = qca.Net(seed=1)
+    N = qca.sample_errors(64, 512, 0.05, seed=2)
+    _, want = net.gradients(N)
+    torch.cuda.synchronize()
+    held = torch.cuda.mem_get_info()[0]
+    assert qca.lib().qca_free_workspace() == 0
+    assert torch.cuda.mem_get_info()[0] - held >= (3 + 7 * 32 * 2 + 4 * 4) << 21
+    _, again = net.gradients(N)
+    assert (again == want).all()
+    net.close()
