@@ -214,7 +214,28 @@ int launch_history(const DecodeArgs& a, cudaStream_t stream) {
     return QCA_ERR_UNSUPPORTED;
   }
   const bool plain = plain_rules(a);
+  // Threads per shot where the batch is too small to fill the SMs with the fewest
+  // (threads_for): a shot's steps then take as long as one warp or four need for
+  // them.  us per call, 32 / 128 threads: L = 64, p = 0.05, 32 shots 87 / 76, 912
+  // shots 122 / 116, 2000 shots 321 / 347.  128 / 256 / 512 threads: L = 256, p =
+  // 0.05, 32 shots 224 / 178 / 159, 304 shots 260 / 215 / 307, 912 shots 356 / 406 /
+  // 709; p = 0.3 (anyons stay dense), 32 shots 2343 / 1687 / 1197 (sweep over message
+  // planes: 1173).  L = 128, p = 0.08, 304 shots 758 / 740 / 940, 912 shots 846 / 1139.
+  int sms = 0;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (threads == 32 && a.shots <= 6 * sms)
+    threads = 128;
+  else if (threads == 128 && a.L > 128 && a.shots <= sms)
+    threads = 512;
+  else if (threads == 128 && a.shots <= (a.L > 128 ? 3 : 2) * sms)
+    threads = 256;
   switch (threads) {
+    case 256:
+      return plain ? launch_small<256, true>(a, g, smem, dev, stream)
+                   : launch_small<256, false>(a, g, smem, dev, stream);
+    case 512:
+      return plain ? launch_small<512, true>(a, g, smem, dev, stream)
+                   : launch_small<512, false>(a, g, smem, dev, stream);
     case 32:
       return plain ? launch_small<32, true>(a, g, smem, dev, stream)
                    : launch_small<32, false>(a, g, smem, dev, stream);
@@ -226,8 +247,6 @@ int launch_history(const DecodeArgs& a, cudaStream_t stream) {
       // workspace stays small (1000 shots, p = 0.05: L = 384 1.51 -> 1.27 ms, L =
       // 512 2.14 -> 1.83 ms; at L = 1024 the same for 512 shots, and 1.23 -> 1.71 ms
       // for 100)
-      int sms = 0;
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
       if (a.L <= 512 && a.shots > sms)
         return plain ? launch_large<512, true>(a, g, smem, slot_words, dev, stream)
                      : launch_large<512, false>(a, g, smem, slot_words, dev, stream);

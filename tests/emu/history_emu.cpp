@@ -223,14 +223,16 @@ void lane_body(int tid) {
 // Decodes `shots` shots (noise, or anyon indicators) of size L <= 256 one after
 // the other.  `fill`: byte that the correction and the shared memory hold before;
 // `skew`: bytes by which the arrays start off a 16-byte boundary; `order`: seed of
-// the lanes' order.  A shot left pending has steps -1.  Returns 0, -1 (no
-// geometry), -2 (lanes went apart) or -3 (a write next to an array).
+// the lanes' order; `threads`: per shot, 0 for those of a large batch.  A shot left
+// pending has steps -1.  Returns 0, -1 (no geometry), -2 (lanes went apart) or -3 (a
+// write next to an array).
 extern "C" int emu_history(const uint8_t* in, int L, int shots, int max_steps, int m_max,
                            uint64_t move_thr, uint64_t seed, int tie, int bal, int from_sigma,
-                           int open, int all, int fill, int skew, uint64_t order, uint8_t* out_C,
-                           int32_t* out_steps, uint8_t* out_flag) {
+                           int open, int all, int fill, int skew, uint64_t order, int threads,
+                           uint8_t* out_C, int32_t* out_steps, uint8_t* out_flag) {
   size_t smem, slot_words;
   if (L > 256 || !make_hist_geom(L, m_max, g_geom, g_threads, smem, slot_words, all != 0)) return -1;
+  if (threads) g_threads = threads;
   DecodeArgs& a = g_args;
   memset(&a, 0, sizeof(a));
   a.L = L;
@@ -257,8 +259,13 @@ extern "C" int emu_history(const uint8_t* in, int L, int shots, int max_steps, i
   void (*body)(int) = nullptr;
   if (g_threads == 32)
     body = open ? lane_body<32, true, true> : (plain ? lane_body<32, true, false> : lane_body<32, false, false>);
+  else if (open ? g_threads > 128 : g_threads == 256 || g_threads == 512)
+    body = open ? nullptr
+                : (g_threads == 256 ? (plain ? lane_body<256, true, false> : lane_body<256, false, false>)
+                                    : (plain ? lane_body<512, true, false> : lane_body<512, false, false>));
   else
     body = open ? lane_body<128, true, true> : (plain ? lane_body<128, true, false> : lane_body<128, false, false>);
+  if (!body) return -1;
   for (int s = 0; s < shots; ++s) {
     std::fill(obuf.begin(), obuf.end(), (uint8_t)fill);
     std::fill(sbuf.begin(), sbuf.end(), (uint8_t)fill);

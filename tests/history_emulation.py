@@ -28,7 +28,7 @@ def lib():
 
 
 def decode(x, max_steps=400, m_max=255, move_thr=0, seed=0, tie=0, bal=0, sigma=False, open=False,
-           all_slots=False, fill=0xFF, skew=0, order=1):
+           all_slots=False, fill=0xFF, skew=0, order=1, threads=0):
     """Noise [shots][2][L][L] or (sigma) anyon indicators [shots][L][L]; returns
     correction, steps (PENDING where the shot is left), flag (sigma: exhausted)."""
     x = np.ascontiguousarray(x)
@@ -42,7 +42,7 @@ def decode(x, max_steps=400, m_max=255, move_thr=0, seed=0, tie=0, bal=0, sigma=
 
     rc = lib().emu_history(p(x), L, n, max_steps, m_max, ctypes.c_uint64(move_thr),
                            ctypes.c_uint64(seed), tie, bal, int(sigma), int(open), int(all_slots),
-                           fill, skew, ctypes.c_uint64(order), p(C), p(steps), p(flag))
+                           fill, skew, ctypes.c_uint64(order), threads, p(C), p(steps), p(flag))
     if rc == -2:
         raise AssertionError("lanes of a warp or block went apart")
     assert rc == 0, rc

@@ -105,3 +105,19 @@ def test_archive_against_oracle(L):
         make = strip_and_far if i & 1 or L < 24 else patch_and_far
         s = make(L, rng, 1 + 3 * i)
         compare_sigma(s, max_steps=100, tie=i % 3 == 2, skew=i, order=i, m_max=255 - 60 * (i % 3))
+
+
+@pytest.mark.parametrize("L,threads", [(8, 128), (17, 128), (32, 128), (33, 128), (64, 128),
+                                       (65, 256), (100, 256), (128, 256), (129, 512), (144, 256),
+                                       (177, 512), (224, 256), (256, 512)])
+def test_threads_of_small_batches(L, threads):
+    N = oracle.sample_errors(L, 2 if L < 130 else 1, 0.1, seed=L)
+    for kw in (dict(), dict(tie=1), dict(bal=1, seed=4),
+               dict(move_thr=oracle.prob_threshold(0.1), tie=1, seed=5)):
+        compare_noise(N, max_steps=40, threads=threads, skew=L % 3, order=L, **kw)
+    if L <= 32:
+        compare_noise(N, max_steps=100, threads=threads, all_slots=True)
+    if L >= 24:
+        rng = np.random.default_rng(L)
+        for i, make in enumerate((patch_and_far, strip_and_far)):
+            compare_sigma(make(L, rng, 5), max_steps=60, threads=threads, order=i, tie=i)
