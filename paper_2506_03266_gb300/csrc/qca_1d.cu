@@ -178,13 +178,17 @@ __global__ void __launch_bounds__(NT)
 }
 
 // The history form of the ring: L from 64 up, one thread per 32 sites, where the
-// ring's history fits shared memory (every size at v = 3).  Returns whether it
-// takes the call, and its result in rc.
+// ring's history fits shared memory (every size at v = 3).  Short rings with v = 1
+// stay with the byte fields: their anyons keep up with the messages, so a search goes
+// far (us, history / byte fields: L = 100, 2000 rings, p = 0.4 1080 / 461, p = 0.3 with
+// 10 % random moves 1122 / 467; 20 000 rings, p = 0.2 85 / 160; L = 160, 2000 rings, p =
+// 0.4 681 / 798, p = 0.3 with random moves 160 / 167).  Returns whether it takes the
+// call, and its result in rc.
 bool launch_ring_history(const Args1D& a, cudaStream_t stream, int& rc) {
   const int W = (a.L + 31) / 32;
   const int depth = (int)std::min<int64_t>((a.m_max - 1) / a.v, a.max_steps) + 2;
   const size_t smem = ((size_t)depth * W + 2 * W + 4) * 4;
-  if (a.L < 64 || W > 512 || smem > 220 * 1024 || a.shots >= (int64_t)1 << 31) return false;
+  if (a.L < (a.v == 1 ? 129 : 64) || W > 512 || smem > 220 * 1024 || a.shots >= (int64_t)1 << 31) return false;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   rc = cuda_fail(e, "cudaGetDevice");
