@@ -163,6 +163,7 @@ struct Archive {
   int size;  // words of the ring
   int head;  // next free word
   int next;  // syndromes that have left their slot
+  bool round;  // the ring has been filled once: new entries cover old ones
   uint32_t listed;  // bit i: the (i + 1)-th last step was archived as a list
 };
 
@@ -675,9 +676,11 @@ struct Decoder {
   // First word of a new entry of at most n words (the ring has more); marks the
   // entries that it covers.
   __device__ __forceinline__ int reserve(int n) {
-    const int at = ar.head + n > ar.size ? 0 : ar.head;
+    const bool back = ar.head + n > ar.size;
+    const int at = back ? 0 : ar.head;
+    ar.round |= back;
 #pragma unroll 1
-    for (int i = tid; i < kSteps; i += NT)
+    for (int i = ar.round ? tid : kSteps; i < kSteps; i += NT)
       if (nset[i] != kNotKept && place[i] < at + n && place[i] + entry_words(i) > at)
         nset[i] = kNotKept;
     return at;
@@ -1553,6 +1556,7 @@ struct Decoder {
       ar.size = (2 * LL - (int)(room - outC)) >> 2;
       ar.head = ar.next = 0;
       ar.listed = 0;
+      ar.round = false;
     }
     if (tid < 8) misc[tid] = 0;
     ph = 0;
