@@ -276,8 +276,8 @@ def run_reference(args, rank):
 def run_uneven(args, rank, world, local):
     """Mixed-size batch: shots with L in {24, 48, 64, 96, 128, 192}
     (30/25/20/12/8/5 %) and p ~ U[0.01, 0.07), decoded by one CUDA-graph replay
-    of one persistent mixed-size launch (a single work queue, largest L first).
-    The per-size form (one persistent launch per size, side by side on forked
+    of one launch per CTA shape, largest L first, and one for pending shots.
+    The per-size form (launches of their own for each size, side by side on forked
     streams) is timed after it on the same noise for comparison."""
     import numpy as np
     import torch
@@ -358,7 +358,7 @@ def run_uneven(args, rank, world, local):
         "decoder": {"per_size": per_size, "budget_exhausted": int((fail_h == 2).sum())},
         "per_size_launches": {"shot_decodes_per_s": shots / (per_size_ms / 1e3),
                               "ms_per_step": per_size_ms, "identical_outputs": same,
-                              "note": "one persistent launch per size on forked streams, "
+                              "note": "launches per size on forked streams, "
                                       "same noise, not graph-captured"},
         "roofline": hbm_roofline(4 * float(np.sum(L_s.astype(np.float64) ** 2)) + 5 * shots,
                                  ms_per_step / 1e3),

@@ -24,10 +24,11 @@
  *   - a correction array may be the input array itself (in place); otherwise
  *     inputs and outputs do not overlap.
  *   - a typed array (int32, int64, float ...) must start on a multiple of its
- *     element size, else QCA_ERR_ARG.  uint8 arrays may start anywhere: where
- *     an input or correction array (or a packed shot block) is not 4-byte
- *     aligned, the decoder uses its byte-access kernel instead of the faster
- *     word-access ones, with the same results.
+ *     element size, else QCA_ERR_ARG.  uint8 arrays may start anywhere:
+ *     where an input or correction array (or a packed shot block) is off the
+ *     boundary that wide accesses need (16 bytes for the history decoder, 4 for
+ *     the sweeps with message fields), it is read and written in smaller pieces,
+ *     with the same results.
  *   - "stream" arguments are cudaStream_t handles passed as void*; NULL means
  *     the legacy default stream.  *_async calls return after enqueueing; the
  *     others synchronise before returning.
@@ -108,7 +109,9 @@ int qca_sample_errors_async(int L, int64_t shot0, int64_t shots, double p, uint6
                             uint8_t* out_errors, void* stream);
 
 /* Decode a batch of noise realisations (the decoding problem of
- * Def. plogandtdec; Sec. 7 Monte Carlo).
+ * Def. plogandtdec; Sec. 7 Monte Carlo).  With v = 3 and L from 8 up the decoder
+ * keeps the past syndromes instead of the message fields; up to L = 256 a second
+ * launch decodes the shots whose syndromes outgrow what it keeps (qca_kernel_path).
  *   syndrome          device uint8 [shots][2][L][L]: the per-shot noise realisation N
  *                     (link bits); the syndrome sigma is measured from it on the device
  *                     (Def. synch_ccqs).  N is needed because the failure flag is a
@@ -251,8 +254,12 @@ int qca_sample_errors_uneven_async(const int32_t* L_dev, const int64_t* offsets_
  * shots these left pending (usually none); other sizes and speeds go to launches
  * per size on streams forked from `stream` and joined back to it, which run
  * beside them.  Mode 1: launches per size for every size.  The outputs are the
- * same in both modes, and both can be captured in a CUDA graph.  Calls of one
- * plan that overlap on the GPU race on its work counters. */
+ * same in both modes.  Only kernel launches, memsets and event operations are enqueued,
+ * so a plan whose sizes are all multiples of 4 up to 128 or of 8 up to 256 can be
+ * captured in a CUDA graph (v = 3, m_max from 3 up) once an uncaptured call has set
+ * the kernels up; the other sizes' kernels share workspaces that one call hands to
+ * the next through an event, which a capture cannot wait for.  Calls of one plan that overlap on
+ * the GPU race on its work counters. */
 int qca_decode_uneven_async(qca_uneven_plan_t plan, const uint8_t* errors, int max_steps,
                             uint64_t rng_seed, uint8_t* out_correction, int32_t* out_steps,
                             uint8_t* out_logical_fail, const qca_config* cfg, void* stream);
@@ -319,9 +326,11 @@ int qca_decode_1d_batch_async(const uint8_t* noise, int L, int64_t shots, int ma
                               void* stream);
 
 /* ---------------------------------------------------------------------------
- * Two variants of the 2D decoder (literal per-site sweep, state in a cached
- * device workspace of 14 L^2 bytes per resident shot; noise, correction,
- * steps and flag arrays as in qca_decode_batch).
+ * Two variants of the 2D decoder (noise, correction, steps and flag arrays as
+ * in qca_decode_batch).  A literal per-site sweep, with 14 L^2 bytes of state per
+ * resident shot (in a cached device workspace from L = 86 on); on the open lattice
+ * with v = 3 and 8 <= L <= 256 it decodes only the shots that the history decoder
+ * leaves (see qca_kernel_path).
  * ------------------------------------------------------------------------- */
 
 /* Open boundaries (Appendix "Open boundary conditions", Def. "message passing

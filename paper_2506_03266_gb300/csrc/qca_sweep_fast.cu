@@ -1083,8 +1083,9 @@ std::vector<LaunchShape> g_shapes;
 
 // ------------------------------------------------ mixed lattice sizes ----
 //
-// One persistent launch for a batch of shots of different sizes.  The items
-// (shots) are queued by group size, then largest L first, so that the long
+// One persistent launch for the shots of a packed batch that the history decoder
+// left pending (usually none: it then returns at once).  The items
+// (shots; those that are done are passed over) are queued by group size, then largest L first, so that the long
 // shots start early and the short ones fill the tail, and every group takes
 // the next item from one counter when it has finished its last (work stealing
 // across sizes; every shot retires after its own number of steps).

@@ -7,8 +7,9 @@
 // mixed-size on-chip sweep for the shots it left pending (usually none).  Sizes
 // above 256 and below 8, other speeds, and, in the per-size form
 // (qca_uneven_plan_set_mode), every size go to launches of their own on side
-// streams forked from and joined back to the caller's stream.  Either way the
-// decode can be captured in one CUDA graph.
+// streams forked from and joined back to the caller's stream.  Both forms can be
+// captured in a CUDA graph where no size needs a workspace of the library's (one
+// that the on-chip sweep takes; not above 256).
 #include <math.h>
 #include <stdlib.h>
 #include <string.h>
@@ -63,8 +64,8 @@ __global__ void __launch_bounds__(256) sample_uneven_kernel(const int32_t* Ls, c
 using namespace qca;
 
 struct qca_uneven_plan_s {
-  int mode = 0;                  // 0 (default): one mixed-size launch; 1: one launch per size
-  // mixed-size queue: the shots of the sizes the on-chip sweep takes (and whose
+  int mode = 0;                  // 0 (default): launches over many sizes; 1: launches per size
+  // mixed-size queue for pending shots: the shots of the sizes the on-chip sweep takes (and whose
   // blocks are 4-byte aligned), pairs first, then by group size, then largest
   // L first
   std::vector<int> msizes;       // its sizes in queue order
