@@ -3,19 +3,21 @@
 // Up to L = 256 the last 4 to 8 syndrome bitmaps and the anyon list are in the
 // shared memory of the shot's CTA; older syndromes go to the shot's own
 // correction block, which is not written before the shot ends, as bitmaps while
-// the anyons are many and as lists of sites afterwards, so that every shot of
-// random noise keeps all 85 syndromes a message can come from.  A shot that has
+// the anyons are many and as lists of sites afterwards, so that shots of random
+// noise keep all 85 syndromes a message can come from (none was left up to p = 0.2
+// with 8 shots per size and rate, L = 20 to 256).  A shot that has
 // too many large old ones (a syndrome with a part that stays dense for dozens of
 // steps and a part that is sparse) is left pending, and the sweep with message
 // planes decodes it in a second launch, which otherwise only looks for pending
 // shots.  Above L = 256 the bitmaps live in a slot of a cached workspace that
 // holds all 85.
 //
-// What bounds it: instruction issue at 20 to 24 warps per SM (2 of 4 slots used,
-// L = 256), about 160 thousand warp instructions per shot, half of them the
-// anyon searches; instruction fetch for the small sizes, whose warps are all at
-// different places of the code.  L = 256, p = 0.05, 20 000 shots: 4.8 ms, against
-// 55 ms for the sweep over message planes; floor by bytes 0.77 ms.
+// What bounds it: latency at 19 to 24 warps per SM (L = 256: 172 thousand warp
+// instructions per shot, issued in 48 % of the schedulers' cycles; warps wait for their
+// own last instruction, for link maps and correction in L2 and at barriers about
+// equally); instruction fetch for the small sizes, whose warps are all at different
+// places of the code.  L = 256, p = 0.05, 20 000 shots: 4.9 ms, against 55 ms for the
+// sweep over message planes; floor by bytes 0.77 ms.
 #include <stdint.h>
 #include <string.h>
 
