@@ -16,7 +16,7 @@
 // instructions per shot, issued in 48 % of the schedulers' cycles; warps wait for their
 // own last instruction, for link maps and correction in L2 and at barriers about
 // equally); instruction fetch for the small sizes, whose warps are all at different
-// places of the code.  L = 256, p = 0.05, 20 000 shots: 4.9 ms, against 55 ms for the
+// places of the code.  L = 256, p = 0.05, 20 000 shots: 4.85 ms, against 55 ms for the
 // sweep over message planes; floor by bytes 0.77 ms.
 #include <stdint.h>
 #include <string.h>
